@@ -45,13 +45,16 @@ constexpr size_t kOffCellBodies = kOffCellCount + align256(sizeof(int) * kNoAllo
 constexpr size_t kOffHalfCount =
     kOffCellBodies + align256(sizeof(int) * kNoAllocMaxCells * kNoAllocCellCap);
 constexpr size_t kOffLowerCount = kOffHalfCount + align256(sizeof(int) * kNoAllocMaxBodies);
-constexpr size_t kOffHalfNbr = kOffLowerCount + align256(sizeof(int) * kNoAllocMaxBodies);
-constexpr size_t kOffLowerNbr =
-    kOffHalfNbr + align256(sizeof(int) * kNoAllocMaxBodies * kNoAllocMaxNeighbors);
+constexpr size_t kOffNbr = kOffLowerCount + align256(sizeof(int) * kNoAllocMaxBodies);
+constexpr size_t kOffLowerPair =
+    kOffNbr + align256(sizeof(int) * kNoAllocMaxBodies * kNoAllocMaxNeighbors);
 constexpr size_t kOffHalfOff =
-    kOffLowerNbr + align256(sizeof(int) * kNoAllocMaxBodies * kNoAllocMaxNeighbors);
+    kOffLowerPair + align256(sizeof(int) * kNoAllocMaxBodies * kNoAllocMaxNeighbors);
 constexpr size_t kOffDone = kOffHalfOff + align256(sizeof(int) * (kNoAllocMaxBodies + 1));
+constexpr size_t kOffSeg = kOffDone + 64;  // segment sums and bases, cleared with the hand-off counters
 constexpr size_t kOffPairs = kOffDone + 256;
+static_assert(64 + sizeof(int) * 2 * ((kNoAllocMaxBodies + kSegBodies - 1) / kSegBodies) <= 256,
+              "the list build's counters fit their block");
 constexpr size_t kOffPairF = kOffPairs + align256(sizeof(int2) * kNoAllocMaxPairs);
 constexpr size_t kOffPairTi = kOffPairF + align256(sizeof(float4) * kNoAllocMaxPairs);
 constexpr size_t kOffPairTj = kOffPairTi + align256(sizeof(float4) * kNoAllocMaxPairs);
@@ -176,12 +179,13 @@ extern "C" rb_status rb_forces_beads_noalloc(int32_t shape, int64_t n_bodies, co
     s.cells.bodies = reinterpret_cast<int*>(base + kOffCellBodies);
     s.pl.half_count = reinterpret_cast<int*>(base + kOffHalfCount);
     s.pl.lower_count = reinterpret_cast<int*>(base + kOffLowerCount);
-    s.pl.half_nbr = reinterpret_cast<int*>(base + kOffHalfNbr);
-    s.pl.lower_nbr = reinterpret_cast<int*>(base + kOffLowerNbr);
+    s.pl.nbr = reinterpret_cast<int*>(base + kOffNbr);
+    s.pl.lower_pair = reinterpret_cast<int*>(base + kOffLowerPair);
     s.pl.half_off = reinterpret_cast<int*>(base + kOffHalfOff);
     s.pos_ref = reinterpret_cast<float4*>(base + kOffPosRef);
     s.rebuild_flag = reinterpret_cast<int*>(base + kOffRebuild);
     s.pl.done = reinterpret_cast<int*>(base + kOffDone);
+    s.pl.seg = reinterpret_cast<int*>(base + kOffSeg);
     s.pl.pairs = reinterpret_cast<int2*>(base + kOffPairs);
     s.pair_F = reinterpret_cast<float4*>(base + kOffPairF);
     s.pair_ti = reinterpret_cast<float4*>(base + kOffPairTi);
@@ -199,7 +203,7 @@ extern "C" rb_status rb_forces_beads_noalloc(int32_t shape, int64_t n_bodies, co
     // and the cell counts (this call's cell grid may differ from the last).
     RB_CUDA(cudaMemcpyAsync(s.tmpl_dev, tmpl, sizeof(float4) * nb, cudaMemcpyHostToDevice, s.stream));
     RB_CUDA(cudaMemsetAsync(s.status_dev, 0, sizeof(unsigned), s.stream));
-    RB_CUDA(cudaMemsetAsync(s.pl.done, 0, sizeof(int) * 2, s.stream));
+    RB_CUDA(cudaMemsetAsync(s.pl.done, 0, 256, s.stream));
     RB_CUDA(cudaMemsetAsync(s.cells.count, 0, sizeof(int) * n_cells, s.stream));
     RB_TRY(build_pairs_async(&s, true, false));
     RB_TRY(bead_pairs_async(&s));

@@ -131,14 +131,18 @@ __device__ inline float3 min_image(float3 d, float3 L, float3 invL) {
 }
 
 // ------------------------------------------------------------- system
+constexpr int kSegBodies = 256;  // bodies per segment of the pair list's offsets
+__host__ __device__ inline int pair_segments(int64_t n) { return (int)((n + kSegBodies - 1) / kSegBodies); }
+
 struct PairList {
     int max_nbr = 0;
     int64_t cap_pairs = 0;
     int* half_count = nullptr;  // N
-    int* half_nbr = nullptr;    // N x max_nbr (j > i, sorted)
+    int* nbr = nullptr;         // N x max_nbr: lower (j < i), then upper (j > i) neighbours, ascending
     int* lower_count = nullptr; // N
-    int* lower_nbr = nullptr;   // N x max_nbr (j < i, sorted), replaced by pair ids
+    int* lower_pair = nullptr;  // N x max_nbr: pair index of each lower neighbour
     int* half_off = nullptr;    // N + 1
+    int* seg = nullptr;         // pair count (0 between rebuilds), then first pair, of each segment of bodies
     int* done = nullptr;        // 2 counters of the last-CTA hand-offs of a rebuild (0 between)
     int2* pairs = nullptr;      // cap_pairs
     int* n_pairs = nullptr;     // device scalar
@@ -377,7 +381,7 @@ struct StepSeg {
     int cell_cap, n_cells;
     float Rl2;
     int max_nbr;
-    int *half_count, *half_nbr, *lower_count, *lower_nbr, *half_off, *n_pairs, *done;
+    int *half_count, *nbr, *lower_count, *lower_pair, *half_off, *seg, *n_pairs, *done;
     int64_t cap_pairs;
     int2* pairs;
     const float4 *pF, *pti, *ptj;
