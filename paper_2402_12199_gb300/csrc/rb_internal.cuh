@@ -131,7 +131,7 @@ __device__ inline float3 min_image(float3 d, float3 L, float3 invL) {
 }
 
 // ------------------------------------------------------------- system
-constexpr int kSegBodies = 256;  // bodies per segment of the pair list's offsets
+constexpr int kSegBodies = 128;  // bodies per segment of the pair list's offsets
 __host__ __device__ inline int pair_segments(int64_t n) { return (int)((n + kSegBodies - 1) / kSegBodies); }
 
 struct PairList {
@@ -295,7 +295,9 @@ inline int pair_grid(const rb_system* s, int pairs_per_cta, int max_ctas) {
   // force: rebuild regardless of the skin; checked: skin already checked (by the integrator)
 // hs (nullable): a host state block (pos | quat | vel | angmom | force | torque,
 // N float4 each) that the reduction also writes the momenta and forces to
-rb_status reduce_forces_async(rb_system* s, float half_kick_dt, float4* hs = nullptr);
+// out_f, out_t (nullable): the caller's device rows, written beside the system's own
+rb_status reduce_forces_async(rb_system* s, float half_kick_dt, float4* hs = nullptr,
+                              float* out_f = nullptr, float* out_t = nullptr);
 rb_status energy_async(rb_system* s);
 // beads.cu
 rb_status bead_pairs_async(rb_system* s);

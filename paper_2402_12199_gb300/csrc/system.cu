@@ -146,15 +146,19 @@ __device__ inline void scan_segments(const int* __restrict__ seg_sum, int* __res
 // The per-body kernels below are written as bodies that take the block's
 // index among the system's blocks (bid) and their number (nblk): the kernel
 // of one system passes its own grid, the batched kernels a system's share.
+// force: rebuild whatever the flag says (and raise it for the kernels that follow).
 __device__ __forceinline__ void cell_assign_body(const float4* __restrict__ pos, int N, float3 L,
                                                  float3 invL, float3 invw, int3 nc,
                                                  int* __restrict__ count, int* __restrict__ bodies,
-                                                 int cap, unsigned* status,
-                                                 const int* __restrict__ rebuild, int* zero_count,
-                                                 int bid) {
+                                                 int cap, unsigned* status, int* rebuild,
+                                                 int* zero_count, int force, int bid) {
     pdl_wait();
     if (zero_count && bid == 0 && threadIdx.x == 0) *zero_count = 0;
-    if (!*rebuild) return;
+    if (force) {
+        if (bid == 0 && threadIdx.x == 0) *rebuild = 1;
+    } else if (!*rebuild) {
+        return;
+    }
     int i = bid * blockDim.x + threadIdx.x;
     if (i >= N) return;
     float4 p = pos[i];
@@ -172,10 +176,10 @@ __device__ __forceinline__ void cell_assign_body(const float4* __restrict__ pos,
 
 __global__ void k_cell_assign(const float4* __restrict__ pos, int N, float3 L, float3 invL,
                               float3 invw, int3 nc, int* __restrict__ count,
-                              int* __restrict__ bodies, int cap, unsigned* status,
-                              const int* __restrict__ rebuild, int* zero_count) {
+                              int* __restrict__ bodies, int cap, unsigned* status, int* rebuild,
+                              int* zero_count, int force) {
     cell_assign_body(pos, N, L, invL, invw, nc, count, bodies, cap, status, rebuild, zero_count,
-                     blockIdx.x);
+                     force, blockIdx.x);
 }
 
 __device__ inline void sort_row(int* row, int n) {
@@ -271,8 +275,8 @@ __device__ __noinline__ void pair_row_warp(int i, const float4* __restrict__ pos
 // cells read per cell of the block instead of 27 per body) in cell order, so
 // that the stencil of a body is nine contiguous runs of them; then a thread
 // per body of the block tests its candidates (the same minimum-image test as
-// pair_row_warp) and keeps its neighbours sorted in a shared row while it
-// finds them.  The row, its two counts and the segment's share of the pair
+// pair_row_warp), collects its neighbours in a shared row and writes each to
+// its rank.  The row, its two counts and the segment's share of the pair
 // count (an integer sum: the same in any order) go to global memory.  What
 // bounds it: the gathers of the cell counts, cell entries and positions, a
 // chain of three L2 latencies per block; a warp per body had that chain (two
@@ -317,9 +321,9 @@ __device__ __forceinline__ void pair_build_body(
         auto cell_of = [&](int c) {
             const int hx = c % kHaloX, hy = c / kHaloX % kHaloY, hz = c / (kHaloX * kHaloY);
             if (hx > w.x + 1 || hy > w.y + 1 || hz > w.z + 1) return -1;
-            const int gx = (b0.x + hx - 1 + nc.x) % nc.x, gy = (b0.y + hy - 1 + nc.y) % nc.y,
-                      gz = (b0.z + hz - 1 + nc.z) % nc.z;
-            return (gz * nc.y + gy) * nc.x + gx;
+            auto wrap = [](int g, int n) { return g < 0 ? g + n : g >= n ? g - n : g; };  // g in [-1, n]
+            return (wrap(b0.z + hz - 1, nc.z) * nc.y + wrap(b0.y + hy - 1, nc.y)) * nc.x +
+                   wrap(b0.x + hx - 1, nc.x);
         };
         int cnt[2] = {0, 0};
 #pragma unroll
@@ -357,12 +361,20 @@ __device__ __forceinline__ void pair_build_body(
             const int hx = c % kHaloX, hy = c / kHaloX % kHaloY, hz = c / (kHaloX * kHaloY);
             const bool own = hx >= 1 && hx <= w.x && hy >= 1 && hy <= w.y && hz >= 1 && hz <= w.z;
             const int at = own ? atomicAdd(&s_n, n) : 0;
-            for (int s = 0; s < n; ++s) {
-                const int j = cb[s];
-                float4 q = pos[j];
-                q.w = __int_as_float(j);
-                s_body[st + s] = q;
-                if (own) s_list[at + s] = c << 16 | (st + s);
+            for (int s = 0; s < n; s += 4) {  // four entries, then four positions in flight
+                int j[4];
+                float4 q[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) j[u] = cb[min(s + u, n - 1)];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) q[u] = pos[j[u]];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (s + u >= n) break;
+                    q[u].w = __int_as_float(j[u]);
+                    s_body[st + s + u] = q[u];
+                    if (own) s_list[at + s + u] = c << 16 | (st + s + u);
+                }
             }
         }
         __syncthreads();
@@ -388,12 +400,7 @@ __device__ __forceinline__ void pair_build_body(
                             const float3 d =
                                 min_image(make_float3(q.x - p.x, q.y - p.y, q.z - p.z), L, invL);
                             if (d.x * d.x + d.y * d.y + d.z * d.z < Rc2 && j != i) {
-                                if (m < kRowCap) {
-                                    int a = m;
-                                    for (; a > 0 && s_row[a - 1][tid] > j; --a)
-                                        s_row[a][tid] = s_row[a - 1][tid];
-                                    s_row[a][tid] = j;
-                                }
+                                if (m < kRowCap) s_row[m][tid] = j;
                                 ++m;
                                 nl += j < i ? 1 : 0;
                             }
@@ -401,7 +408,12 @@ __device__ __forceinline__ void pair_build_body(
                     }
                 if (m <= min(kRowCap, max_nbr)) {
                     int* row = nbr + (size_t)i * max_nbr;
-                    for (int a = 0; a < m; ++a) row[a] = s_row[a][tid];
+                    for (int a = 0; a < m; ++a) {  // each entry to its rank
+                        const int v = s_row[a][tid];
+                        int rank = 0;
+                        for (int b = 0; b < m; ++b) rank += s_row[b][tid] < v ? 1 : 0;
+                        row[rank] = v;
+                    }
                     for (int a = 0; a < nl; ++a) lower_pair[(size_t)i * max_nbr + a] = -1;
                     lower_count[i] = nl;
                     half_count[i] = m - nl;
@@ -438,7 +450,7 @@ __global__ void __launch_bounds__(256) k_pair_build(
 // pair (i, j > i) writes it and, as the pair's index, the entry of j's row
 // that stands for i (found in j's ascending lower neighbours).  A thread per
 // pair instead of per body keeps the dependent loads of the ~3 pairs of a
-// body in flight together: 53.8 -> 45.2 us at 524288 cubes.  Then remember
+// body in flight together.  Then remember
 // the positions the list was built for and clear the cell counts and the
 // segment sum for the next rebuild.  The CTA that finishes last lowers the
 // rebuild flag (every CTA has read it by then).
@@ -452,21 +464,23 @@ __device__ __forceinline__ void pair_emit_body(
     pdl_wait();
     if (!*rebuild) return;
     __shared__ int s_off[kSegBodies + 1], s_low[kSegBodies];
-    static_assert(kSegBodies == 256, "one body per thread");
+    static_assert(kSegBodies <= 256, "at most one body per thread");
     const int tid = threadIdx.x;
     const int S = (N + kSegBodies - 1) / kSegBodies;
     for (int seg = bid; seg < S; seg += nblk) {
         const int i0 = seg * kSegBodies, i = i0 + tid;
+        const bool own = tid < kSegBodies && i < N;
         const int base = seg_base[seg];
+        const int low = own ? lower_count[i] : 0;
         int n_all;
-        const int e = block_scan256(i < N ? half_count[i] : 0, n_all);
-        s_off[tid] = e;
+        const int e = block_scan256(own ? half_count[i] : 0, n_all);
+        if (tid < kSegBodies) s_off[tid] = e;
         if (tid == 0) {
             s_off[kSegBodies] = n_all;
             seg_sum[seg] = 0;
         }
-        if (i < N) {
-            s_low[tid] = lower_count[i];
+        if (own) {
+            s_low[tid] = low;
             half_off[i] = base + e;
             pos_ref[i] = pos[i];
         }
@@ -479,15 +493,16 @@ __device__ __forceinline__ void pair_emit_body(
             const int j = nbr[(size_t)(i0 + b) * max_nbr + s_low[b] + (t - s_off[b])];
             const int* jrow = nbr + (size_t)j * max_nbr;
             const int nl = lower_count[j];
+            // the first entries are read beside the count (entries past it hold
+            // older values, so a match counts only below it)
             int found = -1;
-            for (int m = 0; m < nl; m += 4) {
+            for (int m = 0; found < 0 && (m == 0 || m < nl); m += 4) {
                 int v[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] = m + u < nl ? jrow[m + u] : -1;
+                for (int u = 0; u < 4; ++u) v[u] = m + u < max_nbr ? jrow[m + u] : -1;
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
-                    if (v[u] == i0 + b) found = m + u;
-                if (found >= 0) break;
+                    if (v[u] == i0 + b && m + u < nl) found = m + u;
             }
             const int p = base + t;
             if (p < cap_pairs) pairs[p] = make_int2(i0 + b, j);
@@ -549,7 +564,8 @@ __device__ __forceinline__ void reduce_body(
     const float4* __restrict__ pti, const float4* __restrict__ ptj, float4* __restrict__ force,
     float4* __restrict__ torque, float kick, float inv_mass, float4* __restrict__ vel,
     float4* __restrict__ angmom, const float4* __restrict__ quat, unsigned* status, float mass,
-    float3 invI, double* __restrict__ ke_part, int bid, float4* __restrict__ hs = nullptr) {
+    float3 invI, double* __restrict__ ke_part, int bid, float4* __restrict__ hs = nullptr,
+    float4* out_f = nullptr, float4* out_t = nullptr) {
     pdl_wait();
     const int t = bid * blockDim.x + threadIdx.x;
     const int i = t >> 2, sub = t & 3;
@@ -604,6 +620,8 @@ __device__ __forceinline__ void reduce_body(
             atomicOr(status, ST_NONFINITE);
         force[i] = make_float4(F.x, F.y, F.z, e);
         torque[i] = make_float4(T.x, T.y, T.z, 0.f);
+        if (out_f) out_f[i] = make_float4(F.x, F.y, F.z, e);
+        if (out_t) out_t[i] = make_float4(T.x, T.y, T.z, 0.f);
         if (HS) {
             hs[4 * (size_t)N + i] = make_float4(F.x, F.y, F.z, e);
             hs[5 * (size_t)N + i] = make_float4(T.x, T.y, T.z, 0.f);
@@ -650,10 +668,10 @@ __global__ void k_reduce(int N, int max_nbr, int64_t cap_pairs, const int* __res
                          float4* __restrict__ force, float4* __restrict__ torque, float kick,
                          float inv_mass, float4* __restrict__ vel, float4* __restrict__ angmom,
                          const float4* __restrict__ quat, unsigned* status, float mass,
-                         float3 invI, double* __restrict__ ke_part) {
+                         float3 invI, double* __restrict__ ke_part, float4* out_f, float4* out_t) {
     reduce_body(N, max_nbr, cap_pairs, half_off, half_count, lower_count, lower_pair, pF, pti, ptj,
                 force, torque, kick, inv_mass, vel, angmom, quat, status, mass, invI, ke_part,
-                blockIdx.x);
+                blockIdx.x, nullptr, out_f, out_t);
 }
 
 // k_reduce (with a kick) that also writes to the host state block hs.
@@ -968,7 +986,7 @@ __global__ void k_cell_assign_batch(const StepSeg* __restrict__ segs, const int*
     const int k = seg_of_block(start, n_seg, blockIdx.x);
     const StepSeg& S = segs[k];
     cell_assign_body(S.pos, S.N, S.L, S.invL, S.invw, S.nc, S.cell_count, S.cell_bodies, S.cell_cap,
-                     S.status, S.rebuild, S.zero_count, blockIdx.x - start[k]);
+                     S.status, S.rebuild, S.zero_count, 0, blockIdx.x - start[k]);
 }
 
 __global__ void __launch_bounds__(256) k_pair_build_batch(const StepSeg* __restrict__ segs, const int* __restrict__ start,
@@ -1017,15 +1035,14 @@ rb_status build_pairs_async(rb_system* s, bool force, bool checked, int* zero_co
     const float3 invw = inv3(s->cells.width);
     const int3 nc = make_int3(s->cells.nc[0], s->cells.nc[1], s->cells.nc[2]);
     const float Rl = s->Rc + s->skin;
-    if (force || !(s->skin > 0.f)) {
-        k_flag_set<<<1, 1, 0, s->stream>>>(s->rebuild_flag);
-    } else if (!checked) {
+    if (!(s->skin > 0.f)) force = true;  // no skin: every evaluation has a list of its own
+    if (!force && !checked) {
         k_skin_check<<<blocks_for(N, 256), 256, 0, s->stream>>>(
             N, 0.25f * s->skin * s->skin, L, invL, s->pos, s->pos_ref, s->rebuild_flag);
     }
     RB_CUDA(launch_pdl(k_cell_assign, blocks_for(N, 256), 256, 0, s->stream, s->pos, N, L, invL,
                        invw, nc, s->cells.count, s->cells.bodies, s->cells.cap, s->status_dev,
-                       s->rebuild_flag, zero_count));
+                       s->rebuild_flag, zero_count, force ? 1 : 0));
     s->fb_zeroed = zero_count != nullptr;
     int* seg_base = s->pl.seg + pair_segments(N);
     RB_CUDA(launch_pdl(k_pair_build, std::min(cell_blocks(nc), s->num_sms * 4), 256, 0, s->stream,
@@ -1043,7 +1060,7 @@ rb_status build_pairs_async(rb_system* s, bool force, bool checked, int* zero_co
     return RB_OK;
 }
 
-rb_status reduce_forces_async(rb_system* s, float kick, float4* hs) {
+rb_status reduce_forces_async(rb_system* s, float kick, float4* hs, float* out_f, float* out_t) {
     const int N = (int)s->N;
     if (hs) {  // a step of rb_step_host_state's direct form (NVE, with a kick)
         RB_CUDA(launch_pdl(k_reduce_hs, blocks_for((int64_t)N * 4, 256), 256, 0, s->stream, N,
@@ -1062,7 +1079,8 @@ rb_status reduce_forces_async(rb_system* s, float kick, float4* hs) {
                        s->force, s->torque, kick, 1.f / s->mass, s->vel, s->angmom, s->quat,
                        s->status_dev, s->mass,
                        make_float3(1.f / s->inertia[0], 1.f / s->inertia[1], 1.f / s->inertia[2]),
-                       nvt ? s->ke_part : (double*)nullptr));
+                       nvt ? s->ke_part : (double*)nullptr, reinterpret_cast<float4*>(out_f),
+                       reinterpret_cast<float4*>(out_t)));
     if (nvt)
         RB_CUDA(launch_pdl(k_thermo_end, blocks_for(N, 256), 256, 0, s->stream, N, 2.f * kick,
                            (const double*)s->ke_part, s->ke_blocks, s->nh, s->vel, s->angmom));
@@ -1778,7 +1796,7 @@ static rb_status state_replaced(rb_system* s, bool positions, bool momenta, bool
         // of the positions it was built for, however the centres got there:
         // the skin check of the next evaluation decides (a state close to the
         // previous one, as a caller feeding each step's state back, keeps it).
-        if (!(s->skin > 0.f)) k_flag_set<<<1, 1, 0, s->stream>>>(s->rebuild_flag);
+        // Without a skin every evaluation rebuilds it in any case.
         if (images) RB_CUDA(cudaMemsetAsync(s->image, 0, sizeof(int4) * s->N, s->stream));
     }
     if (s->nh && momenta)
@@ -1965,11 +1983,19 @@ static rb_status read_energy(rb_system* s, double* energy, double* virial9) {
     return RB_OK;
 }
 
+// The caller's force or torque rows if the reduction can write them itself
+// (float4 stores), else null; finish_forces copies what it could not.
+static float* direct_rows(float* p) {
+    return (reinterpret_cast<uintptr_t>(p) & 15) == 0 ? p : nullptr;
+}
+
 static rb_status finish_forces(rb_system* s, float* force, float* torque, double* energy,
                                double* virial9) {
     const size_t b = sizeof(float4) * s->N;
-    if (force) RB_CUDA(cudaMemcpyAsync(force, s->force, b, cudaMemcpyDeviceToDevice, s->stream));
-    if (torque) RB_CUDA(cudaMemcpyAsync(torque, s->torque, b, cudaMemcpyDeviceToDevice, s->stream));
+    if (force && !direct_rows(force))
+        RB_CUDA(cudaMemcpyAsync(force, s->force, b, cudaMemcpyDeviceToDevice, s->stream));
+    if (torque && !direct_rows(torque))
+        RB_CUDA(cudaMemcpyAsync(torque, s->torque, b, cudaMemcpyDeviceToDevice, s->stream));
     if (energy || virial9) RB_TRY(read_energy(s, energy, virial9));
     return RB_OK;
 }
@@ -1979,7 +2005,7 @@ rb_status rb_forces_beads(rb_system* s, float* force, float* torque, double* ene
     if (!s) return fail(RB_EINVAL, "null system");
     RB_TRY(build_pairs_async(s, false, false));
     RB_TRY(bead_pairs_async(s));
-    RB_TRY(reduce_forces_async(s, 0.f));
+    RB_TRY(reduce_forces_async(s, 0.f, nullptr, direct_rows(force), direct_rows(torque)));
     s->forces_valid = true;
     s->forces_path = RB_PATH_BEADS;
     s->forces_precision = RB_FP32;
@@ -1995,7 +2021,7 @@ rb_status rb_forces_nn(rb_system* s, const rb_mlp* m, int32_t precision, float* 
     RB_TRY(build_pairs_async(s, false, false, fallback_counter(s)));
     RB_TRY(nn_pairs_system_async(s, m, precision));
     RB_TRY(bead_fallback_async(s));
-    RB_TRY(reduce_forces_async(s, 0.f));
+    RB_TRY(reduce_forces_async(s, 0.f, nullptr, direct_rows(force), direct_rows(torque)));
     s->forces_valid = true;
     s->forces_path = RB_PATH_NN;
     s->forces_precision = precision;
@@ -2138,7 +2164,7 @@ rb_status rb_forces_fnet(rb_system* s, const rb_fnet* f, float* force, float* to
     RB_TRY(fnet_ready(f));
     RB_TRY(build_pairs_async(s, false, false));
     RB_TRY(fnet_pairs_system_async(s, f));
-    RB_TRY(reduce_forces_async(s, 0.f));
+    RB_TRY(reduce_forces_async(s, 0.f, nullptr, direct_rows(force), direct_rows(torque)));
     s->forces_valid = true;
     s->forces_path = RB_PATH_FNET;
     s->forces_precision = RB_FP32;
