@@ -282,13 +282,14 @@ __device__ __noinline__ void pair_row_warp(int i, const float4* __restrict__ pos
 // chain of three L2 latencies per block; a warp per body had that chain (two
 // loads deep) once per occupied stencil slot, and sorted its rows in global
 // memory.  The CTA that finishes last scans the segments.  Measured (with the
-// segment scan): 1332 -> 249 us at 524288 cubes, 92 -> 24.5 us at 32768
-// cylinders, 49 -> 24.4 us at 20011 cubes.
+// segment scan): 1332 -> about 145 us at 524288 cubes, 92 -> 21 us at 32768
+// cylinders, 49 -> 21 us at 20011 cubes.
 constexpr int kBlkX = 8, kBlkY = 4, kBlkZ = 4;
 constexpr int kHaloX = kBlkX + 2, kHaloY = kBlkY + 2, kHaloZ = kBlkZ + 2;
 constexpr int kHalo = kHaloX * kHaloY * kHaloZ;
-constexpr int kBlkCap = 1280;  // bodies of a block and its surroundings in shared memory
+constexpr int kBlkCap = 1024;  // bodies of a block and its surroundings in shared memory
 constexpr int kRowCap = 16;    // neighbours per shared row
+constexpr int kBuildCtas = 4;  // CTAs per SM: one wave of the grid-stride loop over blocks
 
 __host__ __device__ inline int cell_blocks(int3 nc) {
     return ((nc.x + kBlkX - 1) / kBlkX) * ((nc.y + kBlkY - 1) / kBlkY) * ((nc.z + kBlkZ - 1) / kBlkZ);
@@ -306,7 +307,7 @@ __device__ __forceinline__ void pair_build_body(
     __shared__ float4 s_body[kBlkCap];            // position, body index in w
     __shared__ int s_start[kHalo + 1];            // first body of each cell, x fastest
     __shared__ int s_list[kBlkCap];               // bodies of the block: cell << 16 | index
-    __shared__ int s_row[kRowCap][256];
+    __shared__ int s_row[kRowCap][256];           // neighbours found, a column per thread
     __shared__ int s_slow[256];
     __shared__ int s_n, s_nslow;
     static_assert(kHalo <= 512 && kBlkCap <= 65536, "two cells per thread; packed indices");
@@ -433,7 +434,7 @@ __device__ __forceinline__ void pair_build_body(
         scan_segments(seg_sum, seg_base, N, half_off, total, cap_pairs, status);
 }
 
-__global__ void __launch_bounds__(256) k_pair_build(
+__global__ void __launch_bounds__(256, kBuildCtas) k_pair_build(
     const float4* __restrict__ pos, int N, float3 L, float3 invL, float3 invw, int3 nc,
     const int* __restrict__ count, const int* __restrict__ bodies, int cap, float Rc2, int max_nbr,
     int* __restrict__ half_count, int* __restrict__ nbr, int* __restrict__ lower_count,
@@ -989,7 +990,7 @@ __global__ void k_cell_assign_batch(const StepSeg* __restrict__ segs, const int*
                      S.status, S.rebuild, S.zero_count, 0, blockIdx.x - start[k]);
 }
 
-__global__ void __launch_bounds__(256) k_pair_build_batch(const StepSeg* __restrict__ segs, const int* __restrict__ start,
+__global__ void __launch_bounds__(256, kBuildCtas) k_pair_build_batch(const StepSeg* __restrict__ segs, const int* __restrict__ start,
                                    int n_seg) {
     const int k = seg_of_block(start, n_seg, blockIdx.x);
     const StepSeg& S = segs[k];
@@ -1045,7 +1046,7 @@ rb_status build_pairs_async(rb_system* s, bool force, bool checked, int* zero_co
                        s->rebuild_flag, zero_count, force ? 1 : 0));
     s->fb_zeroed = zero_count != nullptr;
     int* seg_base = s->pl.seg + pair_segments(N);
-    RB_CUDA(launch_pdl(k_pair_build, std::min(cell_blocks(nc), s->num_sms * 4), 256, 0, s->stream,
+    RB_CUDA(launch_pdl(k_pair_build, std::min(cell_blocks(nc), s->num_sms * kBuildCtas), 256, 0, s->stream,
                        s->pos, N, L, invL, invw, nc, s->cells.count, s->cells.bodies, s->cells.cap,
                        Rl * Rl, s->pl.max_nbr, s->pl.half_count, s->pl.nbr, s->pl.lower_count,
                        s->pl.lower_pair, s->pl.seg, seg_base, s->status_dev, s->rebuild_flag,
@@ -1299,7 +1300,7 @@ rb_status batch_create(const std::vector<BatchMember>& members, const BatchTable
             const int N = (int)s->N;
             need[0].push_back(blocks_for(N, 256));
             need[1].push_back(blocks_for(N, 256));
-            need[2].push_back(std::min(cell_blocks(seg[k].nc), num_sms * 4));
+            need[2].push_back(std::min(cell_blocks(seg[k].nc), num_sms * kBuildCtas));
             need[3].push_back(std::min(blocks_for(std::max(N, s->cells.n_cells), 256), num_sms * 8));
             need[4].push_back(blocks_for((int64_t)N * 4, 256));
         }
