@@ -20,7 +20,7 @@ constexpr int kPadBeads = 3;  // far-away template entries after the last bead
 // sum is the energy itself.  rc2 is the squared cutoff in every kind.
 struct BeadPot {
     float rc2, sig2, eps4, eps24, u_shift;
-    float rc2_test;  // rc2 + a bound on the rounding of the expanded distance test
+    float rc2_test;  // rc2 + a bound on the rounding of the expanded and the box distance tests
     int kind;
     float hA, hb, hc, hp;
     // (r_c + r_circ)^2 with a rounding margin: a column of body i farther
@@ -197,6 +197,38 @@ __device__ inline void bead_terms(const float2 md0, const float2 md1, const floa
         hphc_bead<NP>(md0, md1, md2, Bx, By, Bz, pot, a);
 }
 
+// Reduce-scatter of seven sums over the warp: lanes with bit 16 set keep sums
+// 4..6 (and a zero) and hand 0..3 to their partner, then bits 8 and 4 halve
+// the kept set again and xor 2 and 1 complete it: lane 4 k returns sum k.
+__device__ inline float warp_scatter7(const float (&v)[7]) {
+    const int lane = threadIdx.x & 31;
+    float w[4];
+    {
+        const bool b = lane & 16;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float keep = b ? (j + 4 < 7 ? v[j + 4] : 0.f) : v[j];
+            const float give = b ? v[j] : (j + 4 < 7 ? v[j + 4] : 0.f);
+            w[j] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+        }
+    }
+    float u[2];
+    {
+        const bool b = lane & 8;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float keep = b ? w[j + 2] : w[j];
+            const float give = b ? w[j] : w[j + 2];
+            u[j] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+        }
+    }
+    const bool b = lane & 4;
+    float t = (b ? u[1] : u[0]) + __shfl_xor_sync(0xffffffffu, b ? u[0] : u[1], 4);
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    return t;
+}
+
 // v[0..2] = F_j, v[3..5] = T = sum_l b_l x f_l, v[6] = E, reduced over the
 // warp with xor shuffles (every lane gets the sums).
 template <int NP>
@@ -221,41 +253,7 @@ __device__ inline void warp_finish(const float (&bx)[2 * NP], const float (&by)[
         }
     }
     v[6] = pot.eps4 * (a.acc.x + a.acc.y) - pot.u_shift * (a.cnt.x + a.cnt.y);
-    // Reduce-scatter over the warp: lanes with bit 16 set keep sums 4..7 and
-    // hand 0..3 to their partner, then bits 8 and 4 halve the kept set again,
-    // so that lane l holds one of the 8 (7 and a zero) partial sums, index
-    // 4 b16 + 2 b8 + b4; xor 2 and 1 complete it.  Then every lane reads the
-    // 7 sums from lanes 0, 4, .., 24.  16 shuffles instead of 35.
-    const int lane = threadIdx.x & 31;
-    float w[4];
-    {
-        const bool b = lane & 16;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float keep = b ? (j + 4 < 7 ? v[j + 4] : 0.f) : v[j];
-            const float give = b ? v[j] : (j + 4 < 7 ? v[j + 4] : 0.f);
-            w[j] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
-        }
-    }
-    float u[2];
-    {
-        const bool b = lane & 8;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const float keep = b ? w[j + 2] : w[j];
-            const float give = b ? w[j] : w[j + 2];
-            u[j] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
-        }
-    }
-    float t;
-    {
-        const bool b = lane & 4;
-        const float keep = b ? u[1] : u[0];
-        const float give = b ? u[0] : u[1];
-        t = keep + __shfl_xor_sync(0xffffffffu, give, 4);
-    }
-    t += __shfl_xor_sync(0xffffffffu, t, 2);
-    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    const float t = warp_scatter7(v);
 #pragma unroll
     for (int k = 0; k < 7; ++k) v[k] = __shfl_sync(0xffffffffu, t, 4 * k);
 }
@@ -314,164 +312,179 @@ __device__ inline void bead_pair_warp(const float3 s, const Mat3& Rr, const floa
     warp_finish<NP>(bx, by, bz, a, pot, v);
 }
 
-// Shared-memory form of a column-structured template (see BeadCols): per
-// column c, sC[c] = (-2x, -2x, -2y, -2y) and sTh[8c + m] = thr - |d|^2 for its
-// m-th bead (z = cols.z[m]); thr as in load_template; after the last column,
-// sTh[8 n_cols + m] = -2 z_m.
-__device__ inline void load_columns(const float4* __restrict__ tmpl, const BeadCols& cols,
-                                    float thr, float4* sC, float* sTh) {
-    for (int t = threadIdx.x; t < cols.n_cols * cols.len; t += blockDim.x) {
-        const int c = t / cols.len, m = t % cols.len;
-        const float4 d = tmpl[t];
-        if (m == 0) sC[c] = make_float4(-2.f * d.x, -2.f * d.x, -2.f * d.y, -2.f * d.y);
-        sTh[8 * c + m] = thr - (d.x * d.x + d.y * d.y + d.z * d.z);
+// Shared-memory form of a column-structured template (see BeadCols): the
+// columns' (x, y) and the z values that all of them hold.
+constexpr int kMaxCols = kMaxBeads / 5;
+constexpr int kColWords = (kMaxCols + 31) / 32;  // column masks of 32 bits
+struct ColShared {
+    float2 xy[kMaxCols + 1];
+    float z[kMaxColLen];
+};
+__device__ inline void load_columns(const float4* __restrict__ tmpl, const BeadCols& cols, ColShared& sc) {
+    for (int c = threadIdx.x; c < cols.n_cols; c += blockDim.x) {
+        const float4 d = tmpl[c * cols.len];
+        sc.xy[c] = make_float2(d.x, d.y);
     }
-    for (int m = threadIdx.x; m < cols.len; m += blockDim.x) sTh[8 * cols.n_cols + m] = -2.f * cols.z[m];
+    for (int m = threadIdx.x; m < cols.len; m += blockDim.x) sc.z[m] = cols.z[m];
 }
 
-// Whole-warp bead double sum for a column-structured template of columns of
-// C beads.  The same distances and the same test as bead_pair_warp, with the
-// column's share of the expanded form computed once per slot pair:
-//   P = |b|^2 - 2 (b_x x + b_y y),   |b|^2 - 2 b.d = P - 2 b_z z_m,
-// i.e. (2 + C) packed FMAs per C distances of a slot pair instead of 3 C.
-// Columns of body i whose segment lies farther than r_c + r_circ from body
-// j's centre s hold no bead within r_c of any bead of j (every bead of j is
-// within r_circ of s): one test per column, a lane per column, decides which
-// columns are scanned at all.  A skipped column would have had no hit, so the
-// sums are those of the full scan.
-// One warp vote per bead of a scanned column; result as in warp_finish.
-
-// Lane's share of the column test: column c (< n_cols) near body j's centre.
+// Lane's share of a column test: column c (< n_cols) within sqrt(r2) of the point s.
 template <int C>
-__device__ inline bool column_near(const float3 s, const float4* sC, const BeadCols& cols, int c,
-                                   float cull2) {
+__device__ inline bool column_near(const float3 s, const ColShared& sc, const BeadCols& cols, int c, float r2) {
     if (c >= cols.n_cols) return false;
-    const float4 cxy = sC[c];                  // (-2 x_c, -2 x_c, -2 y_c, -2 y_c)
-    const float dx = fmaf(0.5f, cxy.x, s.x);   // s_x - x_c
-    const float dy = fmaf(0.5f, cxy.z, s.y);
+    const float dx = s.x - sc.xy[c].x, dy = s.y - sc.xy[c].y;
     const float dz = fmaxf(fmaxf(cols.z[0] - s.z, s.z - cols.z[C - 1]), 0.f);
-    return dx * dx + dy * dy + dz * dz <= cull2;
+    return dx * dx + dy * dy + dz * dz <= r2;
 }
 
-// The column loop of bead_pair_warp_cols: for every column of the fixed
-// template near body j, the expanded distance test of all slots against its
-// C beads (running minimum per bead), and the exact terms for the beads with a hit.
-// Columns in ascending order, as a full scan takes them.
-// ZINT: the column z values are -2, -1, 0, 1, 2 (see bead_pair_warp_cols).
-constexpr int kColWords = (kMaxBeads / 5 + 31) / 32;  // column masks of 32 bits
+// Squared distance of (x, y, z) from the box [xl, xh] x [yl, yh] x [zl, zh].
+__device__ inline float box_dist2(float x, float y, float z, float xl, float xh, float yl, float yh,
+                                  float zl, float zh) {
+    const float dx = fmaxf(fmaxf(xl - x, x - xh), 0.f);
+    const float dy = fmaxf(fmaxf(yl - y, y - yh), 0.f);
+    const float dz = fmaxf(fmaxf(zl - z, z - zh), 0.f);
+    return dx * dx + dy * dy + dz * dz;
+}
 
-template <int NP, int C, int POT, bool ZINT>
-__device__ inline bool cols_scan(const unsigned (&nearw)[kColWords], const float4* sC,
-                                 const float* sTh, const BeadCols& cols, const BeadPot& pot,
-                                 const float2 (&Bx)[NP], const float2 (&By)[NP],
-                                 const float2 (&Bz)[NP], const float2 (&BB)[NP], LJAcc<NP>& a) {
-    float2 mz[C];  // -2 z_m, duplicated
-#pragma unroll
-    for (int m = 0; m < C; ++m) mz[m] = make_float2(-2.f * cols.z[m], -2.f * cols.z[m]);
-    float2 U[NP], W[NP];  // ZINT: 2 B_z and 4 B_z (exact)
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-        U[q] = __fmul2_rn(Bz[q], make_float2(2.f, 2.f));
-        W[q] = __fmul2_rn(Bz[q], make_float2(4.f, 4.f));
-    }
-    bool any_hit = false;  // warp-uniform
-#pragma unroll
-    for (int wd = 0; wd < kColWords; ++wd) {
-        const int c0 = 32 * wd;
-        unsigned near = nearw[wd];
-        while (near) {
-            const int c = c0 + __ffs(near) - 1;
-            near &= near - 1u;
-            const float4 cxy = sC[c];
-            const float2 mx = make_float2(cxy.x, cxy.y), my = make_float2(cxy.z, cxy.w);
-            float th[C], mn[C];
-#pragma unroll
-            for (int m = 0; m < C; ++m) {
-                th[m] = sTh[8 * c + m];
-                mn[m] = 3.0e38f;
-            }
-#pragma unroll
-            for (int q = 0; q < NP; ++q) {
-                const float2 P = __ffma2_rn(By[q], my, __ffma2_rn(Bx[q], mx, BB[q]));
-                if constexpr (ZINT) {
-                    float2 t[5];
-                    t[0] = __fadd2_rn(P, W[q]);
-                    t[1] = __fadd2_rn(P, U[q]);
-                    t[2] = P;
-                    t[3] = __fadd2_rn(P, make_float2(-U[q].x, -U[q].y));
-                    t[4] = __fadd2_rn(P, make_float2(-W[q].x, -W[q].y));
-#pragma unroll
-                    for (int m = 0; m < C; ++m) mn[m] = fmin3(mn[m], t[m].x, t[m].y);
-                } else {
-#pragma unroll
-                    for (int m = 0; m < C; ++m) {
-                        const float2 t = __ffma2_rn(Bz[q], mz[m], P);
-                        mn[m] = fmin3(mn[m], t.x, t.y);
-                    }
-                }
-            }
-            // the column's beads with a slot inside the test radius (one vote
-            // each): only those get the exact terms, which for the others
-            // would add masked zeros
-            unsigned zhit = 0;
-#pragma unroll
-            for (int m = 0; m < C; ++m) zhit |= __any_sync(0xffffffffu, mn[m] < th[m]) ? 1u << m : 0u;
-            any_hit |= zhit != 0;
-            while (zhit) {
-                const int m = __ffs(zhit) - 1;
-                zhit &= zhit - 1u;
-                const float z2 = sTh[8 * cols.n_cols + m];  // -2 z_m
-                bead_terms<NP, POT>(mx, my, make_float2(z2, z2), Bx, By, Bz, pot, a);
-            }
+__device__ inline float warp_fmin(float v) {
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ inline float warp_fmax(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+// One bead pair at (dx, dy, dz), squared distance r2 (on: inside the cutoff,
+// else it adds nothing): force on j's bead, energy sum and count, as lj_bead
+// and hphc_bead form them.
+template <int POT>
+__device__ inline void bead_term(float dx, float dy, float dz, float r2, bool on, const BeadPot& pot,
+                                 float& Fx, float& Fy, float& Fz, float& acc, float& cnt) {
+    float fr;
+    if constexpr (POT == 0) {
+        const float inv2 = on ? __fdividef(1.f, r2) : 0.f;
+        const float s2 = pot.sig2 * inv2, s6 = s2 * s2 * s2, s12 = s6 * s6;
+        acc += s12 - s6;
+        fr = inv2 * (2.f * pot.eps24 * s12 - pot.eps24 * s6);
+    } else {
+        const float ir = rsqrtf(r2), r = r2 * ir, x = pot.hb - r;
+        float u;
+        if (x >= 0.f) {
+            const float xp1 = __powf(x, pot.hp - 1.f);  // 0 at x = 0 (p > 1)
+            u = fmaf(xp1, x, -2.f * pot.hA);
+            fr = pot.hp * xp1 * ir;
+        } else {
+            float sn, cs;
+            __sincosf(pot.hc * (r - pot.hb), &sn, &cs);
+            u = fmaf(-pot.hA, cs, pot.kind == 2 ? 0.f : -pot.hA);
+            fr = -pot.hA * pot.hc * sn * ir;
         }
+        acc += on ? u : 0.f;
+        fr = on ? fr : 0.f;
     }
-    return any_hit;
+    cnt += on ? 1.f : 0.f;
+    Fx = fmaf(fr, dx, Fx);
+    Fy = fmaf(fr, dy, Fy);
+    Fz = fmaf(fr, dz, Fz);
 }
 
-template <int NP, int C, int POT = 0>
-__device__ inline void bead_pair_warp_cols(const float3 s, const Mat3& Rr, const float4* sT,
-                                           const float4* sC, const float* sTh,
-                                           const BeadCols& cols, int n_beads, const BeadPot& pot,
-                                           int lane, float (&v)[7]) {
-    // which columns come near body j (one lane per column, one ballot per 32);
-    // none (a third of the listed pairs of a dilute system): every sum is
-    // zero, skip the slots as well
-    unsigned nearw[kColWords];
+// Whole-warp bead double sum of one body pair for a column-structured template
+// of columns of C beads, in the frame of body i: b[m] is body j's bead
+// l = lane + 32 m (unused slots far away).
+//   1. j's beads within the cutoff of the box around body i's beads are packed
+//      into `buf` (room for 32 NS); the others cannot interact.  Of a touching
+//      pair's 125 beads 10 to 40 are left, so a lane holds one bead from here
+//      on instead of four.
+//   2. Per 32 packed beads: the columns of i that come within the cutoff of
+//      those beads' box (a lane per column), then column by column the squared
+//      distances of every lane's bead to its C beads, (dx^2 + dy^2) + dz^2 with
+//      dz^2 kept per lane, and one vote.
+//   3. A lane with beads inside the cutoff evaluates its own ones, the warp
+//      until no lane has any left.
+// What is skipped would have added exact zeros.  Returns false (v untouched)
+// if no bead pair is inside the cutoff; else the lane's partial sums of F_j
+// (v[0..2]), T = sum_l b_l x f_l (v[3..5]) and E (v[6]).
+template <int NS, int C, int POT>
+__device__ inline bool bead_pair_cols(const float (&bx)[NS], const float (&by)[NS], const float (&bz)[NS],
+                                      const ColShared& sc, const BeadCols& cols, const BeadPot& pot,
+                                      float4* buf, int lane, float (&v)[7]) {
+    const unsigned lt = (1u << lane) - 1u;
+    int nb = 0;
+#pragma unroll
+    for (int m = 0; m < NS; ++m) {
+        const bool near = box_dist2(bx[m], by[m], bz[m], cols.x_lo, cols.x_hi, cols.y_lo, cols.y_hi,
+                                    cols.z[0], cols.z[C - 1]) <= pot.rc2_test;
+        const unsigned w = __ballot_sync(0xffffffffu, near);
+        if (near) buf[nb + __popc(w & lt)] = make_float4(bx[m], by[m], bz[m], 0.f);
+        nb += __popc(w);
+    }
+    if (nb == 0) return false;
+    __syncwarp();
     bool any = false;
 #pragma unroll
-    for (int wd = 0; wd < kColWords; ++wd) {
-        nearw[wd] = 32 * wd < cols.n_cols
-                        ? __ballot_sync(0xffffffffu, column_near<C>(s, sC, cols, 32 * wd + lane, pot.cull2))
-                        : 0u;
-        any |= nearw[wd] != 0u;
-    }
-    if (!any) {
+    for (int k = 0; k < 7; ++k) v[k] = 0.f;
+    float acc = 0.f, cnt = 0.f;
+    for (int k0 = 0; k0 < nb; k0 += 32) {
+        const bool own = k0 + lane < nb;
+        const float4 b = buf[min(k0 + lane, nb - 1)];  // surplus lanes repeat the last bead, masked below
+        const float xl = warp_fmin(b.x), xh = warp_fmax(b.x), yl = warp_fmin(b.y), yh = warp_fmax(b.y);
+        const float zl = warp_fmin(b.z), zh = warp_fmax(b.z);
+        float zz[C];
 #pragma unroll
-        for (int k = 0; k < 7; ++k) v[k] = 0.f;
-        return;
-    }
-    float bx[2 * NP], by[2 * NP], bz[2 * NP];
-    float2 Bx[NP], By[NP], Bz[NP], BB[NP];
-    slots_setup<NP>(s, Rr, sT, n_beads, lane, bx, by, bz, Bx, By, Bz, BB);
-    LJAcc<NP> a;
-    a.zero();
-    // The cube's columns have z = -2, -1, 0, 1, 2 (bead spacing 1): then
-    // -2 z_m B_z is 4 B_z, 2 B_z, 0, -2 B_z, -4 B_z, exact multiples, and
-    // P + (-2 z_m) B_z is formed with one add (or none for z = 0) from U = 2 B_z
-    // and W = 4 B_z kept per slot, rounding exactly as the fused multiply-add
-    // of the general form would.
-    bool zint = false;
-    if constexpr (C == 5)
-        zint = cols.z[0] == -2.f && cols.z[1] == -1.f && cols.z[2] == 0.f && cols.z[3] == 1.f &&
-               cols.z[4] == 2.f;
-    const bool hit = zint ? cols_scan<NP, C, POT, true>(nearw, sC, sTh, cols, pot, Bx, By, Bz, BB, a)
-                          : cols_scan<NP, C, POT, false>(nearw, sC, sTh, cols, pot, Bx, By, Bz, BB, a);
-    if (!hit) {  // no bead pair within r_c: the sums are zero
+        for (int m = 0; m < C; ++m) {
+            const float dz = b.z - cols.z[m];
+            zz[m] = own ? __fmul_rn(dz, dz) : 3.0e38f;
+        }
+        float Fx = 0.f, Fy = 0.f, Fz = 0.f;
 #pragma unroll
-        for (int k = 0; k < 7; ++k) v[k] = 0.f;
-        return;
+        for (int wd = 0; wd < kColWords; ++wd) {
+            if (32 * wd >= cols.n_cols) break;
+            const int cl = min(32 * wd + lane, cols.n_cols - 1);
+            const float2 cxy = sc.xy[cl];
+            // the column as the point nearest to the beads' box
+            const bool near = 32 * wd + lane < cols.n_cols &&
+                              box_dist2(cxy.x, cxy.y, fminf(fmaxf(cols.z[0], zl), cols.z[C - 1]), xl, xh, yl,
+                                        yh, zl, zh) <= pot.rc2_test;
+            unsigned todo = __ballot_sync(0xffffffffu, near);
+            while (todo) {
+                const int c = 32 * wd + __ffs(todo) - 1;
+                todo &= todo - 1u;
+                const float2 xy = sc.xy[c];
+                const float dx = b.x - xy.x, dy = b.y - xy.y;
+                const float p = __fmaf_rn(dy, dy, __fmul_rn(dx, dx));
+                float r2[C], mn = 3.0e38f;
+#pragma unroll
+                for (int m = 0; m < C; ++m) r2[m] = __fadd_rn(p, zz[m]);
+#pragma unroll
+                for (int m = 0; m + 1 < C; m += 2) mn = fmin3(mn, r2[m], r2[m + 1]);
+                if (C & 1) mn = fminf(mn, r2[C - 1]);
+                if (!__any_sync(0xffffffffu, mn < pot.rc2)) continue;
+                any = true;
+                unsigned mine = 0;
+#pragma unroll
+                for (int m = 0; m < C; ++m) mine |= r2[m] < pot.rc2 ? 1u << m : 0u;
+                do {
+                    const bool on = mine != 0u;
+                    const int m = on ? __ffs(mine) - 1 : 0;
+                    mine &= mine - 1u;
+                    const float dz = b.z - sc.z[m];
+                    bead_term<POT>(dx, dy, dz, __fadd_rn(p, __fmul_rn(dz, dz)), on, pot, Fx, Fy, Fz, acc, cnt);
+                } while (__any_sync(0xffffffffu, mine != 0u));
+            }
+        }
+        v[0] += Fx;
+        v[1] += Fy;
+        v[2] += Fz;
+        v[3] += b.y * Fz - b.z * Fy;
+        v[4] += b.z * Fx - b.x * Fz;
+        v[5] += b.x * Fy - b.y * Fx;
     }
-    warp_finish<NP>(bx, by, bz, a, pot, v);
+    __syncwarp();  // buf is read before the next pair's beads are packed
+    v[6] = pot.eps4 * acc - pot.u_shift * cnt;
+    return any;
 }
 
 // Smallest squared bead-bead distance between the two bodies (warp min).

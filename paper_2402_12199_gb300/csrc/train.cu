@@ -101,15 +101,16 @@ __global__ void __launch_bounds__(256)
                    float4* __restrict__ cfg, float4* __restrict__ lab, float* __restrict__ rho_c) {
     constexpr int MB = 2 * NP;
     __shared__ float4 sT[kMaxBeads + 1];
-    constexpr int kSN = C == 0 ? 2 * (kMaxBeads + kPadBeads) : kMaxBeads / 5 + 1 + 2 * (kMaxBeads / 5 + 2);
+    // any template: its distance-test form; columns: per warp the packed beads of j
+    constexpr int kSN = C == 0 ? 2 * (kMaxBeads + kPadBeads) : 8 * 32 * MB;
     __shared__ float4 sN[kSN];
+    __shared__ ColShared sc;
     __shared__ unsigned short s_cand[8][kCand];  // bead of i << 8 | bead of j
-    float* sTh = reinterpret_cast<float*>(sN + (C == 0 ? 0 : kMaxBeads / 5 + 1));  // C > 0 only
     if (C == 0) {
         load_template(tmpl, n_beads, pot.rc2_test, sT, sN);
     } else {
         for (int t = threadIdx.x; t < n_beads; t += blockDim.x) sT[t] = tmpl[t];
-        load_columns(tmpl, cols, pot.rc2_test, sN, sTh);
+        load_columns(tmpl, cols, sc);
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(256)
                 near[wd] = 0u;
                 if constexpr (C > 0) {
                     if (32 * wd < cols.n_cols)
-                        near[wd] = __ballot_sync(0xffffffffu, column_near<C>(s, sN, cols, 32 * wd + lane, t * t));
+                        near[wd] = __ballot_sync(0xffffffffu, column_near<C>(s, sc, cols, 32 * wd + lane, t * t));
                 }
             }
         };
@@ -172,8 +173,7 @@ __global__ void __launch_bounds__(256)
                     while (near[wd]) {
                         const int c = 32 * wd + __ffs(near[wd]) - 1;
                         near[wd] &= near[wd] - 1u;
-                        const float4 cxy = sN[c];
-                        const float mn = column_min<NP, C>(-0.5f * cxy.x, -0.5f * cxy.z, cols, bx, by, bz, 3.0e38f);
+                        const float mn = column_min<NP, C>(sc.xy[c].x, sc.xy[c].y, cols, bx, by, bz, 3.0e38f);
                         if (__any_sync(0xffffffffu, mn < sig2)) return true;
                     }
                 return false;
@@ -207,8 +207,7 @@ __global__ void __launch_bounds__(256)
                     while (near[wd]) {
                         const int c = 32 * wd + __ffs(near[wd]) - 1;
                         near[wd] &= near[wd] - 1u;
-                        const float4 cxy = sN[c];
-                        const float x = -0.5f * cxy.x, y = -0.5f * cxy.z;
+                        const float x = sc.xy[c].x, y = sc.xy[c].y;
                         const float mn = column_min<NP, C>(x, y, cols, bx, by, bz, 3.0e38f);
                         if (!__any_sync(0xffffffffu, mn < r2)) continue;
                         for (int k = 0; k < C; ++k) test(C * c + k, x, y, cols.z[k]);
@@ -265,10 +264,17 @@ __global__ void __launch_bounds__(256)
         const float rho = rc + ub[5] * (Rc - rc);
         const float3 s = make_float3(rho * dir.x, rho * dir.y, rho * dir.z);
         float v[7];
-        if constexpr (C > 0)
-            bead_pair_warp_cols<NP, C, POT>(s, Rr, sT, sN, sTh, cols, n_beads, pot, lane, v);
-        else
+        if constexpr (C > 0) {
+            place(rho);
+            float w[7];
+            float t = 0.f;
+            if (bead_pair_cols<MB, C, POT>(bx, by, bz, sc, cols, pot, sN + 32 * MB * warp, lane, w))
+                t = warp_scatter7(w);
+#pragma unroll
+            for (int k = 0; k < 7; ++k) v[k] = __shfl_sync(0xffffffffu, t, 4 * k);
+        } else {
             bead_pair_warp<NP, POT>(s, Rr, sT, sN, n_beads, pot, lane, v);
+        }
         if (lane == 0) {
             cfg[2 * b] = make_float4(s.x, s.y, s.z, 0.f);
             cfg[2 * b + 1] = q;
