@@ -48,6 +48,15 @@ constexpr int kMaxBeads = 256;
 // visible.  Without the launch attribute the wait returns at once.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// As pdl_wait, and lets the kernel after this one start its launch as soon as
+// every CTA of this one is running instead of when the last has ended: for the
+// step's short kernels (integrator, list kernels), whose launch latency it
+// hides.  The kernel after waits here in turn, so the order of the work is
+// unchanged.
+__device__ __forceinline__ void pdl_chain() {
+    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t stream, Args... args) {

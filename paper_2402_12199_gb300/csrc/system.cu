@@ -152,7 +152,7 @@ __device__ __forceinline__ void cell_assign_body(const float4* __restrict__ pos,
                                                  int* __restrict__ count, int* __restrict__ bodies,
                                                  int cap, unsigned* status, int* rebuild,
                                                  int* zero_count, int force, int bid) {
-    pdl_wait();
+    pdl_chain();
     if (zero_count && bid == 0 && threadIdx.x == 0) *zero_count = 0;
     if (force) {
         if (bid == 0 && threadIdx.x == 0) *rebuild = 1;
@@ -302,7 +302,7 @@ __device__ __forceinline__ void pair_build_body(
     int* __restrict__ lower_pair, int* __restrict__ seg_sum, int* __restrict__ seg_base,
     unsigned* status, const int* __restrict__ rebuild, int* __restrict__ half_off, int* total,
     int64_t cap_pairs, int* done, int bid, int nblk) {
-    pdl_wait();
+    pdl_chain();
     if (!*rebuild) return;
     __shared__ float4 s_body[kBlkCap];            // position, body index in w
     __shared__ int s_start[kHalo + 1];            // first body of each cell, x fastest
@@ -462,7 +462,7 @@ __device__ __forceinline__ void pair_emit_body(
     int64_t cap_pairs, unsigned* status, int n_cells, const float4* __restrict__ pos,
     float4* __restrict__ pos_ref, int* __restrict__ cell_count, int* rebuild, int* done, int bid,
     int nblk) {
-    pdl_wait();
+    pdl_chain();
     if (!*rebuild) return;
     __shared__ int s_off[kSegBodies + 1], s_low[kSegBodies];
     static_assert(kSegBodies <= 256, "at most one body per thread");
@@ -767,7 +767,7 @@ __device__ __forceinline__ void integrate_body(
     const float4* __restrict__ force, const float4* __restrict__ torque,
     const float4* __restrict__ pos_ref, float half_skin2, int* rebuild, NHDev* nh,
     int4* __restrict__ image, int force_rebuild, int bid, float4* __restrict__ hs = nullptr) {
-    pdl_wait();
+    pdl_chain();
     if (force_rebuild && bid == 0 && threadIdx.x == 0) *rebuild = 1;
     // NVT: first thermostat half T(dt/2) from the state between steps; one
     // thread per block computes it (FP64, identical in every block), block 0
