@@ -457,12 +457,6 @@ __device__ inline void write_pair_outputs(const PairDst& dst, int64_t gp, const 
     }
 }
 
-// symmetry.cu: canonical configurations and a tangent mapped with them
-// (cfg, ucfg: n x 2 float4 as rb_nn_weight_vjp takes them).
-__global__ void k_canon_tangent(int64_t n, PairSrc sym, const float4* __restrict__ cfg,
-                                const float4* __restrict__ ucfg, float4* __restrict__ cfg_out,
-                                float4* __restrict__ u_out);
-
 // The bead-fallback list of a system into a pair destination (and its count
 // reset), when the system has a fallback separation.
 inline rb_status set_fallback(PairDst& dst, rb_system* s) {

@@ -168,27 +168,6 @@ __global__ void k_nn_features(int64_t n, PairSrc src, float* __restrict__ x_out)
 
 }  // namespace
 
-// (cfg', u') = canonical configurations and the tangent u mapped with them:
-// u_s' = sg R(Q_k) u_s, u_q' = Q_k u_q Q_j (the map is linear in (s, q)).
-__global__ void k_canon_tangent(int64_t n, PairSrc sym, const float4* __restrict__ cfg,
-                                const float4* __restrict__ ucfg, float4* __restrict__ cfg_out,
-                                float4* __restrict__ u_out) {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= n) return;
-    const float4 c0 = cfg[2 * b];
-    float3 s = make_float3(c0.x, c0.y, c0.z);
-    float4 q = cfg[2 * b + 1];
-    float4 qk, qj;
-    float sg;
-    canon_pair(sym, s, q, qk, qj, sg);
-    cfg_out[2 * b] = make_float4(s.x, s.y, s.z, 0.f);
-    cfg_out[2 * b + 1] = q;
-    const float4 u0 = ucfg[2 * b];
-    const float3 us = mul(qmat(qk), make_float3(u0.x, u0.y, u0.z));
-    u_out[2 * b] = make_float4(sg * us.x, sg * us.y, sg * us.z, 0.f);
-    u_out[2 * b + 1] = qmul(qmul(qk, ucfg[2 * b + 1]), qj);
-}
-
 }  // namespace rb
 
 using namespace rb;

@@ -27,14 +27,15 @@
 //     a_zdot = a_hdot phi'(z),  a_z = a_h phi'(z) + a_hdot phi''(z) z_dot,
 //     dW_l += a_z h_{l-1}^T + a_zdot h_dot_{l-1}^T,  db_l += a_z,
 //     a_h_{l-1} = W_l^T a_z,  a_hdot_{l-1} = W_l^T a_zdot,
-//   with phi(z) = z sigma(z).  All arithmetic FP32; every reduction (GEMM
-//   k-loops, column sums, loss) in a fixed order.
+//   with phi(z) = z sigma(z).  The seed a_hdot_D = w_o is that of the plain
+//   reverse pass, so a_zdot_l is its signal g_l and is formed once, with the
+//   predicted forces.  All arithmetic FP32; every sum in a fixed order.
 #include <algorithm>
 #include <cmath>
 #include <new>
 
 #include "beads_common.cuh"
-#include "nn_common.cuh"
+#include "nn_f32_common.cuh"
 
 struct rb_trainer {
     rb_mlp* mlp = nullptr;
@@ -44,10 +45,12 @@ struct rb_trainer {
     float* m = nullptr;        // Adam first moment (n_params)
     float* v = nullptr;        // Adam second moment
     float* grad = nullptr;     // gradient of the last rb_train_grad / vjp
-    float* work = nullptr;     // batch workspace
-    size_t work_floats = 0;
+    float* pred = nullptr;     // predicted pair outputs of a batch (12 floats per pair)
+    float* part = nullptr;     // per CTA: its share of the gradient (n_params)
+    float* scratch = nullptr;  // per CTA: phi', phi'' terms of its tile (kTrSlots)
     double* loss_part = nullptr;
     double* loss_out = nullptr;
+    int sms = 1;
 };
 
 namespace rb {
@@ -305,28 +308,137 @@ __global__ void k_colsum(int M, int N, const float* __restrict__ A, int64_t lda,
     if (threadIdx.x == 0) out[n] = (accumulate ? out[n] : 0.f) + sh[0];
 }
 
-__device__ inline float sig_f(float z) { return 1.f / (1.f + __expf(-z)); }
+// One Adam step of a parameter; m and v in place.
+__device__ __forceinline__ float adam_update(float p, float g, float& m, float& v, float lr, float b1, float b2,
+                                             float eps, float c1, float c2) {
+    m = b1 * m + (1.f - b1) * g;
+    v = b2 * v + (1.f - b2) * g * g;
+    return p - lr * (m / c1) / (sqrtf(v / c2) + eps);
+}
 
-// Features x_hat and the tangent u_hat (x-hat space) of each pair, padded to 16.
-// desc = 1: the paper's six numbers, whose tangent follows from the rotation
+// ------------------------------------------------------------- weight gradient
+// One CTA computes a tile of S = 1024 CPT / W samples from the configurations
+// to its share of every parameter's gradient; k_train_update sums the shares
+// and applies Adam.  A thread owns CPT samples x 4 units of every layer;
+// activations and signals live in shared memory as [unit][sample] (row stride
+// S + 4: the weight-gradient loop reads rows of consecutive units, which then
+// fall on different banks), weights stream through the cp.async ring of
+// nn.cu.  phi'(z), phi''(z) terms and h_D are only needed by the thread that
+// formed them: they go to a global scratch (coalesced per thread, L2-resident).
+// Per tile: forward and plain reverse (energy, dE/dx, g_l), the residual and
+// its tangent u per sample, tangent forward, one reverse stream (a_h), and for
+// every layer dW += a_z h^T + g h_dot^T.  Samples past the batch have u = c = 0
+// and so add zeros.
+// What bounds it: FP32 FMA issue at about half rate (8 warps per SM).  A step
+// of this pass was 45 launches (split-TF32 GEMMs of 4096 x 128 x 128, each bound
+// by its load latency, and elementwise kernels between them); the GEMMs of one
+// tile are too small to pay for splitting operands and moving tiles to tensor
+// memory, and without the kernels between them there is no traffic to save.
+// Measured, batch 4096 at width 128: step 375 -> 79 us (this kernel 65 us, the
+// update 10 us), error of the gradient against FP64 2.5e-6 -> 1.8e-7; width 256:
+// 606 -> 362 us, where the shares of the 256 x 256 gradients (0.5 MB a tile)
+// weigh as much as the arithmetic.
+constexpr int kTrSlotFloats = 4 * 256;  // x CPT: one quantity of one layer, all threads
+__host__ __device__ inline int tr_slots(int D) { return 2 * D + 1; }  // phi', phi'' term per layer, h_D
+
+template <int W, int CPT, int KC>
+struct TrShape {
+    static constexpr int S = 1024 * CPT / W;  // samples per tile
+    static constexpr int LD = S + 4;
+    static constexpr int NTP = S / CPT;       // thread groups along samples
+    static constexpr int NG = 256 / NTP;      // along units
+    static_assert(NG * 4 == W && NTP <= 32, "4 units per thread; a unit's samples within a warp");
+    static size_t smem(int D) {
+        return sizeof(float) * ((size_t)(3 * D - 1) * W * LD + 2 * (size_t)KC * W + 2 * (size_t)kInPad * LD +
+                                (size_t)NG * S + 32 + (size_t)D * W + W + S);
+    }
+};
+
+// What a sample's tangent comes from: labels (force matching) or a given (u, c).
+struct TrArgs {
+    int64_t n;
+    const float4 *cfg, *lab, *ucfg;
+    const float* c;
+    float4* pred;
+    float lam_tau, lam_E, inv_f2, inv_kTw, inv_n, sw_on, sw_inv;
+};
+
+// u (tangent in (s, q) space), c and the loss of one sample from its residuals.
+__device__ inline double tr_residual(const TrArgs& A, int64_t b, float e_scale, float4& u0, float4& u1, float& c) {
+    const float scale = e_scale * A.inv_n;  // dE/dE_hat over the batch mean
+    const float4 c0 = A.cfg[2 * b], q = A.cfg[2 * b + 1];
+    const float3 s = make_float3(c0.x, c0.y, c0.z);
+    const float4 p0 = A.pred[3 * b], p1 = A.pred[3 * b + 1], p2 = A.pred[3 * b + 2];
+    const float4 l0 = A.lab[3 * b], l1 = A.lab[3 * b + 1], l2 = A.lab[3 * b + 2];
+    const float3 dF = make_float3(p0.x - l0.x, p0.y - l0.y, p0.z - l0.z);
+    const float3 di = make_float3(p1.x - l1.x, p1.y - l1.y, p1.z - l1.z);
+    const float3 dj = make_float3(p2.x - l2.x, p2.y - l2.y, p2.z - l2.z);
+    const float dE = p0.w - l0.w;
+    // per-sample weight 1 / (1 + |label|^2 / f_scale^2): relative error for
+    // large forces, absolute for small ones (1 when inv_f2 = 0)
+    const float mag2 = l0.x * l0.x + l0.y * l0.y + l0.z * l0.z +
+                       A.lam_tau * (l1.x * l1.x + l1.y * l1.y + l1.z * l1.z + l2.x * l2.x + l2.y * l2.y +
+                                    l2.z * l2.z);
+    // Boltzmann importance weight min(1, exp(-E* / kT_w)) (1 when inv_kTw = 0)
+    const float wgt = __expf(-fmaxf(l0.w, 0.f) * A.inv_kTw) / (1.f + mag2 * A.inv_f2);
+    const double l = wgt * ((double)(dF.x * dF.x + dF.y * dF.y + dF.z * dF.z) +
+                            A.lam_tau * (double)(di.x * di.x + di.y * di.y + di.z * di.z + dj.x * dj.x +
+                                                 dj.y * dj.y + dj.z * dj.z) +
+                            A.lam_E * (double)dE * dE);
+    // dl/dF = 2 w dF, dl/dtau_i = 2 w lam di, dl/dtau_j = 2 w lam dj
+    const float a2 = 2.f * wgt, b2 = 2.f * wgt * A.lam_tau;
+    const float3 rF = make_float3(a2 * dF.x, a2 * dF.y, a2 * dF.z);
+    const float3 ri = make_float3(b2 * di.x, b2 * di.y, b2 * di.z);
+    const float3 rj = make_float3(b2 * dj.x, b2 * dj.y, b2 * dj.z);
+    // F_j = -G_s, tau_i = s x G_s - tau_j, tau_j = -1/2 (-G_w v + w G_v + v x G_v)
+    const float3 rixs = cross3(ri, s);
+    const float3 us = make_float3(-rF.x + rixs.x, -rF.y + rixs.y, -rF.z + rixs.z);
+    const float3 rv = make_float3(rj.x - ri.x, rj.y - ri.y, rj.z - ri.z);
+    const float w = q.x;
+    const float3 v = make_float3(q.y, q.z, q.w);
+    const float uw = 0.5f * (rv.x * v.x + rv.y * v.y + rv.z * v.z);
+    const float3 rvxv = cross3(rv, v);
+    const float3 uv = make_float3(-0.5f * (w * rv.x + rvxv.x), -0.5f * (w * rv.y + rvxv.y),
+                                  -0.5f * (w * rv.z + rvxv.z));
+    u0 = make_float4(scale * us.x, scale * us.y, scale * us.z, 0.f);
+    u1 = make_float4(scale * uw, scale * uv.x, scale * uv.y, scale * uv.z);
+    c = scale * 2.f * wgt * A.lam_E * dE;
+    return l;
+}
+
+// Tangent of the 10 (or the paper's six) features along (u0, u1), which are
+// given for the configuration as passed.  With the smooth cutoff the output is
+// S(rho) E_hat: d/dW [u . grad(S E_hat) + c S E_hat] = d/dW [u' . grad E_hat +
+// c' E_hat] with u' = S u and c' = S c + S' (u_s . s / rho).  With a point group
+// the tangent is mapped with the configuration: u_s' = sg R(Q_k) u_s,
+// u_q' = Q_k u_q Q_j.  desc = 1: the tangent follows from the rotation
 // delta theta = 2 vec(delta q (x) q^*) of cube 2 (paper6_geometry).
-__global__ void k_tr_inputs(int64_t n, const float4* __restrict__ cfg, const float4* __restrict__ ucfg,
-                            const float* __restrict__ flat, FlatLayout fl, int desc,
-                            float* __restrict__ X, float* __restrict__ U) {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= n) return;
-    PairSrc src{};
-    src.cfg = cfg;
-    src.n_explicit = n;
-    src.desc = desc;
-    const PairGeom g = load_pair<false>(src, b, true);
-    float x[kIn];
-    raw_features(g, x);
-    const float4 u0 = ucfg[2 * b], u1 = ucfg[2 * b + 1];
-    const float3 sd = make_float3(u0.x, u0.y, u0.z);
-    const float rd = (g.s.x * sd.x + g.s.y * sd.y + g.s.z * sd.z) / g.rho;
-    float xd[kIn] = {sd.x, sd.y, sd.z, g.sgn * u1.x, g.sgn * u1.y, g.sgn * u1.z,
-                     g.sgn * u1.w, rd, -rd / (g.rho * g.rho), 2.f * g.rho * rd};
+__device__ inline void tr_tangent(const TrArgs& A, const PairGeom& g, const float4& c0, float4 u0, float4 u1,
+                                  float& c, float (&xd)[kIn]) {
+    if (A.sw_inv > 0.f) {
+        const float rho = sqrtf(c0.x * c0.x + c0.y * c0.y + c0.z * c0.z);
+        float S, dS;
+        cutoff_switch(rho, A.sw_on, A.sw_inv, S, dS);
+        c = S * c + dS * (u0.x * c0.x + u0.y * c0.y + u0.z * c0.z) / rho;
+        u0 = make_float4(S * u0.x, S * u0.y, S * u0.z, 0.f);
+        u1 = make_float4(S * u1.x, S * u1.y, S * u1.z, S * u1.w);
+    }
+    if (g.sym) {
+        const float3 r = mul(qmat(g.sym_qk), make_float3(u0.x, u0.y, u0.z));
+        u0 = make_float4(g.sym_sg * r.x, g.sym_sg * r.y, g.sym_sg * r.z, 0.f);
+        u1 = qmul(qmul(g.sym_qk, u1), g.sym_qj);
+    }
+    const float rd = (g.s.x * u0.x + g.s.y * u0.y + g.s.z * u0.z) / g.rho;
+    xd[0] = u0.x;
+    xd[1] = u0.y;
+    xd[2] = u0.z;
+    xd[3] = g.sgn * u1.x;
+    xd[4] = g.sgn * u1.y;
+    xd[5] = g.sgn * u1.z;
+    xd[6] = g.sgn * u1.w;
+    xd[7] = rd;
+    xd[8] = -rd / (g.rho * g.rho);
+    xd[9] = 2.f * g.rho * rd;
     if (g.paper6) {
         const Paper6 P = paper6_geometry(g.s, g.qc);
         const float4 t = qmul(make_float4(xd[3], xd[4], xd[5], xd[6]), qconj(g.qc));
@@ -337,129 +449,447 @@ __global__ void k_tr_inputs(int64_t n, const float4* __restrict__ cfg, const flo
         xd[5] = P.w.x * th.x + P.w.y * th.y + P.w.z * th.z + P.cot * e1t;
         xd[6] = xd[7] = xd[8] = xd[9] = 0.f;
     }
-    for (int k = 0; k < kInPad; ++k) {
-        const float isd = k < kIn ? flat[fl.inv_sd + k] : 0.f;
-        X[b * kInPad + k] = k < kIn ? (x[k] - flat[fl.mu + k]) * isd : 0.f;
-        U[b * kInPad + k] = k < kIn ? xd[k] * isd : 0.f;
+}
+
+template <int CPT>
+struct TrVec {
+    float v[CPT];
+};
+template <int CPT>
+__device__ __forceinline__ TrVec<CPT> tr_ld(const float* p) {
+    TrVec<CPT> r;
+    if constexpr (CPT == 4) {
+        const float4 a = *reinterpret_cast<const float4*>(p);
+        r.v[0] = a.x, r.v[1] = a.y, r.v[2] = a.z, r.v[3] = a.w;
+    } else {
+        const float2 a = *reinterpret_cast<const float2*>(p);
+        r.v[0] = a.x, r.v[1] = a.y;
+    }
+    return r;
+}
+template <int CPT>
+__device__ __forceinline__ void tr_st(float* p, const TrVec<CPT>& r) {
+    if constexpr (CPT == 4)
+        *reinterpret_cast<float4*>(p) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
+    else
+        *reinterpret_cast<float2*>(p) = make_float2(r.v[0], r.v[1]);
+}
+
+// acc[i][j / 2].(x, y) = sum_k A[k][p0 + i] B[k][o0 + j]: A in shared memory
+// [K][LD], B the next K / KC weight chunks.
+template <int W, int CPT, int KC>
+__device__ __forceinline__ void tr_gemm(const float* __restrict__ As, int K, ChunkFeed<W, KC>& feed, int p0,
+                                        int o0, float2 (&acc)[CPT][2]) {
+    constexpr int LD = TrShape<W, CPT, KC>::LD;
+#pragma unroll
+    for (int i = 0; i < CPT; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
+    for (int kc = 0; kc < K; kc += KC) {
+        const float* Bs = feed.acquire();
+        const int kn = min(KC, K - kc);
+#pragma unroll 16
+        for (int k = 0; k < kn; ++k) {
+            const TrVec<CPT> a = tr_ld<CPT>(As + (size_t)(kc + k) * LD + p0);
+            const float4 b = *reinterpret_cast<const float4*>(Bs + (size_t)k * W + o0);
+            const float2 b0 = make_float2(b.x, b.y), b1 = make_float2(b.z, b.w);
+#pragma unroll
+            for (int i = 0; i < CPT; ++i) {
+                const float2 aa = make_float2(a.v[i], a.v[i]);
+                acc[i][0] = __ffma2_rn(aa, b0, acc[i][0]);
+                acc[i][1] = __ffma2_rn(aa, b1, acc[i][1]);
+            }
+        }
+        feed.release();
     }
 }
-
-// Z += b (bias, row broadcast); H = phi(Z); Hd = phi'(Z) Zd.
-__global__ void k_tr_act(int64_t n, int W, const float* __restrict__ bias, float* __restrict__ Z,
-                         const float* __restrict__ Zd, float* __restrict__ H, float* __restrict__ Hd) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= n * W) return;
-    const float z = Z[t] + bias[t % W];
-    Z[t] = z;
-    const float s = sig_f(z);
-    H[t] = z * s;
-    Hd[t] = s * (1.f + z * (1.f - s)) * Zd[t];
+template <int CPT>
+__device__ __forceinline__ float tr_at(const float2 (&acc)[CPT][2], int i, int j) {
+    const float2 v = acc[i][j >> 1];
+    return (j & 1) ? v.y : v.x;
 }
 
-// Seeds of the reverse pass at the top layer: a_h = c w_o, a_hdot = w_o.
-__global__ void k_tr_seed(int64_t n, int W, const float* __restrict__ wo, const float* __restrict__ c,
-                          float* __restrict__ Ah, float* __restrict__ Ahd) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= n * W) return;
-    const float w = wo[t % W];
-    Ah[t] = c[t / W] * w;
-    Ahd[t] = w;
+// out[o * W + i] (+)= sum_c A1[o][c] B1[i][c] + A2[o][c] B2[i][c] over the
+// tile's samples: a warp per 8 units o, lanes on consecutive i; FP32x2 over
+// pairs of samples.
+template <int W, int S, int LD>
+__device__ __forceinline__ void tr_weight_grad(const float* __restrict__ A1, const float* __restrict__ B1,
+                                               const float* __restrict__ A2, const float* __restrict__ B2,
+                                               float* __restrict__ out, bool first) {
+    constexpr int JN = W / 32 < 4 ? W / 32 : 4;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int o0 = 8 * warp; o0 < W; o0 += 64)
+        for (int i0 = 0; i0 < W; i0 += 32 * JN) {
+            float2 acc[8][JN];
+#pragma unroll
+            for (int o = 0; o < 8; ++o)
+#pragma unroll
+                for (int j = 0; j < JN; ++j) acc[o][j] = make_float2(0.f, 0.f);
+#pragma unroll 1
+            for (int t = 0; t < 2; ++t) {
+                const float* A = t == 0 ? A1 : A2;
+                const float* B = t == 0 ? B1 : B2;
+#pragma unroll 2
+                for (int c = 0; c < S; c += 4) {
+                    float4 b[JN];
+#pragma unroll
+                    for (int j = 0; j < JN; ++j)
+                        b[j] = *reinterpret_cast<const float4*>(B + (size_t)(i0 + lane + 32 * j) * LD + c);
+#pragma unroll
+                    for (int o = 0; o < 8; ++o) {
+                        const float4 a = *reinterpret_cast<const float4*>(A + (size_t)(o0 + o) * LD + c);
+#pragma unroll
+                        for (int j = 0; j < JN; ++j) {
+                            acc[o][j] = __ffma2_rn(make_float2(a.x, a.y), make_float2(b[j].x, b[j].y), acc[o][j]);
+                            acc[o][j] = __ffma2_rn(make_float2(a.z, a.w), make_float2(b[j].z, b[j].w), acc[o][j]);
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int o = 0; o < 8; ++o)
+#pragma unroll
+                for (int j = 0; j < JN; ++j) {
+                    float* p = out + (size_t)(o0 + o) * W + i0 + lane + 32 * j;
+                    const float v = acc[o][j].x + acc[o][j].y;
+                    *p = first ? v : *p + v;
+                }
+        }
 }
 
-// a_zdot = a_hdot phi'(z);  a_z = a_h phi'(z) + a_hdot phi''(z) z_dot (in place).
-__global__ void k_tr_back(int64_t n, int W, const float* __restrict__ Z, const float* __restrict__ Zd,
-                          float* __restrict__ Ah, float* __restrict__ Ahd) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= n * W) return;
-    const float z = Z[t], s = sig_f(z);
-    const float d1 = s * (1.f + z * (1.f - s));
-    const float d2 = s * (1.f - s) * (2.f + z * (1.f - 2.f * s));
-    const float ah = Ah[t], ahd = Ahd[t];
-    Ah[t] = ah * d1 + ahd * d2 * Zd[t];
-    Ahd[t] = ahd * d1;
-}
+template <int W, int CPT, int KC>
+__global__ void __launch_bounds__(256, 1)
+    k_train_tile(const float* __restrict__ flat, const float* __restrict__ prep, FlatLayout fl, F32Layout pl,
+                 int D, PairSrc src, TrArgs A, float* __restrict__ part, int64_t np,
+                 float* __restrict__ scratch, double* __restrict__ loss_part) {
+    using Sh = TrShape<W, CPT, KC>;
+    constexpr int S = Sh::S, LD = Sh::LD, NTP = Sh::NTP, NG = Sh::NG;
+    constexpr int NS = 256 / S < W / 16 ? 256 / S : W / 16;  // unit slices of the dE/dx reduction
+    static_assert(NS * kIn * S <= W * LD, "dE/dx partial sums fit in one array");
+    pdl_wait();
+    extern __shared__ float4 smem4[];
+    float* Hs = reinterpret_cast<float*>(smem4);   // h_1 .. h_{D-1}
+    float* Ds = Hs + (size_t)(D - 1) * W * LD;     // h_dot_1 .. h_dot_{D-1}
+    float* Gs = Ds + (size_t)(D - 1) * W * LD;     // g_1 .. g_D, then a_z_{l-1} in the place of g_l
+    float* Zs = Gs + (size_t)D * W * LD;           // dE/dx partial sums, then a_z_D
+    float* Bs = Zs + (size_t)W * LD;               // 2 x [KC][W] weight chunks
+    float* Xs = Bs + (size_t)2 * KC * W;           // [16][LD] normalised features
+    float* Us = Xs + (size_t)kInPad * LD;          // [16][LD] their tangent
+    float* Red = Us + (size_t)kInPad * LD;         // [NG][S] energy partial sums
+    float* mu = Red + (size_t)NG * S;              // 16
+    float* isd = mu + 16;                          // 16
+    float* bias = isd + 16;                        // D x W
+    float* wo = bias + (size_t)D * W;              // W
+    float* cs = wo + W;                            // S
+    const int tid = threadIdx.x, tp = tid % NTP, to = tid / NTP;
+    const int p0 = tp * CPT, o0 = to * 4;
+    float* mine = scratch + (size_t)blockIdx.x * tr_slots(D) * kTrSlotFloats * CPT + (size_t)tid * CPT;
+    auto slot = [&](int k, int j) { return mine + ((size_t)k * 4 + j) * 256 * CPT; };  // unit j of the thread
+    float* gp = part + (size_t)blockIdx.x * np;
 
-// T = Hd + c H (for the w_o gradient).
-__global__ void k_tr_wo(int64_t n, int W, const float* __restrict__ H, const float* __restrict__ Hd,
-                        const float* __restrict__ c, float* __restrict__ T) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= n * W) return;
-    T[t] = Hd[t] + c[t / W] * H[t];
-}
-
-// Copy the padded [W x 16] first-layer gradient into the flat [W x 10] slot.
-__global__ void k_tr_w1(int W, const float* __restrict__ G16, float* __restrict__ g) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= W * kIn) return;
-    g[t] = G16[(t / kIn) * kInPad + t % kIn];
-}
-
-// Residuals of the force-matching loss: u (tangent in (s, q) space), c, and
-// the per-block FP64 loss partial sums.
-__global__ void k_tr_residual(int64_t n, const float4* __restrict__ cfg, const float4* __restrict__ pred,
-                              const float4* __restrict__ lab, float lam_tau, float lam_E,
-                              float inv_f2, float inv_kTw, const float* __restrict__ escale,
-                              float inv_n,
-                              float4* __restrict__ ucfg, float* __restrict__ c,
-                              double* __restrict__ part) {
-    __shared__ double sh[256];
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    double l = 0.0;
-    if (b < n) {
-        const float scale = *escale * inv_n;  // dE/dE_hat over the batch mean
-        const float4 c0 = cfg[2 * b], q = cfg[2 * b + 1];
-        const float3 s = make_float3(c0.x, c0.y, c0.z);
-        const float4 p0 = pred[3 * b], p1 = pred[3 * b + 1], p2 = pred[3 * b + 2];
-        const float4 l0 = lab[3 * b], l1 = lab[3 * b + 1], l2 = lab[3 * b + 2];
-        const float3 dF = make_float3(p0.x - l0.x, p0.y - l0.y, p0.z - l0.z);
-        const float3 di = make_float3(p1.x - l1.x, p1.y - l1.y, p1.z - l1.z);
-        const float3 dj = make_float3(p2.x - l2.x, p2.y - l2.y, p2.z - l2.z);
-        const float dE = p0.w - l0.w;
-        // per-sample weight 1 / (1 + |label|^2 / f_scale^2): relative error for
-        // large forces, absolute for small ones (1 when inv_f2 = 0)
-        const float mag2 = l0.x * l0.x + l0.y * l0.y + l0.z * l0.z +
-                           lam_tau * (l1.x * l1.x + l1.y * l1.y + l1.z * l1.z + l2.x * l2.x +
-                                      l2.y * l2.y + l2.z * l2.z);
-        // Boltzmann importance weight min(1, exp(-E* / kT_w)) (1 when inv_kTw = 0)
-        const float wgt = __expf(-fmaxf(l0.w, 0.f) * inv_kTw) / (1.f + mag2 * inv_f2);
-        l = wgt * ((double)(dF.x * dF.x + dF.y * dF.y + dF.z * dF.z) +
-                   lam_tau * (double)(di.x * di.x + di.y * di.y + di.z * di.z + dj.x * dj.x +
-                                      dj.y * dj.y + dj.z * dj.z) +
-                   lam_E * (double)dE * dE);
-        // dl/dF = 2 w dF, dl/dtau_i = 2 w lam di, dl/dtau_j = 2 w lam dj
-        const float a2 = 2.f * wgt, b2 = 2.f * wgt * lam_tau;
-        const float3 rF = make_float3(a2 * dF.x, a2 * dF.y, a2 * dF.z);
-        const float3 ri = make_float3(b2 * di.x, b2 * di.y, b2 * di.z);
-        const float3 rj = make_float3(b2 * dj.x, b2 * dj.y, b2 * dj.z);
-        // F_j = -G_s, tau_i = s x G_s - tau_j, tau_j = -1/2 (-G_w v + w G_v + v x G_v)
-        const float3 rixs = cross3(ri, s);
-        const float3 us = make_float3(-rF.x + rixs.x, -rF.y + rixs.y, -rF.z + rixs.z);
-        const float3 rv = make_float3(rj.x - ri.x, rj.y - ri.y, rj.z - ri.z);
-        const float w = q.x;
-        const float3 v = make_float3(q.y, q.z, q.w);
-        const float uw = 0.5f * (rv.x * v.x + rv.y * v.y + rv.z * v.z);
-        const float3 rvxv = cross3(rv, v);
-        const float3 uv = make_float3(-0.5f * (w * rv.x + rvxv.x), -0.5f * (w * rv.y + rvxv.y),
-                                      -0.5f * (w * rv.z + rvxv.z));
-        ucfg[2 * b] = make_float4(scale * us.x, scale * us.y, scale * us.z, 0.f);
-        ucfg[2 * b + 1] = make_float4(scale * uw, scale * uv.x, scale * uv.y, scale * uv.z);
-        c[b] = scale * 2.f * wgt * lam_E * dE;
+    for (int t = tid; t < 16; t += 256) {
+        mu[t] = t < kIn ? flat[fl.mu + t] : 0.f;
+        isd[t] = t < kIn ? flat[fl.inv_sd + t] : 0.f;
     }
-    sh[threadIdx.x] = l;
+    for (int t = tid; t < D * W; t += 256) bias[t] = flat[fl.b_(1 + t / W, W) + t % W];
+    for (int t = tid; t < W; t += 256) wo[t] = flat[fl.wo + t];
+    const float b_o = flat[fl.bo], e_scale = flat[fl.escale], e_shift = flat[fl.eshift];
+    const int64_t n_tiles = (A.n + S - 1) / S;
+    ChunkFeed<W, KC> feed;
+    feed.prep = prep;
+    feed.pl = pl;
+    feed.D = D;
+    feed.n_chunks = 1 + 2 * (D - 1) * ChunkFeed<W, KC>::NK;
+    feed.c = 0;
+    feed.total = ((n_tiles - 1 - blockIdx.x) / gridDim.x + 1) * 2 * feed.n_chunks;  // two passes per tile
+    feed.buf = Bs;
+    feed.issue(0);
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+
+    double loss = 0.0;
+    float bo_sum = 0.f;  // this sample thread's c
+    bool first = true;
+    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, first = false) {
+        const int64_t b = tile * S + tid;
+        const bool sample = tid < S, valid = sample && b < A.n;
+        PairGeom geo;
+        if (sample) {
+            geo = load_pair<false>(src, b, valid);
+            float x[kIn];
+            raw_features(geo, x);
+#pragma unroll
+            for (int k = 0; k < kInPad; ++k) Xs[k * LD + tid] = k < kIn ? (x[k] - mu[k]) * isd[k] : 0.f;
+        }
+        float2 acc[CPT][2];
+        // ---- forward: h_l, phi'(z_l), phi''(z_l); at the top g_D = w_o phi', w_o phi''
+        for (int l = 1; l <= D; ++l) {
+            tr_gemm<W, CPT, KC>(l == 1 ? Xs : Hs + (size_t)(l - 2) * W * LD, l == 1 ? kInPad : W, feed, p0, o0, acc);
+            TrVec<CPT> e;
+#pragma unroll
+            for (int i = 0; i < CPT; ++i) e.v[i] = 0.f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float bj = bias[(l - 1) * W + o0 + j], w = wo[o0 + j];
+                TrVec<CPT> h, d1, d2;
+#pragma unroll
+                for (int i = 0; i < CPT; ++i) {
+                    const float z = tr_at<CPT>(acc, i, j) + bj;
+                    const float sg = 1.f / (1.f + __expf(-z));
+                    h.v[i] = z * sg;
+                    d1.v[i] = sg * (1.f + z * (1.f - sg));
+                    d2.v[i] = sg * (1.f - sg) * (2.f + z * (1.f - 2.f * sg));
+                    e.v[i] = fmaf(w, h.v[i], e.v[i]);
+                }
+                tr_st<CPT>(slot(l - 1, j), d1);
+                if (l < D) {
+                    tr_st<CPT>(slot(D + l - 1, j), d2);
+                    tr_st<CPT>(Hs + (size_t)(l - 1) * W * LD + (size_t)(o0 + j) * LD + p0, h);
+                } else {
+                    tr_st<CPT>(slot(2 * D, j), h);
+#pragma unroll
+                    for (int i = 0; i < CPT; ++i) {
+                        d1.v[i] *= w;
+                        d2.v[i] *= w;
+                    }
+                    tr_st<CPT>(slot(2 * D - 1, j), d2);
+                    tr_st<CPT>(Gs + (size_t)(D - 1) * W * LD + (size_t)(o0 + j) * LD + p0, d1);
+                }
+            }
+            if (l == D) tr_st<CPT>(Red + (size_t)to * S + p0, e);
+        }
+        // ---- plain reverse: g_{l-1} = (W_l^T g_l) phi', and (W_l^T g_l) phi''
+        for (int l = D; l >= 2; --l) {
+            tr_gemm<W, CPT, KC>(Gs + (size_t)(l - 1) * W * LD, W, feed, p0, o0, acc);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                TrVec<CPT> d1 = tr_ld<CPT>(slot(l - 2, j)), d2 = tr_ld<CPT>(slot(D + l - 2, j));
+#pragma unroll
+                for (int i = 0; i < CPT; ++i) {
+                    const float a = tr_at<CPT>(acc, i, j);
+                    d1.v[i] *= a;
+                    d2.v[i] *= a;
+                }
+                tr_st<CPT>(slot(D + l - 2, j), d2);
+                tr_st<CPT>(Gs + (size_t)(l - 2) * W * LD + (size_t)(o0 + j) * LD + p0, d1);
+            }
+        }
         __syncthreads();
+        // ---- dE/dx_hat = W_1^T g_1 in unit slices; outputs, residual, tangent
+        if (A.lab) {
+            const int pp = tid % S, ks = tid / S;
+            constexpr int SL = W / NS;
+            const float4* W1p = reinterpret_cast<const float4*>(prep + pl.w1p);
+            float g[kIn];
+#pragma unroll
+            for (int k = 0; k < kIn; ++k) g[k] = 0.f;
+#pragma unroll 4
+            for (int o = ks * SL; o < (ks < NS ? ks + 1 : ks) * SL; ++o) {
+                const float gv = Gs[(size_t)o * LD + pp];
+                const float4 w0 = W1p[4 * o], w1 = W1p[4 * o + 1], w2 = W1p[4 * o + 2];
+                g[0] = fmaf(gv, w0.x, g[0]);
+                g[1] = fmaf(gv, w0.y, g[1]);
+                g[2] = fmaf(gv, w0.z, g[2]);
+                g[3] = fmaf(gv, w0.w, g[3]);
+                g[4] = fmaf(gv, w1.x, g[4]);
+                g[5] = fmaf(gv, w1.y, g[5]);
+                g[6] = fmaf(gv, w1.z, g[6]);
+                g[7] = fmaf(gv, w1.w, g[7]);
+                g[8] = fmaf(gv, w2.x, g[8]);
+                g[9] = fmaf(gv, w2.y, g[9]);
+            }
+#pragma unroll
+            for (int k = 0; k < kIn; ++k)
+                if (ks < NS) Zs[(size_t)(ks * kIn + k) * S + pp] = g[k];
+            __syncthreads();
+        }
+        if (sample) {
+            float xd[kIn], c = 0.f;
+#pragma unroll
+            for (int k = 0; k < kIn; ++k) xd[k] = 0.f;
+            if (valid) {
+                float4 u0, u1;
+                if (A.lab) {
+                    float e = 0.f;
+                    for (int g = 0; g < NG; ++g) e += Red[(size_t)g * S + tid];
+                    float gx[kIn];
+#pragma unroll
+                    for (int k = 0; k < kIn; ++k) {
+                        float a = 0.f;
+                        for (int q = 0; q < NS; ++q) a += Zs[(size_t)(q * kIn + k) * S + tid];
+                        gx[k] = e_scale * a * isd[k];
+                    }
+                    PairDst dst{};
+                    dst.sw_on = A.sw_on;
+                    dst.sw_inv = A.sw_inv;
+                    dst.out = A.pred;
+                    write_pair_outputs<false>(dst, b, geo, gx, e_scale * (e + b_o) + e_shift);
+                    loss += tr_residual(A, b, e_scale, u0, u1, c);
+                } else {
+                    u0 = A.ucfg[2 * b];
+                    u1 = A.ucfg[2 * b + 1];
+                    c = A.c[b];
+                }
+                tr_tangent(A, geo, A.cfg[2 * b], u0, u1, c, xd);
+            }
+#pragma unroll
+            for (int k = 0; k < kInPad; ++k) Us[k * LD + tid] = k < kIn ? xd[k] * isd[k] : 0.f;
+            cs[tid] = c;
+            bo_sum += c;
+        }
+        // ---- tangent forward: h_dot_l = phi' z_dot, (phi'' terms) z_dot; at the
+        // top the gradient of w_o and a_z_D = c g_D + (phi'' terms) z_dot
+        for (int l = 1; l <= D; ++l) {
+            tr_gemm<W, CPT, KC>(l == 1 ? Us : Ds + (size_t)(l - 2) * W * LD, l == 1 ? kInPad : W, feed, p0, o0, acc);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                TrVec<CPT> d1 = tr_ld<CPT>(slot(l - 1, j)), d2 = tr_ld<CPT>(slot(D + l - 1, j));
+#pragma unroll
+                for (int i = 0; i < CPT; ++i) {
+                    const float zd = tr_at<CPT>(acc, i, j);
+                    d1.v[i] *= zd;
+                    d2.v[i] *= zd;
+                }
+                const size_t at = (size_t)(o0 + j) * LD + p0;
+                if (l < D) {
+                    tr_st<CPT>(slot(D + l - 1, j), d2);
+                    tr_st<CPT>(Ds + (size_t)(l - 1) * W * LD + at, d1);
+                } else {
+                    const TrVec<CPT> h = tr_ld<CPT>(slot(2 * D, j)), g = tr_ld<CPT>(Gs + (size_t)(D - 1) * W * LD + at);
+                    float sum = 0.f;
+#pragma unroll
+                    for (int i = 0; i < CPT; ++i) {
+                        const float c = cs[p0 + i];
+                        sum += fmaf(c, h.v[i], d1.v[i]);
+                        d2.v[i] = fmaf(c, g.v[i], d2.v[i]);
+                    }
+                    tr_st<CPT>(Zs + at, d2);
+#pragma unroll
+                    for (int o = 1; o < NTP; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                    if (tp == 0) {
+                        float* q = gp + fl.wo + o0 + j;
+                        *q = first ? sum : *q + sum;
+                    }
+                }
+            }
+        }
+        // ---- reverse: dW_l, db_l, then a_z_{l-1} = (W_l^T a_z_l) phi' + (phi'' terms) z_dot
+        float* az = Zs;
+        for (int l = D; l >= 1; --l) {
+            __syncthreads();
+            const float* g = Gs + (size_t)(l - 1) * W * LD;
+            for (int o = tid; o < W; o += 256) {
+                float a = 0.f;
+                for (int c = 0; c < S; ++c) a += az[(size_t)o * LD + c];
+                float* q = gp + fl.b_(l, W) + o;
+                *q = first ? a : *q + a;
+            }
+            if (l == 1) {
+                for (int t = tid; t < W * 16; t += 256) {
+                    const int o = t >> 4, k = t & 15;
+                    if (k >= kIn) continue;
+                    float a = 0.f;
+                    for (int c = 0; c < S; ++c)
+                        a += az[(size_t)o * LD + c] * Xs[k * LD + c] + g[(size_t)o * LD + c] * Us[k * LD + c];
+                    float* q = gp + fl.W1 + o * kIn + k;
+                    *q = first ? a : *q + a;
+                }
+                break;
+            }
+            tr_weight_grad<W, S, LD>(az, Hs + (size_t)(l - 2) * W * LD, g, Ds + (size_t)(l - 2) * W * LD,
+                                     gp + fl.W_(l, W), first);
+            tr_gemm<W, CPT, KC>(az, W, feed, p0, o0, acc);
+            float* nz = Gs + (size_t)(l - 1) * W * LD;  // g_l has been used
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                TrVec<CPT> d1 = tr_ld<CPT>(slot(l - 2, j));
+                const TrVec<CPT> d2 = tr_ld<CPT>(slot(D + l - 2, j));
+#pragma unroll
+                for (int i = 0; i < CPT; ++i) d1.v[i] = fmaf(tr_at<CPT>(acc, i, j), d1.v[i], d2.v[i]);
+                tr_st<CPT>(nz + (size_t)(o0 + j) * LD + p0, d1);
+            }
+            az = nz;
+        }
+        __syncthreads();  // the next tile overwrites what this one read
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+    // the sample threads' sums, in order (Red and the arrays are free)
+    double* sl = reinterpret_cast<double*>(smem4);
+    float* sb = reinterpret_cast<float*>(sl + 256);
+    if (tid < S) {
+        sl[tid] = loss;
+        sb[tid] = bo_sum;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        double a = 0.0;
+        float f = 0.f;
+        for (int k = 0; k < S; ++k) {
+            a += sl[k];
+            f += sb[k];
+        }
+        loss_part[blockIdx.x] = a;
+        gp[fl.bo] = f;
+    }
 }
 
-__global__ void k_sum_partials(const double* __restrict__ part, int nb, double inv_n,
-                               double* __restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+// Sum of the CTAs' gradient shares (in order), Adam on the trainable parameters
+// when `step`, and the updated weights' prepared FP32 copies.  Block 0 also
+// sums the loss.
+struct AdamArgs {
+    float *p, *m, *v, *prep;
+    float lr, b1, b2, eps, c1, c2;
+};
+__global__ void __launch_bounds__(256)
+    k_train_update(int64_t np, int W, int D, int n_part, const float* __restrict__ part,
+                   float* __restrict__ grad, bool step, AdamArgs a, const double* __restrict__ loss_part,
+                   double inv_n, double* __restrict__ loss_out) {
+    pdl_wait();
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
         double x = 0.0;
-        for (int k = 0; k < nb; ++k) x += part[k];
-        *out = x * inv_n;
+        for (int k = threadIdx.x; k < n_part; k += 32) x += loss_part[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (threadIdx.x == 0) *loss_out = x * inv_n;
+    }
+    // 64 parameters per block, four threads each: a quarter of the shares, in
+    // order, then the quarters in order
+    __shared__ float s_q[4][64];
+    const int lane = threadIdx.x & 63, q = threadIdx.x >> 6;
+    const int64_t t = blockIdx.x * (int64_t)64 + lane;
+    const FlatLayout f = flat_layout(W, D);
+    const bool train = t >= f.W1 && t < f.escale;
+    float g = 0.f;
+    if (train) {
+        const int per = (n_part + 3) / 4, e = min(n_part, (q + 1) * per);
+        int k = q * per;
+        for (; k + 16 <= e; k += 16) {
+            float v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[u] = part[(size_t)(k + u) * np + t];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) g += v[u];
+        }
+        for (; k < e; ++k) g += part[(size_t)k * np + t];
+    }
+    s_q[q][lane] = g;
+    __syncthreads();
+    if (q > 0 || t >= np) return;
+    g = ((s_q[0][lane] + s_q[1][lane]) + s_q[2][lane]) + s_q[3][lane];
+    grad[t] = g;
+    if (!step || !train) return;
+    const float p = adam_update(a.p[t], g, a.m[t], a.v[t], a.lr, a.b1, a.b2, a.eps, a.c1, a.c2);
+    a.p[t] = p;
+    const F32Layout L = f32_layout(W, D);
+    if (t < f.b1) {
+        const int e = (int)(t - f.W1), o = e / kIn, k = e % kIn;
+        a.prep[L.wt1 + (int64_t)k * W + o] = p;
+        a.prep[L.w1p + (int64_t)o * kInPad + k] = p;
+    } else if (t >= f.Wl && t < f.wo) {
+        const int64_t r = t - f.Wl, wl = (int64_t)W * W + W;
+        const int l = (int)(r / wl);  // layer l + 2
+        const int64_t e = r % wl;
+        if (e < (int64_t)W * W) {
+            const int64_t o = e / W, k = e % W;
+            a.prep[L.wt + (int64_t)l * W * W + k * W + o] = p;
+            a.prep[L.wr + (int64_t)l * W * W + e] = p;
+        }
     }
 }
 
@@ -468,184 +898,90 @@ __global__ void k_adam(int64_t n, int64_t lo, int64_t hi, float* __restrict__ p,
                        float lr, float b1, float b2, float eps, float c1, float c2) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= n || t < lo || t >= hi) return;
-    const float gt = g[t];
-    const float mt = b1 * m[t] + (1.f - b1) * gt;
-    const float vt = b2 * v[t] + (1.f - b2) * gt * gt;
-    m[t] = mt;
-    v[t] = vt;
-    p[t] -= lr * (mt / c1) / (sqrtf(vt / c2) + eps);
+    p[t] = adam_update(p[t], g[t], m[t], v[t], lr, b1, b2, eps, c1, c2);
 }
 
-static inline unsigned nblk(int64_t n, int t = 256) { return (unsigned)std::max<int64_t>(1, (n + t - 1) / t); }
+static inline unsigned nblk(int64_t n, int t) { return (unsigned)std::max<int64_t>(1, (n + t - 1) / t); }
 
-// Workspace layout for batch B, width W, depth D (floats):
-//   X, U [B x 16]; per layer Z, Zd, H, Hd [B x W]; Ah0, Ahd0, Ah1, Ahd1 [B x W];
-//   T [B x W]; c [B]; ucfg, pred [B x 8], [B x 12]; G16 [W x 16];
-//   cfg_c, ucfg_c [B x 8] (canonical configurations and tangents);
-//   u_sw [B x 8], c_sw [B] (tangents and coefficients of the switched energy);
-//   SK [kSplitMax x W x W] (split-K partial tiles of the weight gradients)
-struct TrWork {
-    float *X, *U, *Z[4], *Zd[4], *H[4], *Hd[4], *Ah[2], *Ahd[2], *T, *c, *ucfg, *pred, *G16;
-    float *cfg_c, *ucfg_c, *u_sw, *c_sw, *SK;
-};
-static size_t tr_split_floats(int W) { return (size_t)kSplitMax * W * std::max(W, kInPad); }
-static size_t tr_work_floats(int64_t B, int W, int D) {
-    return (size_t)B * 32 + (size_t)D * 4 * B * W + 5 * (size_t)B * W + B + 8 * B + 12 * B +
-           (size_t)W * 16 + 25 * (size_t)B + tr_split_floats(W) +
-           16 * 49;  // + rounding of every buffer to 16
+// Tiles of 4 samples per thread; 2 where a batch would leave half of the SMs
+// without a tile (a step of width 128: 59.6 against 73.9 us for 1000 samples,
+// 63.7 against 75.9 us for 2048; from 3000 on both forms fill the GPU), and at
+// depth 4, whose arrays would not fit.
+static int tr_cols(const rb_trainer* t, int64_t B) {
+    const int W = t->mlp->width;
+    return t->mlp->depth > 3 || B * W <= (int64_t)4096 * (t->sms / 2) ? 2 : 4;
 }
-static TrWork tr_work(float* base, int64_t B, int W, int D) {
-    TrWork w{};
-    float* p = base;
-    auto take = [&](size_t n) {
-        float* r = p;
-        p += (n + 15) & ~size_t(15);
-        return r;
-    };
-    w.X = take(B * 16);
-    w.U = take(B * 16);
-    for (int l = 0; l < D; ++l) {
-        w.Z[l] = take((size_t)B * W);
-        w.Zd[l] = take((size_t)B * W);
-        w.H[l] = take((size_t)B * W);
-        w.Hd[l] = take((size_t)B * W);
-    }
-    for (int k = 0; k < 2; ++k) {
-        w.Ah[k] = take((size_t)B * W);
-        w.Ahd[k] = take((size_t)B * W);
-    }
-    w.T = take((size_t)B * W);
-    w.c = take(B);
-    w.ucfg = take(8 * B);
-    w.pred = take(12 * B);
-    w.G16 = take((size_t)W * 16);
-    w.cfg_c = take(8 * B);
-    w.ucfg_c = take(8 * B);
-    w.u_sw = take(8 * B);
-    w.c_sw = take(B);
-    w.SK = take(tr_split_floats(W));
-    return w;
+static int tr_grid(const rb_trainer* t, int64_t B, int cols) {
+    const int64_t S = 1024 * cols / t->mlp->width;
+    return (int)std::min<int64_t>((B + S - 1) / S, t->sms);
 }
 
-// With the smooth cutoff the output is S(rho) E_hat: d/dW [u . grad(S E_hat) +
-// c S E_hat] = d/dW [u' . grad E_hat + c' E_hat] with u' = S u and
-// c' = S c + S' (u_s . s / rho), since grad(S E_hat) = S grad E_hat + E_hat S'
-// grad rho and rho = |s|.
-__global__ void k_switch_tangent(int64_t n, const float4* __restrict__ cfg,
-                                 const float4* __restrict__ ucfg, const float* __restrict__ c,
-                                 float on, float inv, float4* __restrict__ u_out,
-                                 float* __restrict__ c_out) {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= n) return;
-    const float4 c0 = cfg[2 * b];
-    const float rho = sqrtf(c0.x * c0.x + c0.y * c0.y + c0.z * c0.z);
-    float S, dS;
-    cutoff_switch(rho, on, inv, S, dS);
-    const float4 u0 = ucfg[2 * b], u1 = ucfg[2 * b + 1];
-    c_out[b] = S * c[b] + dS * (u0.x * c0.x + u0.y * c0.y + u0.z * c0.z) / rho;
-    u_out[2 * b] = make_float4(S * u0.x, S * u0.y, S * u0.z, 0.f);
-    u_out[2 * b + 1] = make_float4(S * u1.x, S * u1.y, S * u1.z, S * u1.w);
-}
-
-// grad = d/dW sum_b [u_b . grad_(s,q) E_hat_b + c_b E_hat_b] (flat layout; the
-// normalisation and output-scale entries stay zero).
-static rb_status weight_vjp(rb_trainer* tr, int64_t B, const float4* cfg, const float4* ucfg,
-                            const float* c, float* grad) {
-    rb_mlp* m = tr->mlp;
-    const int W = m->width, D = m->depth;
-    const FlatLayout fl = flat_layout(W, D);
-    cudaStream_t st = m->stream;
-    TrWork w = tr_work(tr->work, tr->max_batch, W, D);
-    const float* flat = m->params;
-    RB_CUDA(cudaMemsetAsync(grad, 0, sizeof(float) * m->n_params, st));
-    if (m->sw_off > m->sw_on) {  // switched output S E_hat (see k_switch_tangent)
-        k_switch_tangent<<<nblk(B), 256, 0, st>>>(B, cfg, ucfg, c, m->sw_on,
-                                                  1.f / (m->sw_off - m->sw_on),
-                                                  reinterpret_cast<float4*>(w.u_sw), w.c_sw);
-        ucfg = reinterpret_cast<const float4*>(w.u_sw);
-        c = w.c_sw;
+template <int W, int CPT, int KC>
+static rb_status launch_tile(rb_trainer* t, int grid, const PairSrc& src, const TrArgs& A) {
+    rb_mlp* m = t->mlp;
+    const size_t smem = TrShape<W, CPT, KC>::smem(m->depth);
+    static std::atomic<size_t> allowed{0};
+    if (smem > allowed.load()) {
+        RB_CUDA(cudaFuncSetAttribute(k_train_tile<W, CPT, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     227 * 1024));
+        allowed.store(227 * 1024);
     }
-    if (m->n_sym > 0) {  // the network sees canonical configurations: map cfg and u
-        PairSrc sym{};
-        set_symmetry(sym, m);
-        k_canon_tangent<<<nblk(B), 256, 0, st>>>(B, sym, cfg, ucfg,
-                                                 reinterpret_cast<float4*>(w.cfg_c),
-                                                 reinterpret_cast<float4*>(w.ucfg_c));
-        cfg = reinterpret_cast<const float4*>(w.cfg_c);
-        ucfg = reinterpret_cast<const float4*>(w.ucfg_c);
-    }
-    k_tr_inputs<<<nblk(B), 256, 0, st>>>(B, cfg, ucfg, flat, fl, m->desc, w.X, w.U);
-    // forward with tangent
-    const float* W1p = m->f32_prep + (int64_t)kInPad * W + (int64_t)(D - 1) * W * W;  // [W][16]
-    for (int l = 1; l <= D; ++l) {
-        const float* Ain = l == 1 ? w.X : w.H[l - 2];
-        const float* Uin = l == 1 ? w.U : w.Hd[l - 2];
-        const int K = l == 1 ? kInPad : W;
-        const float* Wl = l == 1 ? W1p : flat + fl.W_(l, W);  // [W][K] row-major
-        RB_TRY(sgemm(st, (int)B, W, K, Ain, K, 1, Wl, 1, K, w.Z[l - 1], W, 1.f, 0.f, m->status_dev));
-        RB_TRY(sgemm(st, (int)B, W, K, Uin, K, 1, Wl, 1, K, w.Zd[l - 1], W, 1.f, 0.f, m->status_dev));
-        k_tr_act<<<nblk(B * W), 256, 0, st>>>(B, W, flat + fl.b_(l, W), w.Z[l - 1], w.Zd[l - 1],
-                                              w.H[l - 1], w.Hd[l - 1]);
-    }
-    // output layer gradients
-    k_tr_wo<<<nblk(B * W), 256, 0, st>>>(B, W, w.H[D - 1], w.Hd[D - 1], c, w.T);
-    k_colsum<<<W, 256, 0, st>>>((int)B, W, w.T, W, grad + fl.wo, 0);
-    k_colsum<<<1, 256, 0, st>>>((int)B, 1, c, 1, grad + fl.bo, 0);
-    // reverse
-    int cur = 0;
-    k_tr_seed<<<nblk(B * W), 256, 0, st>>>(B, W, flat + fl.wo, c, w.Ah[0], w.Ahd[0]);
-    for (int l = D; l >= 1; --l) {
-        k_tr_back<<<nblk(B * W), 256, 0, st>>>(B, W, w.Z[l - 1], w.Zd[l - 1], w.Ah[cur], w.Ahd[cur]);
-        k_colsum<<<W, 256, 0, st>>>((int)B, W, w.Ah[cur], W, grad + fl.b_(l, W), 0);
-        const float* Hp = l == 1 ? w.X : w.H[l - 2];
-        const float* Hdp = l == 1 ? w.U : w.Hd[l - 2];
-        const int K = l == 1 ? kInPad : W;
-        float* gW = l == 1 ? w.G16 : grad + fl.W_(l, W);
-        // gW[o][i] = sum_b Az[b][o] Hp[b][i] + Azd[b][o] Hdp[b][i]
-        RB_TRY(sgemm(st, W, K, (int)B, w.Ah[cur], 1, W, Hp, K, 1, gW, K, 1.f, 0.f, m->status_dev,
-                     w.SK, tr_split_floats(W)));
-        RB_TRY(sgemm(st, W, K, (int)B, w.Ahd[cur], 1, W, Hdp, K, 1, gW, K, 1.f, 1.f, m->status_dev,
-                     w.SK, tr_split_floats(W)));
-        if (l == 1) {
-            k_tr_w1<<<nblk(W * kIn), 256, 0, st>>>(W, w.G16, grad + fl.W1);
-        } else {
-            const float* Wl = flat + fl.W_(l, W);  // a_{l-1} = a_l W_l: B(k=o, n=i) = W[o][i]
-            RB_TRY(sgemm(st, (int)B, W, W, w.Ah[cur], W, 1, Wl, W, 1, w.Ah[1 - cur], W, 1.f, 0.f,
-                         m->status_dev));
-            RB_TRY(sgemm(st, (int)B, W, W, w.Ahd[cur], W, 1, Wl, W, 1, w.Ahd[1 - cur], W, 1.f, 0.f,
-                         m->status_dev));
-            cur = 1 - cur;
-        }
-    }
-    RB_CUDA(cudaGetLastError());
+    RB_CUDA(launch_pdl(k_train_tile<W, CPT, KC>, grid, 256, smem, m->stream, m->params, m->f32_prep,
+                       flat_layout(W, m->depth), f32_layout(W, m->depth), m->depth, src, A, t->part,
+                       m->n_params, t->scratch, t->loss_part));
     return RB_OK;
 }
 
-static rb_status train_grad(rb_trainer* tr, int64_t B, const float* cfg, const float* labels,
-                            float lam_tau, float lam_E, float f_scale, float kT_w,
-                            double* loss_host) {
-    rb_mlp* m = tr->mlp;
-    const int W = m->width, D = m->depth;
-    TrWork w = tr_work(tr->work, tr->max_batch, W, D);
-    cudaStream_t st = m->stream;
-    // network outputs and their (s, q) gradient at the current weights (FP32 kernel)
-    RB_TRY(nn_pairs_f32_async(m, B, reinterpret_cast<const float4*>(cfg),
-                              reinterpret_cast<float4*>(w.pred), nullptr));
-    const FlatLayout fl = flat_layout(W, D);
-    const unsigned nb = nblk(B);
-    k_tr_residual<<<nb, 256, 0, st>>>(B, reinterpret_cast<const float4*>(cfg),
-                                      reinterpret_cast<const float4*>(w.pred),
-                                      reinterpret_cast<const float4*>(labels), lam_tau, lam_E,
-                                      f_scale > 0.f ? 1.f / (f_scale * f_scale) : 0.f,
-                                      kT_w > 0.f ? 1.f / kT_w : 0.f, m->params + fl.escale,
-                                      1.f / (float)B,
-                                      reinterpret_cast<float4*>(w.ucfg), w.c, tr->loss_part);
-    k_sum_partials<<<1, 32, 0, st>>>(tr->loss_part, (int)nb, 1.0 / (double)B, tr->loss_out);
-    RB_TRY(weight_vjp(tr, B, reinterpret_cast<const float4*>(cfg),
-                      reinterpret_cast<const float4*>(w.ucfg), w.c, tr->grad));
+// The gradient of a batch into `grad` (and the parameters' Adam step).
+static rb_status train_pass(rb_trainer* t, TrArgs A, float* grad, bool step) {
+    rb_mlp* m = t->mlp;
+    PairSrc src{};
+    set_symmetry(src, m);
+    src.cfg = A.cfg;
+    src.n_explicit = A.n;
+    A.pred = reinterpret_cast<float4*>(t->pred);
+    A.sw_on = m->sw_on;
+    A.sw_inv = m->sw_off > m->sw_on ? 1.f / (m->sw_off - m->sw_on) : 0.f;
+    A.inv_n = 1.f / (float)A.n;
+    const int cols = tr_cols(t, A.n), grid = tr_grid(t, A.n, cols);
+    switch (m->width * 8 + cols) {
+        case 64 * 8 + 4: RB_TRY((launch_tile<64, 4, 64>(t, grid, src, A))); break;
+        case 64 * 8 + 2: RB_TRY((launch_tile<64, 2, 64>(t, grid, src, A))); break;
+        case 128 * 8 + 4: RB_TRY((launch_tile<128, 4, 64>(t, grid, src, A))); break;
+        case 128 * 8 + 2: RB_TRY((launch_tile<128, 2, 32>(t, grid, src, A))); break;
+        case 256 * 8 + 4: RB_TRY((launch_tile<256, 4, 16>(t, grid, src, A))); break;
+        case 256 * 8 + 2: RB_TRY((launch_tile<256, 2, 16>(t, grid, src, A))); break;
+        default: return fail(RB_ENOTSUP, "training supports widths 64, 128, 256");
+    }
+    AdamArgs a{m->params, t->m, t->v, m->f32_prep, t->lr, t->beta1, t->beta2, t->eps, 1.f, 1.f};
+    if (step) {
+        t->t += 1;
+        // Bias corrections 1 - beta^t in FP64: in FP32, 1 - beta2^t loses about
+        // five digits to cancellation (beta2^t is within 1e-3 of 1 early on).
+        a.c1 = (float)(1.0 - std::pow((double)t->beta1, (double)t->t));
+        a.c2 = (float)(1.0 - std::pow((double)t->beta2, (double)t->t));
+    }
+    RB_CUDA(launch_pdl(k_train_update, nblk(m->n_params, 64), 256, 0, m->stream, m->n_params, m->width, m->depth,
+                       grid, t->part, grad, step, a, t->loss_part, 1.0 / (double)A.n, t->loss_out));
+    if (step) m->version++;  // the BF16 / F16X3 images follow on their next use (ensure_images)
+    return RB_OK;
+}
+
+static rb_status train_batch(rb_trainer* t, int64_t B, const float* cfg, const float* labels, float lam_tau,
+                             float lam_E, float f_scale, float kT_w, bool step, double* loss_host) {
+    RB_TRY(check_mlp(t->mlp));
+    TrArgs A{};
+    A.n = B;
+    A.cfg = reinterpret_cast<const float4*>(cfg);
+    A.lab = reinterpret_cast<const float4*>(labels);
+    A.lam_tau = lam_tau;
+    A.lam_E = lam_E;
+    A.inv_f2 = f_scale > 0.f ? 1.f / (f_scale * f_scale) : 0.f;
+    A.inv_kTw = kT_w > 0.f ? 1.f / kT_w : 0.f;
+    RB_TRY(train_pass(t, A, t->grad, step));
     if (loss_host) {
-        RB_CUDA(cudaMemcpyAsync(loss_host, tr->loss_out, sizeof(double), cudaMemcpyDeviceToHost, st));
-        RB_CUDA(cudaStreamSynchronize(st));
+        RB_CUDA(cudaMemcpyAsync(loss_host, t->loss_out, sizeof(double), cudaMemcpyDeviceToHost, t->mlp->stream));
+        RB_CUDA(cudaStreamSynchronize(t->mlp->stream));
     }
     return RB_OK;
 }
@@ -745,12 +1081,17 @@ rb_status rb_trainer_create(rb_mlp* mlp, int64_t max_batch, float lr, float beta
     t->beta2 = beta2;
     t->eps = eps;
     const int64_t np = mlp->n_params;
-    t->work_floats = tr_work_floats(max_batch, mlp->width, mlp->depth);
+    cudaDeviceGetAttribute(&t->sms, cudaDevAttrMultiProcessorCount, mlp->device);
+    // the most CTAs a batch of up to max_batch takes, in either tile form
+    const size_t ctas = std::max(tr_grid(t, max_batch, 2), tr_grid(t, max_batch, 4));
     cudaError_t e = cudaMalloc(&t->m, sizeof(float) * np);
     if (e == cudaSuccess) e = cudaMalloc(&t->v, sizeof(float) * np);
     if (e == cudaSuccess) e = cudaMalloc(&t->grad, sizeof(float) * np);
-    if (e == cudaSuccess) e = cudaMalloc(&t->work, sizeof(float) * t->work_floats);
-    if (e == cudaSuccess) e = cudaMalloc(&t->loss_part, sizeof(double) * (max_batch / 256 + 2));
+    if (e == cudaSuccess) e = cudaMalloc(&t->pred, sizeof(float4) * 3 * max_batch);
+    if (e == cudaSuccess) e = cudaMalloc(&t->part, sizeof(float) * np * ctas);
+    if (e == cudaSuccess)
+        e = cudaMalloc(&t->scratch, sizeof(float) * tr_slots(mlp->depth) * kTrSlotFloats * 4 * ctas);
+    if (e == cudaSuccess) e = cudaMalloc(&t->loss_part, sizeof(double) * ctas);
     if (e == cudaSuccess) e = cudaMalloc(&t->loss_out, sizeof(double));
     if (e == cudaSuccess) e = cudaMemsetAsync(t->m, 0, sizeof(float) * np, mlp->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(t->v, 0, sizeof(float) * np, mlp->stream);
@@ -771,7 +1112,7 @@ rb_status rb_trainer_set_lr(rb_trainer* t, float lr) {
 rb_status rb_trainer_destroy(rb_trainer* t) {
     if (!t) return RB_OK;
     if (t->mlp && t->mlp->stream) cudaStreamSynchronize(t->mlp->stream);
-    void* ptrs[] = {t->m, t->v, t->grad, t->work, t->loss_part, t->loss_out};
+    void* ptrs[] = {t->m, t->v, t->grad, t->pred, t->part, t->scratch, t->loss_part, t->loss_out};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete t;
@@ -783,7 +1124,7 @@ rb_status rb_train_grad(rb_trainer* t, int64_t batch, const float* cfg, const fl
                         double* loss_host) {
     if (!t || !cfg || !labels) return fail(RB_EINVAL, "null argument");
     if (batch < 1 || batch > t->max_batch) return fail(RB_EINVAL, "batch out of range");
-    RB_TRY(train_grad(t, batch, cfg, labels, lam_tau, lam_E, f_scale, kT_w, loss_host));
+    RB_TRY(train_batch(t, batch, cfg, labels, lam_tau, lam_E, f_scale, kT_w, false, loss_host));
     if (grad_out)
         RB_CUDA(cudaMemcpyAsync(grad_out, t->grad, sizeof(float) * t->mlp->n_params,
                                 cudaMemcpyDeviceToDevice, t->mlp->stream));
@@ -795,26 +1136,20 @@ rb_status rb_train_step(rb_trainer* t, int64_t batch, const float* cfg, const fl
                         double* loss_host) {
     if (!t || !cfg || !labels) return fail(RB_EINVAL, "null argument");
     if (batch < 1 || batch > t->max_batch) return fail(RB_EINVAL, "batch out of range");
-    RB_TRY(train_grad(t, batch, cfg, labels, lam_tau, lam_E, f_scale, kT_w, loss_host));
-    rb_mlp* m = t->mlp;
-    t->t += 1;
-    // Bias corrections 1 - beta^t in FP64: in FP32, 1 - beta2^t loses about
-    // five digits to cancellation (beta2^t is within 1e-3 of 1 early on).
-    const float c1 = (float)(1.0 - std::pow((double)t->beta1, (double)t->t));
-    const float c2 = (float)(1.0 - std::pow((double)t->beta2, (double)t->t));
-    const int64_t np = m->n_params;
-    k_adam<<<nblk(np), 256, 0, m->stream>>>(np, 2 * kIn, np - 2, m->params, t->grad, t->m, t->v,
-                                            t->lr, t->beta1, t->beta2, t->eps, c1, c2);
-    RB_CUDA(cudaGetLastError());
-    return mlp_refresh(m);
+    return train_batch(t, batch, cfg, labels, lam_tau, lam_E, f_scale, kT_w, true, loss_host);
 }
 
 rb_status rb_nn_weight_vjp(rb_trainer* t, int64_t n, const float* cfg, const float* u_cfg,
                            const float* c, float* grad_out) {
     if (!t || !cfg || !u_cfg || !c || !grad_out) return fail(RB_EINVAL, "null argument");
     if (n < 1 || n > t->max_batch) return fail(RB_EINVAL, "n out of range");
-    return weight_vjp(t, n, reinterpret_cast<const float4*>(cfg),
-                      reinterpret_cast<const float4*>(u_cfg), c, grad_out);
+    RB_TRY(check_mlp(t->mlp));
+    TrArgs A{};
+    A.n = n;
+    A.cfg = reinterpret_cast<const float4*>(cfg);
+    A.ucfg = reinterpret_cast<const float4*>(u_cfg);
+    A.c = c;
+    return train_pass(t, A, grad_out, false);
 }
 
 }  // extern "C"
