@@ -26,13 +26,13 @@
 // L = mean_b w_b sum_c (y_c - t_c)^2, the targets optionally capped to
 // [-cap, cap] (the paper caps the wide force and torque range of its training
 // data, SI Sec. 6) and optionally weighted, w_b = 1 / (1 + |t_b|^2 / f^2)
-// (else 1), forward and backward passes as fixed-order GEMMs
-// (deterministic), Adam.
+// (else 1); one kernel for the gradient (a CTA per network and tile of
+// samples), one for the fixed-order sum of its shares and Adam.
 #include <algorithm>
 #include <cmath>
 #include <new>
 
-#include "rb_internal.cuh"
+#include "nn_f32_common.cuh"
 
 struct rb_fnet {
     int device = 0;
@@ -42,6 +42,7 @@ struct rb_fnet {
     int64_t img_floats = 0;   // one network, kernel image (multiple of 4)
     float* params = nullptr;  // 5 networks, flat FP32 (device), the ABI layout
     float* img = nullptr;     // 5 networks, kernel image (device)
+    float* wr = nullptr;      // 5 x (D-1) hidden matrices as stored, [out][in] (training's reverse pass)
     uint64_t version = 1;
     std::atomic<uint64_t> ready_version{0};  // the version other streams have waited for
 };
@@ -52,12 +53,11 @@ struct rb_fnet_trainer {
     float lr = 1e-3f, beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
     int64_t t = 0;
     float *m = nullptr, *v = nullptr, *grad = nullptr;
-    float* work = nullptr;
-    float* sk = nullptr;          // split-K partial tiles of the weight gradients
-    size_t sk_floats = 0;
-    double* loss_part = nullptr;  // per block, 5 networks
+    float* part = nullptr;        // per CTA: its share of one network's gradient (net_floats)
+    float* scratch = nullptr;     // per CTA: silu' of its tile and the top activations
+    double* loss_part = nullptr;  // per CTA
     double* loss_out = nullptr;
-    int loss_blocks = 0;
+    int sms = 1;
     float cap = 0.f;      // targets clamped to [-cap, cap] (0: no cap)
     float f_scale = 0.f;  // sample weight 1 / (1 + |t|^2 / f_scale^2) (0: none)
 };
@@ -95,9 +95,17 @@ __host__ __device__ inline FnLayout fn_layout(int W, int D) {
 
 // Kernel image: the flat layout with every weight matrix transposed
 // ([out][in] -> [in][out]), padded to a multiple of 4 floats.
-__global__ void k_fn_prepare(const float* __restrict__ flat, int W, int D, float* __restrict__ img) {
+// wr: the hidden matrices as stored, 16-byte aligned.
+__global__ void k_fn_prepare(const float* __restrict__ flat, int W, int D, float* __restrict__ img,
+                             float* __restrict__ wr) {
     const int64_t n = fn_net_size(W, D), m = fn_img_size(W, D);
     const FnLayout L = fn_layout(W, D);
+    const int64_t ww = (int64_t)W * W, nw = (int64_t)kFnNets * (D - 1) * ww;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nw;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t k = t / ww;  // network and layer
+        wr[t] = flat[k / (D - 1) * n + L.w(1 + (int)(k % (D - 1))) + t % ww];
+    }
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < kFnNets * m;
          t += (int64_t)gridDim.x * blockDim.x) {
         const int c = (int)(t / m);
@@ -357,175 +365,385 @@ rb_status fnet_pairs_system_async(rb_system* s, const rb_fnet* f) {
 }
 
 // ------------------------------------------------------------- training
-// Descriptions and targets of a sampled batch: X[b] (4), T[b] (5 components).
-__global__ void k_fn_inputs(int64_t n, const float4* __restrict__ cfg, const float4* __restrict__ lab,
-                            float cap, float f_scale, float* __restrict__ X, float* __restrict__ T,
-                            float* __restrict__ Wb) {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= n) return;
-    const float4 c0 = cfg[2 * b], c1 = cfg[2 * b + 1];
-    const FnFrame f = fn_frame(make_float3(c0.x, c0.y, c0.z), c1);
-    const float4 F = lab[3 * b], ti = lab[3 * b + 1];
-#pragma unroll
-    for (int k = 0; k < kFnIn; ++k) X[4 * b + k] = f.d[k];
-    float t[5] = {F.x * f.xh.x + F.y * f.xh.y, F.x * f.yh.x + F.y * f.yh.y, F.z * f.zh.z,
-                  ti.x * f.xh.x + ti.y * f.xh.y, ti.x * f.yh.x + ti.y * f.yh.y};
-    float t2 = 0.f;
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-        t[c] = cap > 0.f ? fminf(fmaxf(t[c], -cap), cap) : t[c];
-        T[5 * b + c] = t[c];
-        t2 = fmaf(t[c], t[c], t2);
+// The gradient of L for one network and a tile of S = 4096 / W samples per CTA
+// and pass (blockIdx: network x share of the tiles): description, target and
+// weight of every sample, forward, residual, backward, and the layer gradients
+// added to the CTA's own share.  A thread owns 4 samples x 4 units of every
+// layer; activations and signals live in shared memory as [unit][sample] (row
+// stride S + 4, so that rows of consecutive units fall on different banks),
+// silu' and the top activations, which only their own thread reads again, in a
+// global scratch; the weights (4 KB a matrix at width 32) come through L1.
+// A step was about 130 launches (GEMMs, column sums and elementwise kernels of
+// the five networks one after the other, 880 us at batch 4096 and width 32, for
+// 0.27 GFLOP); it is two, 40 us (this kernel 34 us), and the gradient's error
+// against FP64 went from 8.6e-7 to 1.1e-7.  Bound by latency: a dozen dependent
+// short stages.
+struct FnTrainArgs {
+    int64_t n;
+    const float4 *cfg, *lab;
+    float cap, f_scale;
+};
+
+constexpr int kFnCpt = 4;
+template <int W>
+struct FnTile {
+    static constexpr int S = 1024 * kFnCpt / W, LD = S + 4;
+    static constexpr int NTP = S / kFnCpt, NG = W / 4;
+    static constexpr int kWarpsPerUnit = NTP > 32 ? NTP / 32 : 1;
+    static size_t smem(int D) {
+        return sizeof(float) * ((size_t)(D + 1) * W * LD + kFnIn * LD + NG * S + 2 * S + kWarpsPerUnit * W + 16) +
+               sizeof(double) * 256;
     }
-    Wb[b] = f_scale > 0.f ? 1.f / (1.f + t2 / (f_scale * f_scale)) : 1.f;
-}
+};
+__host__ __device__ inline size_t fn_scratch_floats(int D) { return (size_t)(D + 1) * 4 * 256 * kFnCpt; }
 
-// Normalised inputs of network c: Xc[b][k] = (X[b][k] - mu_k) inv_sd_k.
-__global__ void k_fn_norm(int64_t n, const float* __restrict__ X, const float* __restrict__ net,
-                          float* __restrict__ Xc) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= 4 * n) return;
-    const int k = (int)(t % 4);
-    Xc[t] = (X[t] - net[k]) * net[4 + k];
-}
-
-// Z += b (per column); S = silu'(Z); H = silu(Z).
-__global__ void k_fn_act(int64_t n, int W, const float* __restrict__ bias, float* __restrict__ Z,
-                         float* __restrict__ H, float* __restrict__ S) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= n * W) return;
-    const float z = Z[t] + bias[t % W];
-    const float sg = 1.f / (1.f + __expf(-z));
-    H[t] = z * sg;
-    S[t] = sg * (1.f + z * (1.f - sg));
-}
-
-// Output of network c, the residual r = 2 (y - t_c) / n scaled by y_scale
-// (the gradient of L with respect to w_o . h + b_o) and per-block sums of the
-// squared errors (fixed order).
-__global__ void k_fn_out(int64_t n, int W, const float* __restrict__ H, const float* __restrict__ net,
-                         int64_t wo, const float* __restrict__ T, const float* __restrict__ Wb, int c,
-                         float* __restrict__ r, double* __restrict__ part) {
-    __shared__ double sh[256];
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    double e2 = 0.0;
-    if (b < n) {
-        float y = net[wo + W];
-        for (int o = 0; o < W; ++o) y = fmaf(net[wo + o], H[b * W + o], y);
-        const float ys = net[wo + W + 1];
-        const float yv = fmaf(ys, y, net[wo + W + 2]);
-        const float d = yv - T[5 * b + c];
-        r[b] = 2.f * Wb[b] * d / (float)n * ys;
-        e2 = (double)Wb[b] * d * d;
+// out[o * W + i] (+)= sum_c A[o][c] B[i][c], every thread W * W / 256 outputs.
+template <int W>
+__device__ inline void fn_weight_grad(const float* __restrict__ A, const float* __restrict__ B,
+                                      float* __restrict__ out, bool first) {
+    constexpr int S = FnTile<W>::S, LD = FnTile<W>::LD;
+    constexpr int LI = W < 32 ? W : 32;               // lanes along i
+    constexpr int IN = W / LI, RO = 8 * (32 / LI), ON = W / RO;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i0 = lane % LI, r0 = warp * (32 / LI) + lane / LI;
+    float2 acc[ON][IN];
+#pragma unroll
+    for (int o = 0; o < ON; ++o)
+#pragma unroll
+        for (int j = 0; j < IN; ++j) acc[o][j] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int c = 0; c < S; c += 4) {
+        float4 b[IN];
+#pragma unroll
+        for (int j = 0; j < IN; ++j) b[j] = *reinterpret_cast<const float4*>(B + (i0 + LI * j) * LD + c);
+#pragma unroll
+        for (int o = 0; o < ON; ++o) {
+            const float4 a = *reinterpret_cast<const float4*>(A + (r0 + RO * o) * LD + c);
+#pragma unroll
+            for (int j = 0; j < IN; ++j) {
+                acc[o][j] = __ffma2_rn(make_float2(a.x, a.y), make_float2(b[j].x, b[j].y), acc[o][j]);
+                acc[o][j] = __ffma2_rn(make_float2(a.z, a.w), make_float2(b[j].z, b[j].w), acc[o][j]);
+            }
+        }
     }
-    sh[threadIdx.x] = e2;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+#pragma unroll
+    for (int o = 0; o < ON; ++o)
+#pragma unroll
+        for (int j = 0; j < IN; ++j) {
+            float* p = out + (r0 + RO * o) * W + i0 + LI * j;
+            const float v = acc[o][j].x + acc[o][j].y;
+            *p = first ? v : *p + v;
+        }
+}
+
+// acc[i][.] = sum_k A[k][p0 + i] B[k][o0 + .], A in shared memory, B global.
+template <int W>
+__device__ inline void fn_gemm(const float* __restrict__ As, const float* __restrict__ B, int K, int p0, int o0,
+                               float2 (&acc)[kFnCpt][2]) {
+#pragma unroll
+    for (int i = 0; i < kFnCpt; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
+#pragma unroll 8
+    for (int k = 0; k < K; ++k) {
+        const TrVec<kFnCpt> a = tr_ld<kFnCpt>(As + k * FnTile<W>::LD + p0);
+        const float4 b = *reinterpret_cast<const float4*>(B + k * W + o0);
+        const float2 b0 = make_float2(b.x, b.y), b1 = make_float2(b.z, b.w);
+#pragma unroll
+        for (int i = 0; i < kFnCpt; ++i) {
+            const float2 aa = make_float2(a.v[i], a.v[i]);
+            acc[i][0] = __ffma2_rn(aa, b0, acc[i][0]);
+            acc[i][1] = __ffma2_rn(aa, b1, acc[i][1]);
+        }
+    }
+}
+
+template <int W>
+__global__ void __launch_bounds__(256)
+    k_fn_tile(const float* __restrict__ img, int64_t img_sz, const float* __restrict__ wr, int D, FnTrainArgs A,
+              float* __restrict__ part, int64_t nn, float* __restrict__ scratch,
+              double* __restrict__ loss_part) {
+    using T = FnTile<W>;
+    constexpr int S = T::S, LD = T::LD, NTP = T::NTP, NG = T::NG;
+    pdl_wait();
+    extern __shared__ double smem_d[];
+    double* s_loss = smem_d;                                 // 256
+    float* Hs = reinterpret_cast<float*>(smem_d + 256);      // h_1 .. h_{D-1}
+    float* G0 = Hs + (size_t)(D - 1) * W * LD;               // signals of a layer, two in turn
+    float* G1 = G0 + W * LD;
+    float* Xs = G1 + W * LD;                                 // [4][LD] normalised inputs
+    float* Red = Xs + kFnIn * LD;                            // [NG][S] partial sums of w_o . h
+    float* ts = Red + NG * S;                                // S residuals
+    float* Wp = ts + 2 * S;                                  // [warps per unit][W] partial sums of w_o's gradient
+    const int tid = threadIdx.x, tp = tid % NTP, to = tid / NTP;
+    const int p0 = tp * kFnCpt, o0 = to * 4;
+    const int c = blockIdx.x, share = blockIdx.y, n_share = gridDim.y;
+    const int cta = c * n_share + share;
+    const FnLayout L = fn_layout(W, D);
+    const float* net = img + c * img_sz;  // matrices [in][out], everything else as in the flat layout
+    float* gp = part + (size_t)cta * nn;
+    float* mine = scratch + (size_t)cta * fn_scratch_floats(D) + (size_t)tid * kFnCpt;
+    auto slot = [&](int k, int j) { return mine + ((size_t)k * 4 + j) * 256 * kFnCpt; };
+    const float bo = net[L.bo], ys = net[L.ys], yt = net[L.yt];
+    const int64_t n_tiles = (A.n + S - 1) / S;
+    double loss = 0.0;
+    float r_sum = 0.f;
+    bool first = true;
+    for (int64_t tile = share; tile < n_tiles; tile += n_share, first = false) {
+        const int64_t b = tile * S + tid;
+        const bool valid = tid < S && b < A.n;
+        float target = 0.f, weight = 0.f;
+        if (tid < S) {
+            float d[kFnIn] = {0.f, 0.f, 0.f, 0.f};
+            if (valid) {
+                const float4 c0 = A.cfg[2 * b], c1 = A.cfg[2 * b + 1];
+                const FnFrame f = fn_frame(make_float3(c0.x, c0.y, c0.z), c1);
+                const float4 F = A.lab[3 * b], ti = A.lab[3 * b + 1];
+                float t[5] = {F.x * f.xh.x + F.y * f.xh.y, F.x * f.yh.x + F.y * f.yh.y, F.z * f.zh.z,
+                              ti.x * f.xh.x + ti.y * f.xh.y, ti.x * f.yh.x + ti.y * f.yh.y};
+                float t2 = 0.f;
+#pragma unroll
+                for (int k = 0; k < 5; ++k) {
+                    t[k] = A.cap > 0.f ? fminf(fmaxf(t[k], -A.cap), A.cap) : t[k];
+                    t2 = fmaf(t[k], t[k], t2);
+                    target = k == c ? t[k] : target;
+                }
+                weight = A.f_scale > 0.f ? 1.f / (1.f + t2 / (A.f_scale * A.f_scale)) : 1.f;
+#pragma unroll
+                for (int k = 0; k < kFnIn; ++k) d[k] = f.d[k];
+            }
+#pragma unroll
+            for (int k = 0; k < kFnIn; ++k) Xs[k * LD + tid] = (d[k] - net[k]) * net[4 + k];
+        }
         __syncthreads();
+        // ---- forward
+        float2 acc[kFnCpt][2];
+        for (int l = 0; l < D; ++l) {
+            fn_gemm<W>(l == 0 ? Xs : Hs + (size_t)(l - 1) * W * LD, net + L.w(l), l == 0 ? kFnIn : W, p0, o0, acc);
+            TrVec<kFnCpt> e;
+#pragma unroll
+            for (int i = 0; i < kFnCpt; ++i) e.v[i] = 0.f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float bj = net[L.b(l) + o0 + j], w = net[L.wo + o0 + j];
+                TrVec<kFnCpt> h, d1;
+#pragma unroll
+                for (int i = 0; i < kFnCpt; ++i) {
+                    const float z = tr_at<kFnCpt>(acc, i, j) + bj;
+                    const float sg = 1.f / (1.f + __expf(-z));
+                    h.v[i] = z * sg;
+                    d1.v[i] = sg * (1.f + z * (1.f - sg));
+                    e.v[i] = fmaf(w, h.v[i], e.v[i]);
+                }
+                tr_st<kFnCpt>(slot(l, j), d1);
+                if (l < D - 1)
+                    tr_st<kFnCpt>(Hs + (size_t)l * W * LD + (size_t)(o0 + j) * LD + p0, h);
+                else
+                    tr_st<kFnCpt>(slot(D, j), h);
+            }
+            if (l == D - 1) tr_st<kFnCpt>(Red + (size_t)to * S + p0, e);
+            __syncthreads();
+        }
+        // ---- residual r = 2 w (y - t) / n, scaled by y_scale
+        if (tid < S) {
+            float y = bo;
+            for (int g = 0; g < NG; ++g) y += Red[(size_t)g * S + tid];
+            const float dv = fmaf(ys, y, yt) - target;
+            const float r = valid ? 2.f * weight * dv / (float)A.n * ys : 0.f;
+            ts[tid] = r;
+            r_sum += r;
+            if (valid) loss += (double)weight * dv * dv;
+        }
+        __syncthreads();
+        // ---- top: the gradient of w_o and the signal r w_o silu'
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const TrVec<kFnCpt> h = tr_ld<kFnCpt>(slot(D, j));
+            TrVec<kFnCpt> d1 = tr_ld<kFnCpt>(slot(D - 1, j));
+            const float w = net[L.wo + o0 + j];
+            float sum = 0.f;
+#pragma unroll
+            for (int i = 0; i < kFnCpt; ++i) {
+                const float r = ts[p0 + i];
+                sum = fmaf(r, h.v[i], sum);
+                d1.v[i] *= r * w;
+            }
+            tr_st<kFnCpt>(G0 + (size_t)(o0 + j) * LD + p0, d1);
+            constexpr int kGroup = NTP < 32 ? NTP : 32;
+#pragma unroll
+            for (int o = 1; o < kGroup; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (tp % kGroup == 0) Wp[(tp / kGroup) * W + o0 + j] = sum;
+        }
+        __syncthreads();
+        if (tid < W) {
+            float a = Wp[tid];
+            if (T::kWarpsPerUnit > 1) a += Wp[W + tid];
+            float* q = gp + L.wo + tid;
+            *q = first ? a : *q + a;
+        }
+        // ---- backward
+        float* g = G0;
+        float* gn = G1;
+        for (int l = D - 1; l >= 0; --l) {
+            for (int o = tid; o < W; o += 256) {
+                float a = 0.f;
+                for (int k = 0; k < S; k += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(g + (size_t)o * LD + k);
+                    a += (v.x + v.y) + (v.z + v.w);
+                }
+                float* q = gp + L.b(l) + o;
+                *q = first ? a : *q + a;
+            }
+            if (l == 0) {
+                for (int t = tid; t < W * kFnIn; t += 256) {
+                    const int o = t / kFnIn, k = t % kFnIn;
+                    float a = 0.f;
+                    for (int s = 0; s < S; ++s) a = fmaf(g[(size_t)o * LD + s], Xs[k * LD + s], a);
+                    float* q = gp + L.w(0) + t;
+                    *q = first ? a : *q + a;
+                }
+                break;
+            }
+            fn_weight_grad<W>(g, Hs + (size_t)(l - 1) * W * LD, gp + L.w(l), first);
+            fn_gemm<W>(g, wr + ((int64_t)c * (D - 1) + l - 1) * W * W, W, p0, o0, acc);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                TrVec<kFnCpt> d1 = tr_ld<kFnCpt>(slot(l - 1, j));
+#pragma unroll
+                for (int i = 0; i < kFnCpt; ++i) d1.v[i] *= tr_at<kFnCpt>(acc, i, j);
+                tr_st<kFnCpt>(gn + (size_t)(o0 + j) * LD + p0, d1);
+            }
+            __syncthreads();
+            float* tmp = g;
+            g = gn;
+            gn = tmp;
+        }
+        __syncthreads();  // the next tile overwrites what this one read
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+    s_loss[tid] = loss;
+    if (tid < S) ts[tid] = r_sum;
+    __syncthreads();
+    if (tid == 0) {
+        double a = 0.0;
+        float r = 0.f;
+        for (int k = 0; k < S; ++k) {
+            a += s_loss[k];
+            r += ts[k];
+        }
+        loss_part[cta] = a;
+        gp[L.bo] = r;
+    }
 }
 
-// G[b][o] = r[b] w_o[o] S[b][o].
-__global__ void k_fn_seed(int64_t n, int W, const float* __restrict__ r, const float* __restrict__ wo,
-                          const float* __restrict__ S, float* __restrict__ G) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= n * W) return;
-    G[t] = r[t / W] * wo[t % W] * S[t];
-}
-
-__global__ void k_fn_mul(int64_t m, float* __restrict__ G, const float* __restrict__ S) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t < m) G[t] *= S[t];
-}
-
-__global__ void k_fn_loss(const double* __restrict__ part, int nb, double inv_n,
-                          double* __restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+// Sum of each network's shares (in order), the loss, Adam when `step`, and the
+// kernel images of the updated parameters.
+struct FnAdam {
+    float *p, *m, *v, *img, *wr;
+    float lr, b1, b2, eps, c1, c2;
+};
+__global__ void __launch_bounds__(256)
+    k_fn_update(int W, int D, int64_t nn, int64_t img_sz, int n_share, const float* __restrict__ part,
+                float* __restrict__ grad, bool step, FnAdam a, const double* __restrict__ loss_part,
+                double inv_n, double* __restrict__ loss_out) {
+    pdl_wait();
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
         double x = 0.0;
-        for (int k = 0; k < nb; ++k) x += part[k];
-        *out = x * inv_n;
+        for (int k = threadIdx.x; k < kFnNets * n_share; k += 32) x += loss_part[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (threadIdx.x == 0) *loss_out = x * inv_n;
     }
+    const int64_t t = blockIdx.x * (int64_t)256 + threadIdx.x;
+    if (t >= kFnNets * nn) return;
+    const int64_t c = t / nn, e = t % nn;
+    const FnLayout L = fn_layout(W, D);
+    const bool train = e >= 8 && e <= L.bo;
+    float g = 0.f;
+    if (train) {
+        const float* q = part + (size_t)c * n_share * nn + e;
+        int k = 0;
+        for (; k + 8 <= n_share; k += 8) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = q[(size_t)(k + u) * nn];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) g += v[u];
+        }
+        for (; k < n_share; ++k) g += q[(size_t)k * nn];
+    }
+    grad[t] = g;
+    if (!step || !train) return;
+    const float p = adam_update(a.p[t], g, a.m[t], a.v[t], a.lr, a.b1, a.b2, a.eps, a.c1, a.c2);
+    a.p[t] = p;
+    // the image's place of entry e: matrices transposed, the rest as it is
+    float* im = a.img + c * img_sz;
+    int64_t at = e;
+    if (e < L.b(0)) {
+        const int64_t r = e - 8;
+        at = 8 + r % kFnIn * W + r / kFnIn;
+    } else if (e >= L.w(1) && e < L.wo) {
+        const int64_t per = (int64_t)W * W + W, r = (e - L.w(1)) % per, l = (e - L.w(1)) / per;
+        if (r < (int64_t)W * W) {
+            at = e - r + r % W * W + r / W;
+            a.wr[(c * (D - 1) + l) * W * W + r] = p;
+        }
+    }
+    im[at] = p;
 }
 
 static inline int nblk(int64_t n, int t = 256) { return (int)std::max<int64_t>(1, (n + t - 1) / t); }
 
-// Gradient of L for a batch of B sampled pairs (cfg: 2 float4, labels: 3
-// float4 per pair, as rb_sample_pairs writes them).  grad: the flat layout
-// (zero for mu, inv_sd, y_scale, y_shift).
-static rb_status fn_train_grad(rb_fnet_trainer* tr, int64_t B, const float4* cfg, const float4* lab,
-                               double* loss_host) {
-    rb_fnet* f = tr->f;
-    const int W = f->width, D = f->depth;
-    const int64_t nn = f->net_floats;
-    const FnLayout Ly = fn_layout(W, D);
-    cudaStream_t st = f->stream;
-    float* X = tr->work;            // B x 4
-    float* T = X + 4 * B;           // B x 5
-    float* Xc = T + 5 * B;          // B x 4
-    float* r = Xc + 4 * B;          // B
-    float* Wb = r + B;              // B sample weights
-    float* H = Wb + B;              // D x B x W
-    float* S = H + (int64_t)D * B * W;
-    float* G0 = S + (int64_t)D * B * W;
-    float* G1 = G0 + B * W;
-    k_fn_inputs<<<nblk(B), 256, 0, st>>>(B, cfg, lab, tr->cap, tr->f_scale, X, T, Wb);
-    RB_CUDA(cudaMemsetAsync(tr->grad, 0, sizeof(float) * kFnNets * f->net_floats, st));
-    const int nbo = nblk(B);
-    for (int c = 0; c < kFnNets; ++c) {
-        const float* net = f->params + c * nn;
-        float* g = tr->grad + c * nn;
-        k_fn_norm<<<nblk(4 * B), 256, 0, st>>>(B, X, net, Xc);
-        // forward
-        const float* Hin = Xc;
-        int in = kFnIn;
-        for (int l = 0; l < D; ++l) {
-            float* Hl = H + (int64_t)l * B * W;
-            float* Sl = S + (int64_t)l * B * W;
-            // Z = Hin W_l^T  (W_l stored [out][in])
-            RB_TRY(sgemm(st, (int)B, W, in, Hin, in, 1, net + Ly.w(l), 1, in, Hl, W, 1.f, 0.f, nullptr));
-            k_fn_act<<<nblk(B * W), 256, 0, st>>>(B, W, net + Ly.b(l), Hl, Hl, Sl);
-            Hin = Hl;
-            in = W;
-        }
-        const float* HD = H + (int64_t)(D - 1) * B * W;
-        k_fn_out<<<nbo, 256, 0, st>>>(B, W, HD, net, Ly.wo, T, Wb, c, r, tr->loss_part + c * nbo);
-        // backward: w_o, b_o
-        RB_TRY(sgemm(st, 1, W, (int)B, r, 0, 1, HD, W, 1, g + Ly.wo, W, 1.f, 0.f, nullptr, tr->sk,
-                     tr->sk_floats));
-        k_colsum<<<1, 256, 0, st>>>((int)B, 1, r, 1, g + Ly.bo, 0);
-        k_fn_seed<<<nblk(B * W), 256, 0, st>>>(B, W, r, net + Ly.wo, S + (int64_t)(D - 1) * B * W, G0);
-        float* Gl = G0;
-        float* Gn = G1;
-        for (int l = D - 1; l >= 0; --l) {
-            const int inl = l == 0 ? kFnIn : W;
-            const float* Hprev = l == 0 ? Xc : H + (int64_t)(l - 1) * B * W;
-            // dW_l[o][k] = sum_b G[b][o] Hprev[b][k]
-            RB_TRY(sgemm(st, W, inl, (int)B, Gl, 1, W, Hprev, inl, 1, g + Ly.w(l), inl, 1.f, 0.f,
-                         nullptr, tr->sk, tr->sk_floats));
-            k_colsum<<<W, 256, 0, st>>>((int)B, W, Gl, W, g + Ly.b(l), 0);
-            if (l > 0) {
-                // G_{l-1} = (G_l W_l) * S_{l-1}
-                RB_TRY(sgemm(st, (int)B, W, W, Gl, W, 1, net + Ly.w(l), W, 1, Gn, W, 1.f, 0.f,
-                             nullptr));
-                k_fn_mul<<<nblk(B * W), 256, 0, st>>>(B * W, Gn, S + (int64_t)(l - 1) * B * W);
-                std::swap(Gl, Gn);
-            }
-        }
+// Shares per network: a CTA per tile, at most two per SM over the five networks.
+static int fn_shares(const rb_fnet_trainer* t, int64_t B) {
+    const int64_t S = 1024 * kFnCpt / t->f->width;
+    return (int)std::max<int64_t>(1, std::min<int64_t>((B + S - 1) / S, 2 * t->sms / kFnNets));
+}
+
+template <int W>
+static rb_status launch_fn_tile(rb_fnet_trainer* t, int shares, const FnTrainArgs& A) {
+    rb_fnet* f = t->f;
+    static std::atomic<bool> allowed{false};
+    if (!allowed.load()) {
+        RB_CUDA(cudaFuncSetAttribute(k_fn_tile<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        allowed.store(true);
     }
-    k_fn_loss<<<1, 32, 0, st>>>(tr->loss_part, kFnNets * nbo, 1.0 / (double)B, tr->loss_out);
-    RB_CUDA(cudaGetLastError());
+    RB_CUDA(launch_pdl(k_fn_tile<W>, dim3(kFnNets, shares), 256, FnTile<W>::smem(f->depth), f->stream, f->img,
+                       f->img_floats, f->wr, f->depth, A, t->part, f->net_floats, t->scratch, t->loss_part));
+    return RB_OK;
+}
+
+// Gradient of L for a batch of B sampled pairs (cfg: 2 float4, labels: 3
+// float4 per pair, as rb_sample_pairs writes them) into t->grad (the flat
+// layout; zero for mu, inv_sd, y_scale, y_shift), and the Adam step.
+static rb_status fn_train(rb_fnet_trainer* t, int64_t B, const float4* cfg, const float4* lab, bool step,
+                          double* loss_host) {
+    rb_fnet* f = t->f;
+    const FnTrainArgs A{B, cfg, lab, t->cap, t->f_scale};
+    const int shares = fn_shares(t, B);
+    switch (f->width) {
+        case 16: RB_TRY(launch_fn_tile<16>(t, shares, A)); break;
+        case 32: RB_TRY(launch_fn_tile<32>(t, shares, A)); break;
+        default: RB_TRY(launch_fn_tile<64>(t, shares, A)); break;
+    }
+    FnAdam a{f->params, t->m, t->v, f->img, f->wr, t->lr, t->beta1, t->beta2, t->eps, 1.f, 1.f};
+    if (step) {
+        ++t->t;
+        // bias corrections in FP64 (1 - beta2^t cancels badly in FP32)
+        a.c1 = (float)(1.0 - std::pow((double)t->beta1, (double)t->t));
+        a.c2 = (float)(1.0 - std::pow((double)t->beta2, (double)t->t));
+    }
+    RB_CUDA(launch_pdl(k_fn_update, nblk(kFnNets * f->net_floats), 256, 0, f->stream, f->width, f->depth,
+                       f->net_floats, f->img_floats, shares, t->part, t->grad, step, a, t->loss_part,
+                       1.0 / (double)B, t->loss_out));
+    if (step) ++f->version;
     if (loss_host) {
-        RB_CUDA(cudaMemcpyAsync(loss_host, tr->loss_out, sizeof(double), cudaMemcpyDeviceToHost, st));
-        RB_CUDA(cudaStreamSynchronize(st));
+        RB_CUDA(cudaMemcpyAsync(loss_host, t->loss_out, sizeof(double), cudaMemcpyDeviceToHost, f->stream));
+        RB_CUDA(cudaStreamSynchronize(f->stream));
     }
     return RB_OK;
 }
 
 static rb_status fn_prepare(rb_fnet* f) {
     k_fn_prepare<<<nblk(kFnNets * f->img_floats), 256, 0, f->stream>>>(f->params, f->width, f->depth,
-                                                                      f->img);
+                                                                      f->img, f->wr);
     RB_CUDA(cudaGetLastError());
     ++f->version;
     return RB_OK;
@@ -558,16 +776,20 @@ rb_status rb_fnet_create(int32_t width, int32_t depth, void* stream, rb_fnet** o
     f->img_floats = fn_img_size(width, depth);
     cudaError_t e = cudaMalloc((void**)&f->params, sizeof(float) * kFnNets * f->net_floats);
     if (e == cudaSuccess) e = cudaMalloc((void**)&f->img, sizeof(float) * kFnNets * f->img_floats);
+    if (e == cudaSuccess)
+        e = cudaMalloc((void**)&f->wr, sizeof(float) * std::max<int64_t>(16, (int64_t)kFnNets * (depth - 1) * width * width));
     if (e == cudaSuccess) e = cudaMemsetAsync(f->params, 0, sizeof(float) * kFnNets * f->net_floats, f->stream);
     if (e != cudaSuccess) {
         cudaFree(f->params);
         cudaFree(f->img);
+        cudaFree(f->wr);
         delete f;
         return cuda_fail(e, "per-component network allocation");
     }
     if (sizeof(float) * f->img_floats > 227 * 1024) {
         cudaFree(f->params);
         cudaFree(f->img);
+        cudaFree(f->wr);
         delete f;
         return fail(RB_ENOTSUP, "one network's weights must fit in shared memory (227 KB)");
     }
@@ -580,6 +802,7 @@ rb_status rb_fnet_destroy(rb_fnet* f) {
     if (f->stream) cudaStreamSynchronize(f->stream);
     cudaFree(f->params);
     cudaFree(f->img);
+    cudaFree(f->wr);
     delete f;
     return RB_OK;
 }
@@ -630,16 +853,15 @@ rb_status rb_fnet_trainer_create(rb_fnet* f, int64_t max_batch, float lr, float 
     t->beta1 = beta1;
     t->beta2 = beta2;
     t->eps = eps;
-    const int64_t np = kFnNets * f->net_floats, B = max_batch, W = f->width, D = f->depth;
-    t->loss_blocks = kFnNets * nblk(B);
-    const size_t work = (size_t)(15 * B + 2 * D * B * W + 2 * B * W);  // X, T, Xc, r, w; H, S; G x 2
+    const int64_t np = kFnNets * f->net_floats;
+    cudaDeviceGetAttribute(&t->sms, cudaDevAttrMultiProcessorCount, f->device);
+    const size_t ctas = (size_t)kFnNets * fn_shares(t, max_batch);
     cudaError_t e = cudaMalloc((void**)&t->m, sizeof(float) * np);
     if (e == cudaSuccess) e = cudaMalloc((void**)&t->v, sizeof(float) * np);
     if (e == cudaSuccess) e = cudaMalloc((void**)&t->grad, sizeof(float) * np);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&t->work, sizeof(float) * work);
-    t->sk_floats = (size_t)kSplitMax * W * std::max<int64_t>(W, kFnIn);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&t->sk, sizeof(float) * t->sk_floats);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&t->loss_part, sizeof(double) * t->loss_blocks);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&t->part, sizeof(float) * f->net_floats * ctas);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&t->scratch, sizeof(float) * fn_scratch_floats(f->depth) * ctas);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&t->loss_part, sizeof(double) * ctas);
     if (e == cudaSuccess) e = cudaMalloc((void**)&t->loss_out, sizeof(double));
     if (e == cudaSuccess) e = cudaMemsetAsync(t->m, 0, sizeof(float) * np, f->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(t->v, 0, sizeof(float) * np, f->stream);
@@ -647,8 +869,8 @@ rb_status rb_fnet_trainer_create(rb_fnet* f, int64_t max_batch, float lr, float 
         cudaFree(t->m);
         cudaFree(t->v);
         cudaFree(t->grad);
-        cudaFree(t->work);
-        cudaFree(t->sk);
+        cudaFree(t->part);
+        cudaFree(t->scratch);
         cudaFree(t->loss_part);
         cudaFree(t->loss_out);
         delete t;
@@ -664,8 +886,8 @@ rb_status rb_fnet_trainer_destroy(rb_fnet_trainer* t) {
     cudaFree(t->m);
     cudaFree(t->v);
     cudaFree(t->grad);
-    cudaFree(t->work);
-    cudaFree(t->sk);
+    cudaFree(t->part);
+    cudaFree(t->scratch);
     cudaFree(t->loss_part);
     cudaFree(t->loss_out);
     delete t;
@@ -677,13 +899,8 @@ rb_status rb_fnet_train_grad(rb_fnet_trainer* t, int64_t batch, const float* cfg
     if (!t) return fail(RB_EINVAL, "null trainer");
     if (batch < 1 || batch > t->max_batch || !cfg || !labels)
         return fail(RB_EINVAL, "batch must be in [1, max_batch] with cfg and labels");
-    RB_TRY(fn_train_grad(t, batch, reinterpret_cast<const float4*>(cfg),
-                         reinterpret_cast<const float4*>(labels), loss_host));
-    if (loss_host) {  // the loss read is a synchronisation point: report a timed-out GEMM
-        bool bad = false;
-        RB_TRY(gemm_status_take(t->f->stream, &bad));
-        if (bad) return fail(RB_EFAULT, "tensor-core GEMM timed out waiting for an MMA");
-    }
+    RB_TRY(fn_train(t, batch, reinterpret_cast<const float4*>(cfg), reinterpret_cast<const float4*>(labels), false,
+                    loss_host));
     if (grad_out)
         RB_CUDA(cudaMemcpyAsync(grad_out, t->grad, sizeof(float) * kFnNets * t->f->net_floats,
                                 cudaMemcpyDeviceToDevice, t->f->stream));
@@ -692,17 +909,11 @@ rb_status rb_fnet_train_grad(rb_fnet_trainer* t, int64_t batch, const float* cfg
 
 rb_status rb_fnet_train_step(rb_fnet_trainer* t, int64_t batch, const float* cfg, const float* labels,
                              double* loss_host) {
-    RB_TRY(rb_fnet_train_grad(t, batch, cfg, labels, nullptr, loss_host));
-    rb_fnet* f = t->f;
-    const int64_t np = kFnNets * f->net_floats;
-    ++t->t;
-    // bias corrections in FP64 (1 - beta2^t cancels badly in FP32)
-    const float c1 = (float)(1.0 - std::pow((double)t->beta1, (double)t->t));
-    const float c2 = (float)(1.0 - std::pow((double)t->beta2, (double)t->t));
-    k_adam<<<nblk(np), 256, 0, f->stream>>>(np, 0, np, f->params, t->grad, t->m, t->v, t->lr, t->beta1,
-                                            t->beta2, t->eps, c1, c2);
-    RB_CUDA(cudaGetLastError());
-    return fn_prepare(f);
+    if (!t) return fail(RB_EINVAL, "null trainer");
+    if (batch < 1 || batch > t->max_batch || !cfg || !labels)
+        return fail(RB_EINVAL, "batch must be in [1, max_batch] with cfg and labels");
+    return fn_train(t, batch, reinterpret_cast<const float4*>(cfg), reinterpret_cast<const float4*>(labels), true,
+                    loss_host);
 }
 
 rb_status rb_fnet_trainer_set_lr(rb_fnet_trainer* t, float lr) {

@@ -1,6 +1,6 @@
 // FP32 network pieces shared by the SIMT inference kernel (nn.cu) and the
-// training kernel (train.cu): the prepared weight copies and the cp.async ring
-// that streams them through shared memory.
+// training kernels (train.cu, fnet.cu): the prepared weight copies, the cp.async
+// ring that streams them through shared memory, register tiles and Adam.
 #pragma once
 
 #include "nn_common.cuh"
@@ -87,5 +87,45 @@ struct ChunkFeed {
     }
     __device__ void release() { ++c; }
 };
+
+// ---- pieces of the training kernels (train.cu, fnet.cu)
+// CPT consecutive samples of one unit.
+template <int CPT>
+struct TrVec {
+    float v[CPT];
+};
+template <int CPT>
+__device__ __forceinline__ TrVec<CPT> tr_ld(const float* p) {
+    TrVec<CPT> r;
+    if constexpr (CPT == 4) {
+        const float4 a = *reinterpret_cast<const float4*>(p);
+        r.v[0] = a.x, r.v[1] = a.y, r.v[2] = a.z, r.v[3] = a.w;
+    } else {
+        const float2 a = *reinterpret_cast<const float2*>(p);
+        r.v[0] = a.x, r.v[1] = a.y;
+    }
+    return r;
+}
+template <int CPT>
+__device__ __forceinline__ void tr_st(float* p, const TrVec<CPT>& r) {
+    if constexpr (CPT == 4)
+        *reinterpret_cast<float4*>(p) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
+    else
+        *reinterpret_cast<float2*>(p) = make_float2(r.v[0], r.v[1]);
+}
+
+template <int CPT>
+__device__ __forceinline__ float tr_at(const float2 (&acc)[CPT][2], int i, int j) {
+    const float2 v = acc[i][j >> 1];
+    return (j & 1) ? v.y : v.x;
+}
+
+// One Adam step of a parameter; m and v in place.
+__device__ __forceinline__ float adam_update(float p, float g, float& m, float& v, float lr, float b1, float b2,
+                                             float eps, float c1, float c2) {
+    m = b1 * m + (1.f - b1) * g;
+    v = b2 * v + (1.f - b2) * g * g;
+    return p - lr * (m / c1) / (sqrtf(v / c2) + eps);
+}
 
 }  // namespace rb

@@ -326,13 +326,7 @@ rb_status fnet_pairs_system_async(rb_system* s, const rb_fnet* f);
 rb_status check_fnet(const rb_fnet* f);
 uint64_t fnet_version(const rb_fnet* f);  // bumped whenever its parameters change
 rb_status fnet_ready(const rb_fnet* f);    // waits (outside any capture) for a change to land
-// train.cu: fixed-order GEMM C = beta C + alpha A B with strided operands
-// (A(m, k) = A[m sam + k sak], B(k, n) = B[k sbk + n sbn], C row-major), the
-// fixed-order column sum and Adam, shared with the per-component trainer
 constexpr int kSplitMax = 32;  // most split-K parts of one sgemm (ws: kSplitMax x M x N floats)
-// ws (nullable, ws_floats floats): room for split-K partial tiles; with it a
-// long reduction (K >= 512) onto a small C is split along K over more CTAs and
-// summed in a fixed order.
 // gemm_tc.cu: FP32-accurate GEMM (split TF32 on the tensor cores), C = alpha A B + beta C
 // with A(m, k) = A[m sam + k sak], B(k, n) = B[k sbk + n sbn]; a timed-out MMA wait
 // sets ST_TC_TIMEOUT in *status (or in the module's own word, read by gemm_status_take).
@@ -341,11 +335,6 @@ rb_status sgemm(cudaStream_t st, int M, int N, int K, const float* A, int64_t sa
                 const float* B, int64_t sbk, int64_t sbn, float* C, int64_t ldc, float alpha,
                 float beta, unsigned* status, float* ws = nullptr, size_t ws_floats = 0);
 rb_status gemm_status_take(cudaStream_t st, bool* timed_out);  // synchronises st
-__global__ void k_colsum(int M, int N, const float* __restrict__ A, int64_t lda,
-                         float* __restrict__ out, int accumulate);
-__global__ void k_adam(int64_t n, int64_t lo, int64_t hi, float* __restrict__ p,
-                       const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-                       float lr, float b1, float b2, float eps, float c1, float c2);
 rb_status check_mlp(const rb_mlp* m);
 
 // ---------------------------------------------------------------- batched step

@@ -292,30 +292,6 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// out[n] = accumulate * out[n] + sum_m A[m][n] (fixed-order tree per column).
-__global__ void k_colsum(int M, int N, const float* __restrict__ A, int64_t lda,
-                         float* __restrict__ out, int accumulate) {
-    __shared__ float sh[256];
-    const int n = blockIdx.x;
-    float x = 0.f;
-    for (int m = threadIdx.x; m < M; m += 256) x += A[m * lda + n];
-    sh[threadIdx.x] = x;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[n] = (accumulate ? out[n] : 0.f) + sh[0];
-}
-
-// One Adam step of a parameter; m and v in place.
-__device__ __forceinline__ float adam_update(float p, float g, float& m, float& v, float lr, float b1, float b2,
-                                             float eps, float c1, float c2) {
-    m = b1 * m + (1.f - b1) * g;
-    v = b2 * v + (1.f - b2) * g * g;
-    return p - lr * (m / c1) / (sqrtf(v / c2) + eps);
-}
-
 // ------------------------------------------------------------- weight gradient
 // One CTA computes a tile of S = 1024 CPT / W samples from the configurations
 // to its share of every parameter's gradient; k_train_update sums the shares
@@ -451,30 +427,6 @@ __device__ inline void tr_tangent(const TrArgs& A, const PairGeom& g, const floa
     }
 }
 
-template <int CPT>
-struct TrVec {
-    float v[CPT];
-};
-template <int CPT>
-__device__ __forceinline__ TrVec<CPT> tr_ld(const float* p) {
-    TrVec<CPT> r;
-    if constexpr (CPT == 4) {
-        const float4 a = *reinterpret_cast<const float4*>(p);
-        r.v[0] = a.x, r.v[1] = a.y, r.v[2] = a.z, r.v[3] = a.w;
-    } else {
-        const float2 a = *reinterpret_cast<const float2*>(p);
-        r.v[0] = a.x, r.v[1] = a.y;
-    }
-    return r;
-}
-template <int CPT>
-__device__ __forceinline__ void tr_st(float* p, const TrVec<CPT>& r) {
-    if constexpr (CPT == 4)
-        *reinterpret_cast<float4*>(p) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
-    else
-        *reinterpret_cast<float2*>(p) = make_float2(r.v[0], r.v[1]);
-}
-
 // acc[i][j / 2].(x, y) = sum_k A[k][p0 + i] B[k][o0 + j]: A in shared memory
 // [K][LD], B the next K / KC weight chunks.
 template <int W, int CPT, int KC>
@@ -501,12 +453,6 @@ __device__ __forceinline__ void tr_gemm(const float* __restrict__ As, int K, Chu
         feed.release();
     }
 }
-template <int CPT>
-__device__ __forceinline__ float tr_at(const float2 (&acc)[CPT][2], int i, int j) {
-    const float2 v = acc[i][j >> 1];
-    return (j & 1) ? v.y : v.x;
-}
-
 // out[o * W + i] (+)= sum_c A1[o][c] B1[i][c] + A2[o][c] B2[i][c] over the
 // tile's samples: a warp per 8 units o, lanes on consecutive i; FP32x2 over
 // pairs of samples.
@@ -891,14 +837,6 @@ __global__ void __launch_bounds__(256)
             a.prep[L.wr + (int64_t)l * W * W + e] = p;
         }
     }
-}
-
-__global__ void k_adam(int64_t n, int64_t lo, int64_t hi, float* __restrict__ p,
-                       const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-                       float lr, float b1, float b2, float eps, float c1, float c2) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= n || t < lo || t >= hi) return;
-    p[t] = adam_update(p[t], g[t], m[t], v[t], lr, b1, b2, eps, c1, c2);
 }
 
 static inline unsigned nblk(int64_t n, int t) { return (unsigned)std::max<int64_t>(1, (n + t - 1) / t); }

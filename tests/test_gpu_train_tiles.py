@@ -1,14 +1,15 @@
-"""The fused training gradient against the FP64 oracle at the edges of its tiles: batches of one
+"""The fused training gradients against the FP64 oracle at the edges of their tiles: batches of one
 sample, one below, at and above a tile, and beyond one tile per CTA; every width, depths 1 to 4 (both
-tile forms).  The bound is the
+tile forms of the energy network), the per-component networks' widths and depths.  The bound is the
 one of the FP32 gradients elsewhere in these tests, 1e-5 of the gradient's norm: sums of up to 10^4
 FP32 terms in fixed partial sums of at most 64 samples lose a few 2^-24 each."""
 import numpy as np
 import pytest
 
-from oracle import nn
+from oracle import fnet, nn
 from paper_2402_12199_gb300 import inputs
 from tests.helpers import rel_err
+from tests.test_gpu_fnet import _flat, _sampled
 
 pytestmark = pytest.mark.gpu
 
@@ -56,3 +57,42 @@ def test_energy_network_gradient(width, depth, batch):
     fresh.set_params(w)
     assert torch.equal(m.pairs(cfg, "fp32"), fresh.pairs(cfg, "fp32"))
     assert torch.equal(tr.grad(cfg, labels, 0.5, 0.1)[1], api.Trainer(fresh, batch).grad(cfg, labels, 0.5, 0.1)[1])
+
+
+@pytest.mark.parametrize("width,depth,batch", [
+    (16, 1, 1), (16, 3, 255), (16, 2, 257), (32, 1, 127), (32, 3, 129), (32, 8, 300), (64, 2, 63), (64, 3, 65),
+    (64, 8, 200), (32, 3, 9000),
+])
+def test_per_component_gradient(width, depth, batch):
+    import torch
+
+    from paper_2402_12199_gb300 import api
+
+    flat = _flat(width, depth, 7 * width + depth)
+    f = api.FNet(width, depth)
+    f.set_params(flat)
+    cfg, lab = _sampled(batch + 300, 42)
+    cfg, lab = cfg[:batch].contiguous(), lab[:batch].contiguous()
+    assert len(cfg) == batch
+    tr = api.FNetTrainer(f, batch)
+    tr.set_cap(5.0, 1.5)
+    loss, g = tr.grad(cfg, lab)
+    c, lb = cfg.double().cpu().numpy(), lab.double().cpu().numpy()
+    d, t = fnet.targets(c[:, :3], c[:, 4:8], lb[:, 0:3], lb[:, 4:7], cap=5.0)
+    L_ref, g_ref = fnet.loss_and_grad(flat.astype(np.float64), width, depth, d, t, f_scale=1.5)
+    assert loss == pytest.approx(L_ref, rel=1e-5)
+    assert rel_err(g.double().cpu().numpy(), g_ref) < 1e-5
+    tr.step(cfg, lab)
+    w = f.get_params()
+    fresh = api.FNet(width, depth)
+    fresh.set_params(w)
+    assert torch.equal(f.pairs(cfg), fresh.pairs(cfg))
+    assert torch.equal(tr.grad(cfg, lab)[1], _grad(fresh, batch, cfg, lab))
+
+
+def _grad(f, batch, cfg, lab):
+    from paper_2402_12199_gb300 import api
+
+    tr = api.FNetTrainer(f, batch)
+    tr.set_cap(5.0, 1.5)
+    return tr.grad(cfg, lab)[1]
