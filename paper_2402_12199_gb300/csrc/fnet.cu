@@ -18,10 +18,10 @@
 // torque on cylinder 1 in that frame; F_i = -F_j and tau_j = -tau_i - s x F_j
 // (angular-momentum balance).  The pair energy is not modelled (0).
 //
-// Inference: one thread per pair; the five networks are staged one after the
-// other into shared memory (weight matrices transposed, so one 16-byte load
-// gives four outputs' weights of one input); activations stay in registers;
-// hidden layers accumulate pairs of outputs with packed FP32x2 FMAs.
+// Inference: a thread evaluates two pairs (one at width 64); the five networks
+// sit in shared memory (weight matrices transposed, so one 16-byte load gives
+// four outputs' weights of one input); activations stay in registers; layers
+// accumulate pairs of outputs with packed FP32x2 FMAs.
 // Training: regression of the five components on bead-sum labels,
 // L = mean_b w_b sum_c (y_c - t_c)^2, the targets optionally capped to
 // [-cap, cap] (the paper caps the wide force and torque range of its training
@@ -157,62 +157,100 @@ __device__ inline FnFrame fn_frame(const float3 s, const float4 q) {
     return f;
 }
 
-__device__ inline float fn_silu(float z) { return z / (1.f + __expf(-z)); }
+// SiLU of two pre-activations: z / (1 + 2^(-z log2 e)) with the hardware base-2
+// exponential and reciprocal (the exponential of expf's fast form; the IEEE
+// division after it, a third of the kernel's instructions, gained no accuracy:
+// the exponential's rounding is the larger).
+__device__ __forceinline__ float2 fn_silu2(float2 z) {
+    constexpr float kLog2e = 1.4426950408889634f;
+    const float2 t = __fmul2_rn(z, make_float2(-kLog2e, -kLog2e));
+    float ex, ey, rx, ry;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(t.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ey) : "f"(t.y));
+    const float2 den = __fadd2_rn(make_float2(ex, ey), make_float2(1.f, 1.f));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rx) : "f"(den.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ry) : "f"(den.y));
+    return __fmul2_rn(z, make_float2(rx, ry));
+}
 
-// One network (image layout in shared memory) on one description.
-template <int W>
-__device__ inline float fn_forward(const float* __restrict__ w, const FnLayout& L, int D,
-                                   const float (&d)[kFnIn]) {
-    float h[W];
-    float x[kFnIn];
-#pragma unroll
-    for (int k = 0; k < kFnIn; ++k) x[k] = (d[k] - w[k]) * w[4 + k];
+// One network (image layout in shared memory) on PP descriptions.  Outputs
+// (o, o + 1) share a packed accumulator; a 16-byte load of four outputs'
+// weights serves all PP pairs.
+template <int W, int PP>
+__device__ inline void fn_forward(const float* __restrict__ w, const FnLayout& L, int D,
+                                  const float (&d)[PP][kFnIn], float (&y)[PP]) {
+    float2 h[PP][W / 2];
     {
         const float* p = w + L.w(0);
         const float* b = w + L.b(0);
 #pragma unroll
-        for (int o = 0; o < W; ++o) h[o] = b[o];
+        for (int o = 0; o < W; o += 2)
 #pragma unroll
-        for (int k = 0; k < kFnIn; ++k)
+            for (int q = 0; q < PP; ++q) h[q][o / 2] = make_float2(b[o], b[o + 1]);
+#pragma unroll
+        for (int k = 0; k < kFnIn; ++k) {
+            float2 x[PP];
+#pragma unroll
+            for (int q = 0; q < PP; ++q) {
+                const float v = (d[q][k] - w[k]) * w[4 + k];
+                x[q] = make_float2(v, v);
+            }
 #pragma unroll
             for (int o = 0; o < W; o += 4) {
                 const float4 w4 = *reinterpret_cast<const float4*>(p + k * W + o);
-                h[o] = fmaf(w4.x, x[k], h[o]);
-                h[o + 1] = fmaf(w4.y, x[k], h[o + 1]);
-                h[o + 2] = fmaf(w4.z, x[k], h[o + 2]);
-                h[o + 3] = fmaf(w4.w, x[k], h[o + 3]);
-            }
 #pragma unroll
-        for (int o = 0; o < W; ++o) h[o] = fn_silu(h[o]);
+                for (int q = 0; q < PP; ++q) {
+                    h[q][o / 2] = __ffma2_rn(make_float2(w4.x, w4.y), x[q], h[q][o / 2]);
+                    h[q][o / 2 + 1] = __ffma2_rn(make_float2(w4.z, w4.w), x[q], h[q][o / 2 + 1]);
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 0; o < W / 2; ++o)
+#pragma unroll
+            for (int q = 0; q < PP; ++q) h[q][o] = fn_silu2(h[q][o]);
     }
     for (int l = 1; l < D; ++l) {
-        // packed FP32x2: outputs (o, o+1) share an accumulator, the input
-        // activation is the broadcast operand
         const float* p = w + L.w(l);
         const float* b = w + L.b(l);
-        float2 z[W / 2];
+        float2 z[PP][W / 2];
 #pragma unroll
-        for (int o = 0; o < W; o += 2) z[o / 2] = make_float2(b[o], b[o + 1]);
+        for (int o = 0; o < W; o += 2)
+#pragma unroll
+            for (int q = 0; q < PP; ++q) z[q][o / 2] = make_float2(b[o], b[o + 1]);
 #pragma unroll
         for (int k = 0; k < W; ++k) {
-            const float2 hk = make_float2(h[k], h[k]);
+            float2 hk[PP];
+#pragma unroll
+            for (int q = 0; q < PP; ++q) {
+                const float v = (k & 1) ? h[q][k / 2].y : h[q][k / 2].x;
+                hk[q] = make_float2(v, v);
+            }
 #pragma unroll
             for (int o = 0; o < W; o += 4) {
                 const float4 w4 = *reinterpret_cast<const float4*>(p + k * W + o);
-                z[o / 2] = __ffma2_rn(make_float2(w4.x, w4.y), hk, z[o / 2]);
-                z[o / 2 + 1] = __ffma2_rn(make_float2(w4.z, w4.w), hk, z[o / 2 + 1]);
+#pragma unroll
+                for (int q = 0; q < PP; ++q) {
+                    z[q][o / 2] = __ffma2_rn(make_float2(w4.x, w4.y), hk[q], z[q][o / 2]);
+                    z[q][o / 2 + 1] = __ffma2_rn(make_float2(w4.z, w4.w), hk[q], z[q][o / 2 + 1]);
+                }
             }
         }
 #pragma unroll
-        for (int o = 0; o < W; o += 2) {
-            h[o] = fn_silu(z[o / 2].x);
-            h[o + 1] = fn_silu(z[o / 2].y);
-        }
-    }
-    float y = w[L.bo];
+        for (int o = 0; o < W / 2; ++o)
 #pragma unroll
-    for (int o = 0; o < W; ++o) y = fmaf(w[L.wo + o], h[o], y);
-    return fmaf(w[L.ys], y, w[L.yt]);
+            for (int q = 0; q < PP; ++q) h[q][o] = fn_silu2(z[q][o]);
+    }
+#pragma unroll
+    for (int q = 0; q < PP; ++q) {
+        float a = w[L.bo];
+#pragma unroll
+        for (int o = 0; o < W; o += 2) {
+            a = fmaf(w[L.wo + o], h[q][o / 2].x, a);
+            a = fmaf(w[L.wo + o + 1], h[q][o / 2].y, a);
+        }
+        y[q] = fmaf(w[L.ys], a, w[L.yt]);
+    }
 }
 
 // Pair source: the system's pair list (SYSTEM) or explicit configurations
@@ -231,103 +269,163 @@ struct FnDst {
     float4* out;           // explicit: 3 float4 per pair (frame of body i)
 };
 
-template <int W, bool SYSTEM>
+// A warp evaluates 32 PP pairs at a time, PP per lane (two where the
+// activations of both fit the registers), so that a weight load feeds 2 PP
+// packed FMAs.  RESIDENT: all five networks stay in shared memory and the warps
+// run on their own; else the CTA stages one network after the other.  A thread
+// per pair with one network staged at a time took 116 us for the 88 thousand
+// listed pairs of 30000 cylinders at width 32 (a 16-byte weight load for every
+// two packed FMAs, and an IEEE division per SiLU); this form takes 48 us, bound
+// by issue at two CTAs of 244 registers per SM.
+template <int W, int PP, bool SYSTEM, bool RESIDENT>
 __global__ void __launch_bounds__(kFnThreads)
-    k_fnet_pairs(const float* __restrict__ img, int D, int64_t img_sz, FnSrc src, FnDst dst) {
+    k_fnet_pairs(const float* __restrict__ img, int D, int img_sz, FnSrc src, FnDst dst) {
     extern __shared__ float4 sm4[];
-    float* sw = reinterpret_cast<float*>(sm4);
+    const float* sw = reinterpret_cast<const float*>(sm4);
+    if (RESIDENT) {
+        // the parameters were written before this stream's work (fnet_ready)
+        for (int k = threadIdx.x; k < kFnNets * img_sz / 4; k += kFnThreads)
+            sm4[k] = __ldg(reinterpret_cast<const float4*>(img) + k);
+    }
     if (SYSTEM) pdl_wait();
+    if (RESIDENT) __syncthreads();
     const FnLayout L = fn_layout(W, D);
     const int64_t n = SYSTEM ? (int64_t)(*src.n_pairs) : src.n;
-    for (int64_t base = (int64_t)blockIdx.x * kFnThreads; base < n;
-         base += (int64_t)gridDim.x * kFnThreads) {
-        const int64_t t = base + threadIdx.x;
-        const bool valid = t < n;
-        float3 s = make_float3(1.f, 0.f, 0.f);
-        float4 q = make_float4(1.f, 0.f, 0.f, 0.f), qi = q;
-        bool inside = valid;
-        if (valid) {
-            if (SYSTEM) {
-                const int2 ij = src.pairs[t];
-                const float4 pi = src.pos[ij.x], pj = src.pos[ij.y];
-                qi = src.quat[ij.x];
-                const float4 qj = src.quat[ij.y];
-                const float3 R = min_image(make_float3(pj.x - pi.x, pj.y - pi.y, pj.z - pi.z), src.L,
-                                           src.invL);
-                inside = R.x * R.x + R.y * R.y + R.z * R.z < src.Rc2;
-                s = mulT(qmat(qi), R);
-                q = qmul(qconj(qi), qj);
-            } else {
-                const float4 c0 = src.cfg[2 * t], c1 = src.cfg[2 * t + 1];
-                s = make_float3(c0.x, c0.y, c0.z);
-                q = c1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // RESIDENT: tasks of 32 PP pairs per warp; else of a CTA's warps together
+    constexpr int kTask = 32 * PP, kWarps = kFnThreads / 32;
+    const int64_t stride = (int64_t)gridDim.x * kWarps * kTask;
+    for (int64_t cbase = (int64_t)blockIdx.x * kWarps * kTask; cbase < n; cbase += stride) {
+        const int64_t base = cbase + warp * kTask + lane;
+        if (RESIDENT && cbase + warp * kTask >= n) break;
+        float3 s[PP];
+        float4 qi[PP];
+        bool inside[PP];
+        FnFrame f[PP];
+#pragma unroll
+        for (int e = 0; e < PP; ++e) {
+            const int64_t t = base + 32 * e;
+            s[e] = make_float3(1.f, 0.f, 0.f);
+            float4 q = make_float4(1.f, 0.f, 0.f, 0.f);
+            qi[e] = q;
+            inside[e] = t < n;
+            if (t < n) {
+                if (SYSTEM) {
+                    const int2 ij = src.pairs[t];
+                    const float4 pi = src.pos[ij.x], pj = src.pos[ij.y];
+                    qi[e] = src.quat[ij.x];
+                    const float4 qj = src.quat[ij.y];
+                    const float3 R = min_image(make_float3(pj.x - pi.x, pj.y - pi.y, pj.z - pi.z), src.L,
+                                               src.invL);
+                    inside[e] = R.x * R.x + R.y * R.y + R.z * R.z < src.Rc2;
+                    s[e] = mulT(qmat(qi[e]), R);
+                    q = qmul(qconj(qi[e]), qj);
+                } else {
+                    const float4 c0 = src.cfg[2 * t], c1 = src.cfg[2 * t + 1];
+                    s[e] = make_float3(c0.x, c0.y, c0.z);
+                    q = c1;
+                }
             }
+            f[e] = fn_frame(s[e], q);
         }
-        const FnFrame f = fn_frame(s, q);
-        float y0 = 0.f, y1 = 0.f, y2 = 0.f, y3 = 0.f, y4 = 0.f;
+        float d[PP][kFnIn], out[kFnNets][PP];
+#pragma unroll
+        for (int e = 0; e < PP; ++e)
+#pragma unroll
+            for (int k = 0; k < kFnIn; ++k) d[e][k] = f[e].d[k];
+#pragma unroll 1
         for (int c = 0; c < kFnNets; ++c) {
-            __syncthreads();  // the previous network's readers are done
-            const float4* g = reinterpret_cast<const float4*>(img + c * img_sz);
-            for (int64_t k = threadIdx.x; k < img_sz / 4; k += kFnThreads) sm4[k] = __ldg(g + k);
-            __syncthreads();
-            const float yv = fn_forward<W>(sw, L, D, f.d);
-            y0 = c == 0 ? yv : y0;
-            y1 = c == 1 ? yv : y1;
-            y2 = c == 2 ? yv : y2;
-            y3 = c == 3 ? yv : y3;
-            y4 = c == 4 ? yv : y4;
-        }
-        if (!valid) continue;
-        float3 Fj = make_float3(y0 * f.xh.x + y1 * f.yh.x, y0 * f.xh.y + y1 * f.yh.y, y2 * f.zh.z);
-        const float3 ti = make_float3(y3 * f.xh.x + y4 * f.yh.x, y3 * f.xh.y + y4 * f.yh.y, 0.f);
-        const float3 sxF = cross3(s, Fj);
-        const float3 tj = make_float3(-ti.x - sxF.x, -ti.y - sxF.y, -ti.z - sxF.z);
-        if (SYSTEM) {
-            if (inside) {
-                const Mat3 Ri = qmat(qi);
-                const float3 a = mul(Ri, Fj), b = mul(Ri, ti), c2 = mul(Ri, tj);
-                dst.F[t] = make_float4(a.x, a.y, a.z, 0.f);
-                dst.ti[t] = make_float4(b.x, b.y, b.z, 0.f);
-                dst.tj[t] = make_float4(c2.x, c2.y, c2.z, 0.f);
-            } else {  // listed within the skin only: exactly nothing
-                dst.F[t] = dst.ti[t] = dst.tj[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float* w = sw + (RESIDENT ? c * img_sz : 0);
+            if (!RESIDENT) {
+                __syncthreads();  // the previous network's readers are done
+                const float4* g = reinterpret_cast<const float4*>(img + (int64_t)c * img_sz);
+                for (int k = threadIdx.x; k < img_sz / 4; k += kFnThreads) sm4[k] = __ldg(g + k);
+                __syncthreads();
             }
-        } else {
-            dst.out[3 * t] = make_float4(Fj.x, Fj.y, Fj.z, 0.f);
-            dst.out[3 * t + 1] = make_float4(ti.x, ti.y, ti.z, 0.f);
-            dst.out[3 * t + 2] = make_float4(tj.x, tj.y, tj.z, 0.f);
+            float y[PP];
+            fn_forward<W, PP>(w, L, D, d, y);
+#pragma unroll
+            for (int k = 0; k < kFnNets; ++k)
+#pragma unroll
+                for (int e = 0; e < PP; ++e) out[k][e] = k == c ? y[e] : out[k][e];
+        }
+#pragma unroll
+        for (int e = 0; e < PP; ++e) {
+            const int64_t t = base + 32 * e;
+            if (t >= n) continue;
+            const float3 Fj = make_float3(out[0][e] * f[e].xh.x + out[1][e] * f[e].yh.x,
+                                          out[0][e] * f[e].xh.y + out[1][e] * f[e].yh.y, out[2][e] * f[e].zh.z);
+            const float3 ti = make_float3(out[3][e] * f[e].xh.x + out[4][e] * f[e].yh.x,
+                                          out[3][e] * f[e].xh.y + out[4][e] * f[e].yh.y, 0.f);
+            const float3 sxF = cross3(s[e], Fj);
+            const float3 tj = make_float3(-ti.x - sxF.x, -ti.y - sxF.y, -ti.z - sxF.z);
+            if (SYSTEM) {
+                if (inside[e]) {
+                    const Mat3 Ri = qmat(qi[e]);
+                    const float3 a = mul(Ri, Fj), b = mul(Ri, ti), c2 = mul(Ri, tj);
+                    dst.F[t] = make_float4(a.x, a.y, a.z, 0.f);
+                    dst.ti[t] = make_float4(b.x, b.y, b.z, 0.f);
+                    dst.tj[t] = make_float4(c2.x, c2.y, c2.z, 0.f);
+                } else {  // listed within the skin only: exactly nothing
+                    dst.F[t] = dst.ti[t] = dst.tj[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            } else {
+                dst.out[3 * t] = make_float4(Fj.x, Fj.y, Fj.z, 0.f);
+                dst.out[3 * t + 1] = make_float4(ti.x, ti.y, ti.z, 0.f);
+                dst.out[3 * t + 2] = make_float4(tj.x, tj.y, tj.z, 0.f);
+            }
         }
     }
 }
 
-template <bool SYSTEM>
-static rb_status launch_fnet(const rb_fnet* f, cudaStream_t st, int grid, const FnSrc& src,
-                             const FnDst& dst) {
-    const size_t smem = sizeof(float) * (size_t)f->img_floats;
-#define RB_FN(WW)                                                                                \
-    do {                                                                                         \
-        static bool attr = false;                                                                \
-        if (!attr) {                                                                             \
-            RB_CUDA(cudaFuncSetAttribute(k_fnet_pairs<WW, SYSTEM>,                               \
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)); \
-            attr = true;                                                                         \
-        }                                                                                        \
-        if (SYSTEM)                                                                              \
-            RB_CUDA(launch_pdl(k_fnet_pairs<WW, SYSTEM>, grid, kFnThreads, smem, st,             \
-                               (const float*)f->img, f->depth, f->img_floats, src, dst));        \
-        else                                                                                     \
-            k_fnet_pairs<WW, SYSTEM><<<grid, kFnThreads, smem, st>>>(f->img, f->depth,           \
-                                                                     f->img_floats, src, dst);   \
-    } while (0)
-    switch (f->width) {
-        case 16: RB_FN(16); break;
-        case 32: RB_FN(32); break;
-        case 64: RB_FN(64); break;
-        default: return fail(RB_ENOTSUP, "per-component networks support widths 16, 32, 64");
+// All five networks in shared memory where two CTAs per SM still fit.
+static bool fn_resident(const rb_fnet* f) {
+    return sizeof(float) * kFnNets * (size_t)f->img_floats <= 100 * 1024;
+}
+
+template <int W, int PP, bool SYSTEM, bool RESIDENT>
+static rb_status launch_fnet_form(const rb_fnet* f, cudaStream_t st, int64_t ctas, int sms, const FnSrc& src,
+                                  const FnDst& dst) {
+    const size_t smem = sizeof(float) * (size_t)f->img_floats * (RESIDENT ? kFnNets : 1);
+    static std::atomic<bool> allowed{false};
+    if (!allowed.load()) {
+        RB_CUDA(cudaFuncSetAttribute(k_fnet_pairs<W, PP, SYSTEM, RESIDENT>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        allowed.store(true);
     }
-#undef RB_FN
+    int per_sm = 1;  // one wave of CTAs, each with its own copy of the weights
+    RB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fnet_pairs<W, PP, SYSTEM, RESIDENT>,
+                                                          kFnThreads, smem));
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ctas, (int64_t)sms * std::max(1, per_sm)));
+    if (SYSTEM)
+        RB_CUDA(launch_pdl(k_fnet_pairs<W, PP, SYSTEM, RESIDENT>, grid, kFnThreads, smem, st,
+                           (const float*)f->img, f->depth, (int)f->img_floats, src, dst));
+    else
+        k_fnet_pairs<W, PP, SYSTEM, RESIDENT><<<grid, kFnThreads, smem, st>>>(f->img, f->depth,
+                                                                            (int)f->img_floats, src, dst);
     RB_CUDA(cudaGetLastError());
     return RB_OK;
+}
+
+template <int W, int PP, bool SYSTEM>
+static rb_status launch_fnet_w(const rb_fnet* f, cudaStream_t st, int64_t ctas, int sms, const FnSrc& src,
+                               const FnDst& dst) {
+    ctas = (ctas + PP - 1) / PP;
+    return fn_resident(f) ? launch_fnet_form<W, PP, SYSTEM, true>(f, st, ctas, sms, src, dst)
+                          : launch_fnet_form<W, PP, SYSTEM, false>(f, st, ctas, sms, src, dst);
+}
+
+// ctas: CTAs of kFnThreads pairs
+template <bool SYSTEM>
+static rb_status launch_fnet(const rb_fnet* f, cudaStream_t st, int64_t ctas, const FnSrc& src, const FnDst& dst) {
+    int sms = 1;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, f->device);
+    switch (f->width) {
+        case 16: return launch_fnet_w<16, 2, SYSTEM>(f, st, ctas, sms, src, dst);
+        case 32: return launch_fnet_w<32, 2, SYSTEM>(f, st, ctas, sms, src, dst);
+        case 64: return launch_fnet_w<64, 1, SYSTEM>(f, st, ctas, sms, src, dst);
+        default: return fail(RB_ENOTSUP, "per-component networks support widths 16, 32, 64");
+    }
 }
 
 rb_status check_fnet(const rb_fnet* f) {
@@ -834,10 +932,7 @@ rb_status rb_fnet_pairs(const rb_fnet* f, int64_t n, const float* cfg, float* ou
     src.n = n;
     FnDst dst{};
     dst.out = reinterpret_cast<float4*>(out);
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, f->device);
-    const int grid = (int)std::min<int64_t>((n + kFnThreads - 1) / kFnThreads, (int64_t)sms * 8);
-    return launch_fnet<false>(f, f->stream, grid, src, dst);
+    return launch_fnet<false>(f, f->stream, (n + kFnThreads - 1) / kFnThreads, src, dst);
 }
 
 rb_status rb_fnet_trainer_create(rb_fnet* f, int64_t max_batch, float lr, float beta1, float beta2,
