@@ -470,10 +470,11 @@ rb_status fnet_pairs_system_async(rb_system* s, const rb_fnet* f) {
 // layer; activations and signals live in shared memory as [unit][sample] (row
 // stride S + 4, so that rows of consecutive units fall on different banks),
 // silu' and the top activations, which only their own thread reads again, in a
-// global scratch; the weights (4 KB a matrix at width 32) come through L1.
+// global scratch; the network's weights (17 KB at width 32, depth 3) are staged in shared
+// memory or come through L1 (FnTile::staged).
 // A step was about 130 launches (GEMMs, column sums and elementwise kernels of
 // the five networks one after the other, 880 us at batch 4096 and width 32, for
-// 0.27 GFLOP); it is two, 40 us (this kernel 34 us), and the gradient's error
+// 0.27 GFLOP); it is two, 36 us (this kernel 30 us), and the gradient's error
 // against FP64 went from 8.6e-7 to 1.1e-7.  Bound by latency: a dozen dependent
 // short stages.
 struct FnTrainArgs {
@@ -492,6 +493,11 @@ struct FnTile {
         return sizeof(float) * ((size_t)(D + 1) * W * LD + kFnIn * LD + NG * S + 2 * S + kWarpsPerUnit * W + 16) +
                sizeof(double) * 256;
     }
+    // a network's image and stored matrices beside them, where two CTAs per SM
+    // still fit (width 32: 39.5 -> 35.7 us a step of 4096; width 64, where only
+    // one would: 74 -> 82 us)
+    static size_t weights(int D) { return sizeof(float) * ((size_t)fn_img_size(W, D) + (size_t)(D - 1) * W * W); }
+    static bool staged(int D) { return smem(D) + weights(D) <= 112 * 1024; }
 };
 __host__ __device__ inline size_t fn_scratch_floats(int D) { return (size_t)(D + 1) * 4 * 256 * kFnCpt; }
 
@@ -557,8 +563,8 @@ __device__ inline void fn_gemm(const float* __restrict__ As, const float* __rest
 template <int W>
 __global__ void __launch_bounds__(256)
     k_fn_tile(const float* __restrict__ img, int64_t img_sz, const float* __restrict__ wr, int D, FnTrainArgs A,
-              float* __restrict__ part, int64_t nn, float* __restrict__ scratch,
-              double* __restrict__ loss_part) {
+              float* __restrict__ part, int64_t nn, float* __restrict__ scratch, double* __restrict__ loss_part,
+              int staged) {
     using T = FnTile<W>;
     constexpr int S = T::S, LD = T::LD, NTP = T::NTP, NG = T::NG;
     pdl_wait();
@@ -577,6 +583,16 @@ __global__ void __launch_bounds__(256)
     const int cta = c * n_share + share;
     const FnLayout L = fn_layout(W, D);
     const float* net = img + c * img_sz;  // matrices [in][out], everything else as in the flat layout
+    const float* wrc = wr + (int64_t)c * (D - 1) * W * W;
+    if (staged) {
+        float4* w4 = reinterpret_cast<float4*>(Wp + T::kWarpsPerUnit * W);
+        const int ni = (int)img_sz / 4, nr = (D - 1) * W * W / 4;
+        for (int k = tid; k < ni; k += 256) w4[k] = reinterpret_cast<const float4*>(net)[k];
+        for (int k = tid; k < nr; k += 256) w4[ni + k] = reinterpret_cast<const float4*>(wrc)[k];
+        net = reinterpret_cast<const float*>(w4);
+        wrc = reinterpret_cast<const float*>(w4 + ni);
+        __syncthreads();
+    }
     float* gp = part + (size_t)cta * nn;
     float* mine = scratch + (size_t)cta * fn_scratch_floats(D) + (size_t)tid * kFnCpt;
     auto slot = [&](int k, int j) { return mine + ((size_t)k * 4 + j) * 256 * kFnCpt; };
@@ -701,7 +717,7 @@ __global__ void __launch_bounds__(256)
                 break;
             }
             fn_weight_grad<W>(g, Hs + (size_t)(l - 1) * W * LD, gp + L.w(l), first);
-            fn_gemm<W>(g, wr + ((int64_t)c * (D - 1) + l - 1) * W * W, W, p0, o0, acc);
+            fn_gemm<W>(g, wrc + (size_t)(l - 1) * W * W, W, p0, o0, acc);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 TrVec<kFnCpt> d1 = tr_ld<kFnCpt>(slot(l - 1, j));
@@ -803,8 +819,11 @@ static rb_status launch_fn_tile(rb_fnet_trainer* t, int shares, const FnTrainArg
         RB_CUDA(cudaFuncSetAttribute(k_fn_tile<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         allowed.store(true);
     }
-    RB_CUDA(launch_pdl(k_fn_tile<W>, dim3(kFnNets, shares), 256, FnTile<W>::smem(f->depth), f->stream, f->img,
-                       f->img_floats, f->wr, f->depth, A, t->part, f->net_floats, t->scratch, t->loss_part));
+    const bool staged = FnTile<W>::staged(f->depth);
+    RB_CUDA(launch_pdl(k_fn_tile<W>, dim3(kFnNets, shares), 256,
+                       FnTile<W>::smem(f->depth) + (staged ? FnTile<W>::weights(f->depth) : 0), f->stream, f->img,
+                       f->img_floats, f->wr, f->depth, A, t->part, f->net_floats, t->scratch, t->loss_part,
+                       staged ? 1 : 0));
     return RB_OK;
 }
 
