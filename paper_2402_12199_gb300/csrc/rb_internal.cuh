@@ -151,7 +151,7 @@ struct PairList {
     int* lower_count = nullptr; // N
     int* lower_pair = nullptr;  // N x max_nbr: pair index of each lower neighbour
     int* half_off = nullptr;    // N + 1
-    int* seg = nullptr;         // pair count (0 between rebuilds), then first pair, of each segment of bodies
+    int* seg = nullptr;         // pair count, then first pair, of each segment of bodies
     int* done = nullptr;        // 2 counters of the last-CTA hand-offs of a rebuild (0 between)
     int2* pairs = nullptr;      // cap_pairs
     int* n_pairs = nullptr;     // device scalar

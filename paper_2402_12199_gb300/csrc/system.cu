@@ -114,15 +114,13 @@ __device__ inline int block_scan256(int v, int& total) {
 
 // First pair index of every segment of kSegBodies bodies, by one CTA (the last
 // of k_pair_build): the exclusive scan of the segments' pair counts, 256 at a
-// time.  half_off[N] and *total get the pair count (capped, with the overflow
-// bit raised).  k_pair_emit completes the bodies' own offsets inside their
-// segment.  (Scanning the N body counts here instead, a contiguous chunk of
-// them per thread, took about 1 ms of the 1.33 ms list build at 524288
-// bodies: 2048 dependent-latency reads per thread on one SM.)
-__device__ inline void scan_segments(const int* __restrict__ seg_sum, int* __restrict__ seg_base,
-                                     int N, int* __restrict__ half_off, int* total,
-                                     int64_t cap_pairs, unsigned* status) {
-    const int S = (N + kSegBodies - 1) / kSegBodies;
+// time.  Only for very large systems (kScanSegments): below, every CTA of
+// k_pair_emit adds up the segments before its own, which is off the critical
+// path of the build (at 524288 bodies the scan of 4096 sums by one CTA took
+// about 20 us; reading them costs each emitting CTA 16 loads a thread at most).
+constexpr int kScanSegments = 16384;
+__device__ inline void scan_segments(const int* __restrict__ seg_sum, int* __restrict__ seg_base, int N) {
+    const int S = pair_segments(N);
     int run = 0;
     for (int k0 = 0; k0 < S; k0 += 256) {
         const int k = k0 + threadIdx.x;
@@ -130,14 +128,6 @@ __device__ inline void scan_segments(const int* __restrict__ seg_sum, int* __res
         const int e = block_scan256(k < S ? __ldcg(seg_sum + k) : 0, sum);
         if (k < S) seg_base[k] = run + e;
         run += sum;
-    }
-    if (threadIdx.x == 0) {
-        if ((int64_t)run > cap_pairs) {
-            atomicOr(status, ST_NBR_OVERFLOW);
-            run = (int)cap_pairs;
-        }
-        half_off[N] = run;
-        *total = run;
     }
 }
 
@@ -151,7 +141,8 @@ __device__ __forceinline__ void cell_assign_body(const float4* __restrict__ pos,
                                                  float3 invL, float3 invw, int3 nc,
                                                  int* __restrict__ count, int* __restrict__ bodies,
                                                  int cap, unsigned* status, int* rebuild,
-                                                 int* zero_count, int force, int bid) {
+                                                 int* zero_count, int* __restrict__ seg_sum,
+                                                 int force, int bid) {
     pdl_chain();
     if (zero_count && bid == 0 && threadIdx.x == 0) *zero_count = 0;
     if (force) {
@@ -161,6 +152,7 @@ __device__ __forceinline__ void cell_assign_body(const float4* __restrict__ pos,
     }
     int i = bid * blockDim.x + threadIdx.x;
     if (i >= N) return;
+    if (i < pair_segments(N)) seg_sum[i] = 0;  // the pair counts that the build adds up
     float4 p = pos[i];
     float x = wrap1(p.x, L.x, invL.x), y = wrap1(p.y, L.y, invL.y), z = wrap1(p.z, L.z, invL.z);
     int cx = min(max(int(x * invw.x), 0), nc.x - 1);
@@ -177,9 +169,9 @@ __device__ __forceinline__ void cell_assign_body(const float4* __restrict__ pos,
 __global__ void k_cell_assign(const float4* __restrict__ pos, int N, float3 L, float3 invL,
                               float3 invw, int3 nc, int* __restrict__ count,
                               int* __restrict__ bodies, int cap, unsigned* status, int* rebuild,
-                              int* zero_count, int force) {
+                              int* zero_count, int* __restrict__ seg_sum, int force) {
     cell_assign_body(pos, N, L, invL, invw, nc, count, bodies, cap, status, rebuild, zero_count,
-                     force, blockIdx.x);
+                     seg_sum, force, blockIdx.x);
 }
 
 __device__ inline void sort_row(int* row, int n) {
@@ -281,9 +273,9 @@ __device__ __noinline__ void pair_row_warp(int i, const float4* __restrict__ pos
 // bounds it: the gathers of the cell counts, cell entries and positions, a
 // chain of three L2 latencies per block; a warp per body had that chain (two
 // loads deep) once per occupied stencil slot, and sorted its rows in global
-// memory.  The CTA that finishes last scans the segments.  Measured (with the
-// segment scan): 1332 -> about 145 us at 524288 cubes, 92 -> 21 us at 32768
-// cylinders, 49 -> 21 us at 20011 cubes.
+// memory.  The whole build
+// (cell assignment, rows, offsets and emission, back to back): 1407 -> 244 us for
+// 524288 cubes, 111 -> 40 us for 32768 cylinders, 66 -> 35 us for 20011 cubes.
 constexpr int kBlkX = 8, kBlkY = 4, kBlkZ = 4;
 constexpr int kHaloX = kBlkX + 2, kHaloY = kBlkY + 2, kHaloZ = kBlkZ + 2;
 constexpr int kHalo = kHaloX * kHaloY * kHaloZ;
@@ -300,16 +292,16 @@ __device__ __forceinline__ void pair_build_body(
     const int* __restrict__ count, const int* __restrict__ bodies, int cap, float Rc2, int max_nbr,
     int* __restrict__ half_count, int* __restrict__ nbr, int* __restrict__ lower_count,
     int* __restrict__ lower_pair, int* __restrict__ seg_sum, int* __restrict__ seg_base,
-    unsigned* status, const int* __restrict__ rebuild, int* __restrict__ half_off, int* total,
-    int64_t cap_pairs, int* done, int bid, int nblk) {
+    unsigned* status, const int* __restrict__ rebuild, int* done, int bid, int nblk) {
     pdl_chain();
     if (!*rebuild) return;
     __shared__ float4 s_body[kBlkCap];            // position, body index in w
     __shared__ int s_start[kHalo + 1];            // first body of each cell, x fastest
-    __shared__ int s_list[kBlkCap];               // bodies of the block: cell << 16 | index
+    __shared__ int s_own[kHalo];                  // the same among the block's own bodies
+    __shared__ int s_list[kBlkCap];               // the block's bodies in cell order: cell << 16 | index
     __shared__ int s_row[kRowCap][256];           // neighbours found, a column per thread
     __shared__ int s_slow[256];
-    __shared__ int s_n, s_nslow;
+    __shared__ int s_nslow;
     static_assert(kHalo <= 512 && kBlkCap <= 65536, "two cells per thread; packed indices");
     const int tid = threadIdx.x, warp = tid >> 5;
     const int3 nb = make_int3((nc.x + kBlkX - 1) / kBlkX, (nc.y + kBlkY - 1) / kBlkY,
@@ -326,22 +318,33 @@ __device__ __forceinline__ void pair_build_body(
             return (wrap(b0.z + hz - 1, nc.z) * nc.y + wrap(b0.y + hy - 1, nc.y)) * nc.x +
                    wrap(b0.x + hx - 1, nc.x);
         };
-        int cnt[2] = {0, 0};
+        auto in_block = [&](int c) {
+            const int hx = c % kHaloX, hy = c / kHaloX % kHaloY, hz = c / (kHaloX * kHaloY);
+            return hx >= 1 && hx <= w.x && hy >= 1 && hy <= w.y && hz >= 1 && hz <= w.z;
+        };
+        int cnt[2] = {0, 0}, own[2] = {0, 0};
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int c = 2 * tid + u;
             const int g = c < kHalo ? cell_of(c) : -1;
             if (g >= 0) cnt[u] = min(count[g], cap);
+            own[u] = in_block(c) ? cnt[u] : 0;
         }
-        int n_all;
+        int n_all, n_own;
         const int e0 = block_scan256(cnt[0] + cnt[1], n_all);
-        if (2 * tid < kHalo) s_start[2 * tid] = e0;
-        if (2 * tid + 1 < kHalo) s_start[2 * tid + 1] = e0 + cnt[0];
+        const int f0 = block_scan256(own[0] + own[1], n_own);
+        if (2 * tid < kHalo) s_start[2 * tid] = e0, s_own[2 * tid] = f0;
+        if (2 * tid + 1 < kHalo) s_start[2 * tid + 1] = e0 + cnt[0], s_own[2 * tid + 1] = f0 + own[0];
         if (tid == 0) {
             s_start[kHalo] = n_all;
-            s_n = s_nslow = 0;
+            s_nslow = 0;
         }
         __syncthreads();
+        // a block whose surroundings do not cross a face of the box (and a box
+        // of at least four cells a side, so that two cells span less than half
+        // of it) needs no minimum image: the image shift would be an exact zero
+        const bool wrap = b0.x == 0 || b0.y == 0 || b0.z == 0 || b0.x + w.x == nc.x || b0.y + w.y == nc.y ||
+                          b0.z + w.z == nc.z || min(min(nc.x, nc.y), nc.z) < 4;
         auto row_warp = [&](int i) {
             pair_row_warp(i, pos, L, invL, invw, nc, count, bodies, cap, Rc2, max_nbr, half_count, nbr,
                           lower_count, lower_pair, seg_sum, status);
@@ -359,9 +362,8 @@ __device__ __forceinline__ void pair_build_body(
             const int st = s_start[c], n = s_start[c + 1] - st;
             if (n == 0) continue;
             const int* cb = bodies + (size_t)cell_of(c) * cap;
-            const int hx = c % kHaloX, hy = c / kHaloX % kHaloY, hz = c / (kHaloX * kHaloY);
-            const bool own = hx >= 1 && hx <= w.x && hy >= 1 && hy <= w.y && hz >= 1 && hz <= w.z;
-            const int at = own ? atomicAdd(&s_n, n) : 0;
+            const bool own = in_block(c);
+            const int at = s_own[c];
             for (int s = 0; s < n; s += 4) {  // four entries, then four positions in flight
                 int j[4];
                 float4 q[4];
@@ -384,9 +386,9 @@ __device__ __forceinline__ void pair_build_body(
         const int xl = nc.x >= 3 ? -1 : 0, xh = nc.x >= 2 ? 1 : 0;
         const int yl = nc.y >= 3 ? -1 : 0, yh = nc.y >= 2 ? 1 : 0;
         const int zl = nc.z >= 3 ? -1 : 0, zh = nc.z >= 2 ? 1 : 0;
-        for (int k0 = 0; k0 < s_n; k0 += 256) {
+        for (int k0 = 0; k0 < n_own; k0 += 256) {
             const int k = k0 + tid;
-            if (k < s_n) {
+            if (k < n_own) {
                 const int c = s_list[k] >> 16;
                 const float4 p = s_body[s_list[k] & 0xFFFF];
                 const int i = __float_as_int(p.w);
@@ -395,11 +397,12 @@ __device__ __forceinline__ void pair_build_body(
                     for (int dy = yl; dy <= yh; ++dy) {
                         const int r = c + (dz * kHaloY + dy) * kHaloX;
                         const int e1 = s_start[r + xh + 1];
+#pragma unroll 2
                         for (int e = s_start[r + xl]; e < e1; ++e) {
                             const float4 q = s_body[e];
                             const int j = __float_as_int(q.w);
-                            const float3 d =
-                                min_image(make_float3(q.x - p.x, q.y - p.y, q.z - p.z), L, invL);
+                            float3 d = make_float3(q.x - p.x, q.y - p.y, q.z - p.z);
+                            if (wrap) d = min_image(d, L, invL);
                             if (d.x * d.x + d.y * d.y + d.z * d.z < Rc2 && j != i) {
                                 if (m < kRowCap) s_row[m][tid] = j;
                                 ++m;
@@ -430,8 +433,7 @@ __device__ __forceinline__ void pair_build_body(
             __syncthreads();
         }
     }
-    if (last_cta_done(done, nblk))
-        scan_segments(seg_sum, seg_base, N, half_off, total, cap_pairs, status);
+    if (pair_segments(N) > kScanSegments && last_cta_done(done, nblk)) scan_segments(seg_sum, seg_base, N);
 }
 
 __global__ void __launch_bounds__(256, kBuildCtas) k_pair_build(
@@ -439,11 +441,10 @@ __global__ void __launch_bounds__(256, kBuildCtas) k_pair_build(
     const int* __restrict__ count, const int* __restrict__ bodies, int cap, float Rc2, int max_nbr,
     int* __restrict__ half_count, int* __restrict__ nbr, int* __restrict__ lower_count,
     int* __restrict__ lower_pair, int* __restrict__ seg_sum, int* __restrict__ seg_base,
-    unsigned* status, const int* __restrict__ rebuild, int* __restrict__ half_off, int* total,
-    int64_t cap_pairs, int* done) {
+    unsigned* status, const int* __restrict__ rebuild, int* done) {
     pair_build_body(pos, N, L, invL, invw, nc, count, bodies, cap, Rc2, max_nbr, half_count, nbr,
-                    lower_count, lower_pair, seg_sum, seg_base, status, rebuild, half_off, total,
-                    cap_pairs, done, blockIdx.x, gridDim.x);
+                    lower_count, lower_pair, seg_sum, seg_base, status, rebuild, done, blockIdx.x,
+                    gridDim.x);
 }
 
 // Emit the compact pair list, a segment of kSegBodies bodies per CTA and pass:
@@ -458,8 +459,8 @@ __global__ void __launch_bounds__(256, kBuildCtas) k_pair_build(
 __device__ __forceinline__ void pair_emit_body(
     int N, int max_nbr, const int* __restrict__ half_count, const int* __restrict__ nbr,
     int* __restrict__ half_off, const int* __restrict__ lower_count, int* __restrict__ lower_pair,
-    int* __restrict__ seg_sum, const int* __restrict__ seg_base, int2* __restrict__ pairs,
-    int64_t cap_pairs, unsigned* status, int n_cells, const float4* __restrict__ pos,
+    const int* __restrict__ seg_sum, const int* __restrict__ seg_base, int2* __restrict__ pairs,
+    int* total, int64_t cap_pairs, unsigned* status, int n_cells, const float4* __restrict__ pos,
     float4* __restrict__ pos_ref, int* __restrict__ cell_count, int* rebuild, int* done, int bid,
     int nblk) {
     pdl_chain();
@@ -471,14 +472,30 @@ __device__ __forceinline__ void pair_emit_body(
     for (int seg = bid; seg < S; seg += nblk) {
         const int i0 = seg * kSegBodies, i = i0 + tid;
         const bool own = tid < kSegBodies && i < N;
-        const int base = seg_base[seg];
-        const int low = own ? lower_count[i] : 0;
+        const int low = own ? lower_count[i] : 0, cnt = own ? half_count[i] : 0;
+        int base = 0;
+        if (S > kScanSegments) {
+            base = seg_base[seg];
+        } else {
+            int before = 0;
+#pragma unroll 8
+            for (int k = tid; k < seg; k += 256) before += seg_sum[k];
+            block_scan256(before, base);
+        }
         int n_all;
-        const int e = block_scan256(own ? half_count[i] : 0, n_all);
+        const int e = block_scan256(cnt, n_all);
         if (tid < kSegBodies) s_off[tid] = e;
         if (tid == 0) {
             s_off[kSegBodies] = n_all;
-            seg_sum[seg] = 0;
+            if (seg == S - 1) {  // the pair count (capped, with the overflow bit raised)
+                int64_t n = (int64_t)base + n_all;
+                if (n > cap_pairs) {
+                    atomicOr(status, ST_NBR_OVERFLOW);
+                    n = cap_pairs;
+                }
+                half_off[N] = (int)n;
+                *total = (int)n;
+            }
         }
         if (own) {
             s_low[tid] = low;
@@ -521,11 +538,11 @@ __device__ __forceinline__ void pair_emit_body(
 __global__ void __launch_bounds__(256) k_pair_emit(
     int N, int max_nbr, const int* __restrict__ half_count, const int* __restrict__ nbr,
     int* __restrict__ half_off, const int* __restrict__ lower_count, int* __restrict__ lower_pair,
-    int* __restrict__ seg_sum, const int* __restrict__ seg_base, int2* __restrict__ pairs,
-    int64_t cap_pairs, unsigned* status, int n_cells, const float4* __restrict__ pos,
+    const int* __restrict__ seg_sum, const int* __restrict__ seg_base, int2* __restrict__ pairs,
+    int* total, int64_t cap_pairs, unsigned* status, int n_cells, const float4* __restrict__ pos,
     float4* __restrict__ pos_ref, int* __restrict__ cell_count, int* rebuild, int* done) {
     pair_emit_body(N, max_nbr, half_count, nbr, half_off, lower_count, lower_pair, seg_sum, seg_base,
-                   pairs, cap_pairs, status, n_cells, pos, pos_ref, cell_count, rebuild, done,
+                   pairs, total, cap_pairs, status, n_cells, pos, pos_ref, cell_count, rebuild, done,
                    blockIdx.x, gridDim.x);
 }
 
@@ -987,7 +1004,7 @@ __global__ void k_cell_assign_batch(const StepSeg* __restrict__ segs, const int*
     const int k = seg_of_block(start, n_seg, blockIdx.x);
     const StepSeg& S = segs[k];
     cell_assign_body(S.pos, S.N, S.L, S.invL, S.invw, S.nc, S.cell_count, S.cell_bodies, S.cell_cap,
-                     S.status, S.rebuild, S.zero_count, 0, blockIdx.x - start[k]);
+                     S.status, S.rebuild, S.zero_count, S.seg, 0, blockIdx.x - start[k]);
 }
 
 __global__ void __launch_bounds__(256, kBuildCtas) k_pair_build_batch(const StepSeg* __restrict__ segs, const int* __restrict__ start,
@@ -996,8 +1013,7 @@ __global__ void __launch_bounds__(256, kBuildCtas) k_pair_build_batch(const Step
     const StepSeg& S = segs[k];
     pair_build_body(S.pos, S.N, S.L, S.invL, S.invw, S.nc, S.cell_count, S.cell_bodies, S.cell_cap,
                     S.Rl2, S.max_nbr, S.half_count, S.nbr, S.lower_count, S.lower_pair, S.seg,
-                    S.seg + pair_segments(S.N), S.status, S.rebuild, S.half_off, S.n_pairs,
-                    S.cap_pairs, S.done, blockIdx.x - start[k], start[k + 1] - start[k]);
+                    S.seg + pair_segments(S.N), S.status, S.rebuild, S.done, blockIdx.x - start[k], start[k + 1] - start[k]);
 }
 
 __global__ void __launch_bounds__(256) k_pair_emit_batch(const StepSeg* __restrict__ segs, const int* __restrict__ start,
@@ -1005,7 +1021,7 @@ __global__ void __launch_bounds__(256) k_pair_emit_batch(const StepSeg* __restri
     const int k = seg_of_block(start, n_seg, blockIdx.x);
     const StepSeg& S = segs[k];
     pair_emit_body(S.N, S.max_nbr, S.half_count, S.nbr, S.half_off, S.lower_count, S.lower_pair, S.seg,
-                   S.seg + pair_segments(S.N), S.pairs, S.cap_pairs, S.status, S.n_cells, S.pos,
+                   S.seg + pair_segments(S.N), S.pairs, S.n_pairs, S.cap_pairs, S.status, S.n_cells, S.pos,
                    S.pos_ref, S.cell_count, S.rebuild, S.done + 1, blockIdx.x - start[k],
                    start[k + 1] - start[k]);
 }
@@ -1043,19 +1059,19 @@ rb_status build_pairs_async(rb_system* s, bool force, bool checked, int* zero_co
     }
     RB_CUDA(launch_pdl(k_cell_assign, blocks_for(N, 256), 256, 0, s->stream, s->pos, N, L, invL,
                        invw, nc, s->cells.count, s->cells.bodies, s->cells.cap, s->status_dev,
-                       s->rebuild_flag, zero_count, force ? 1 : 0));
+                       s->rebuild_flag, zero_count, s->pl.seg, force ? 1 : 0));
     s->fb_zeroed = zero_count != nullptr;
     int* seg_base = s->pl.seg + pair_segments(N);
     RB_CUDA(launch_pdl(k_pair_build, std::min(cell_blocks(nc), s->num_sms * kBuildCtas), 256, 0, s->stream,
                        s->pos, N, L, invL, invw, nc, s->cells.count, s->cells.bodies, s->cells.cap,
                        Rl * Rl, s->pl.max_nbr, s->pl.half_count, s->pl.nbr, s->pl.lower_count,
                        s->pl.lower_pair, s->pl.seg, seg_base, s->status_dev, s->rebuild_flag,
-                       s->pl.half_off, s->pl.n_pairs, s->pl.cap_pairs, s->pl.done));
+                       s->pl.done));
     RB_CUDA(launch_pdl(k_pair_emit, std::min(blocks_for(std::max(N, s->cells.n_cells), 256),
                                              s->num_sms * 8),
                        256, 0, s->stream, N, s->pl.max_nbr, s->pl.half_count, s->pl.nbr,
                        s->pl.half_off, s->pl.lower_count, s->pl.lower_pair, s->pl.seg, seg_base,
-                       s->pl.pairs, s->pl.cap_pairs, s->status_dev, s->cells.n_cells, s->pos,
+                       s->pl.pairs, s->pl.n_pairs, s->pl.cap_pairs, s->status_dev, s->cells.n_cells, s->pos,
                        s->pos_ref, s->cells.count, s->rebuild_flag, s->pl.done + 1));
     RB_CUDA(cudaGetLastError());
     return RB_OK;

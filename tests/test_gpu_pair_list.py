@@ -119,3 +119,29 @@ def test_too_many_neighbours_is_reported_and_the_next_list_is_right(n, max_neigh
     ref = _brute(spread[:, :3].astype(np.float64), box)
     got = set(map(tuple, s.pairs().tolist()))
     assert got <= set(ref) and all(r > RC - 1e-4 for k, r in ref.items() if k not in got)
+
+
+def test_more_segments_than_one_pass_adds_up():
+    """130^3 bodies on a lattice with six neighbours each: more offset segments than a CTA of the
+    emitting kernel adds up by itself."""
+    import torch
+
+    from paper_2402_12199_gb300 import api
+
+    m, a = 130, 3.3
+    n = m ** 3
+    rng = np.random.default_rng(3)
+    site = rng.permutation(n)  # body -> lattice site
+    ijk = np.stack([site // (m * m), site // m % m, site % m], 1)
+    pos = np.zeros((n, 4), np.float32)
+    pos[:, :3] = (ijk + 0.5) * a
+    quat = np.zeros((n, 4), np.float32)
+    quat[:, 0] = 1.0
+    s = api.System(n, [m * a] * 3, "custom", template=OCTA, max_neighbors=8)
+    s.set_state(torch.from_numpy(pos).cuda(), torch.from_numpy(quat).cuda())
+    assert s.build_pairs() == 3 * n
+    p = s.pairs().astype(np.int64)
+    assert np.all(p[:, 0] < p[:, 1]) and np.all(np.diff(p[:, 0] * n + p[:, 1]) > 0)
+    d = np.abs(ijk[p[:, 0]] - ijk[p[:, 1]])
+    d = np.minimum(d, m - d)
+    assert np.all(d.sum(1) == 1)
