@@ -520,8 +520,6 @@ inline void set_symmetry(PairSrc& src, const rb_mlp* m) {
 }
 
 // nn.cu
-rb_status nn_pairs_f32_async(const rb_mlp* m, int64_t n, const float4* cfg, float4* out,
-                             float4* grad);
 rb_status mlp_refresh(rb_mlp* m);  // rebuild the derived weight copies after params change
 // nn_tc.cu
 rb_status nn_tc_prepare(rb_mlp* m);

@@ -562,6 +562,7 @@ rb_status nn_f16x3_pairs_async(const rb_mlp* m, int64_t n, const float4* cfg, fl
     dst.out = out;
     dst.grad = grad;
     const int grid = (int)std::min<int64_t>(sm_count_f16x3(), (n + tc::kM - 1) / tc::kM);
+    const_cast<rb_mlp*>(m)->status_used.store(true);
     return launch_f16x3<false>(m, m->stream, std::max(grid, 1), src, dst, m->status_dev);
 }
 

@@ -440,6 +440,7 @@ rb_status nn_tc_pairs_async(const rb_mlp* m, int64_t n, const float4* cfg, float
     dst.out = out;
     dst.grad = grad;
     const int grid = (int)std::min<int64_t>(sm_count_tc(), (n + tc::kM - 1) / tc::kM);
+    const_cast<rb_mlp*>(m)->status_used.store(true);
     return launch_tc<false>(m, m->stream, std::max(grid, 1), src, dst, m->status_dev);
 }
 

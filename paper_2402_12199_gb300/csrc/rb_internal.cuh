@@ -199,6 +199,9 @@ struct rb_mlp {
     void* bf16_img = nullptr;     // BF16 shared-memory image for the tensor-core kernel
     void* f16x3_img = nullptr;    // FP16 hi/lo weight image of the FP32-accurate tensor-core kernel
     unsigned* status_dev = nullptr;  // sticky device-side error bits of pair-level calls
+    // set by the first tensor-core call on explicit pairs (launched or captured)
+    // and never cleared: no other kernel of the network can raise the bits
+    std::atomic<bool> status_used{false};
     uint64_t version = 1;         // bumped on every set_params
     // the version the BF16 and F16X3 images were built for: they are built when
     // a kernel of that precision first runs after a change (ensure_images)
