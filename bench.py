@@ -50,7 +50,7 @@ WIDTH, DEPTH = 128, 3
 #                   --drift-steps 0 --no-paper-workload --fnet-train-steps 0
 #                   --descriptor-comparison 0
 # None marks a kernel not captured since it last changed.
-NCU_DRAM_BYTES = {"k_bead_pairs": 1.869e6, "k_nn_f32": 2.185e6, "k_nn_tc2p": 2.052e6,
+NCU_DRAM_BYTES = {"k_bead_cols": None, "k_nn_f32": 2.185e6, "k_nn_tc2p": 2.052e6,
                   "k_nn_tc256": 2.474e6, "k_nn_f16x3": 2.213e6}
 # The MD step's HBM-side kernels from the same captures (median launch, no
 # list rebuild due): DRAM bytes read + written and the ncu duration (cold L2,
@@ -784,9 +784,9 @@ def main():
         flops = bw["flops"]
         achieved = flops / (d_ms * 1e-3) / 1e12
         peak = unit["fp32_tflops"]
-        roof_beads = {"kernel": "k_bead_pairs", "bound": "alu", "achieved": achieved, "peak": peak,
+        roof_beads = {"kernel": "k_bead_cols", "bound": "alu", "achieved": achieved, "peak": peak,
                       "unit": "TFLOP/s", "frac": achieved / peak,
-                      "traffic": NCU_DRAM_BYTES["k_bead_pairs"],
+                      "traffic": NCU_DRAM_BYTES["k_bead_cols"],
                       "traffic_unit": "bytes per launch (ncu)", "kernel_ms": d_ms,
                       "peak_source": "measured FP32 FMA rate (the larger of the FFMA and FFMA2 "
                                      "probes, measured_unit_peaks)",
@@ -1080,7 +1080,7 @@ def main():
         torch.cuda.synchronize()
         ms_p = statistics.mean(a.elapsed_time(b) for a, b in ev_p)
         _, kt_p, kr_p = sp.energy()
-        # the pair kernel alone (k_bead_pairs with the half-power half-cosine body)
+        # the pair kernel alone (k_bead_cols with the half-power half-cosine body)
         sp.build_pairs()
         kp = []
         for _ in range(10):
@@ -1116,7 +1116,7 @@ def main():
             "ms_per_md_step": ms_p, "md_steps_per_s": 1e3 / ms_p,
             "pair_evals_per_s": n_pairs_p / (ms_p * 1e-3), "pairs": n_pairs_p,
             "steps_timed": 300, "temperature_2K_over_g": 2 * (kt_p + kr_p) / (6 * N_BODIES - 3),
-            "kernel": "k_bead_pairs (half-power half-cosine)", "kernel_ms": kms_p,
+            "kernel": "k_bead_cols (half-power half-cosine)", "kernel_ms": kms_p,
             "kernel_tflops": flops_p / (kms_p * 1e-3) / 1e12,
             "frac_of_fp32_peak": flops_p / (kms_p * 1e-3) / 1e12 / unit["fp32_tflops"],
             "kernel_work": "as roofline_beads (distance tests the column test leaves, bead pairs "
@@ -1530,7 +1530,7 @@ def main():
                                     "note": "the same with one cudaMemcpyAsync each way around "
                                             "the step"}},
             # per MD step and path: integrate (with the skin check), cell assign,
-            # pair build (+ scan), emit (+ finish), pair kernel, reduce; plus the
+            # pair build, emit (+ offsets, finish), pair kernel, reduce; plus the
             # bead fallback kernel on the network paths
             "gpu_launches": args.steps * (6 * len(paths) + (sum(p.startswith("nn") for p in paths)
                                                            if rho_fallback > 0 else 0)),

@@ -644,9 +644,8 @@ rb_status rb_mlp_sync(const rb_mlp* mlp);
 rb_status rb_tc_gemm_check(int32_t N, int32_t K, const float* A, const float* B, float* D,
                            void* cuda_stream);
 
-/* FP32-accurate GEMM on the tensor cores, the product every GEMM of the
- * force-matching training pass (rb_train_grad / rb_train_step,
- * rb_fnet_train_*) uses (paper, Methods: training of the pair network):
+/* FP32-accurate GEMM on the tensor cores, for products of dense layers over a
+ * batch (paper, Methods: training of the pair network):
  *   C = alpha A B + beta C,  A(m, k) = A[m sam + k sak] (M x K),
  *   B(k, n) = B[k sbk + n sbn] (K x N), C row-major M x N with leading
  *   dimension ldc >= N; all device arrays, FP32.

@@ -1,6 +1,6 @@
-// FP32-accurate GEMM on the tensor cores for the force-matching training
-// (the forward, reverse and weight-gradient products of the training pass,
-// Methods: training of the pair network by force matching).
+// FP32-accurate GEMM on the tensor cores (rb_gemm_f32): the products of dense
+// layers over a batch (Methods: training of the pair network).  The library's
+// own training passes multiply tile by tile inside one kernel (train.cu).
 //
 //   C = alpha A B + beta C,  A(m, k) = A[m sam + k sak],  B(k, n) = B[k sbk + n sbn],
 //   C row-major with leading dimension ldc.

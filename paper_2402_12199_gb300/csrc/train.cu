@@ -73,7 +73,7 @@ namespace rb {
 // halving.  Every halving is decided as the scan of all pairs would decide it
 // (up to FP32 rounding of the distances): the labels' error against FP64 is
 // 5.4e-6 (5.6e-6 with full scans).  The label takes the columns near body j
-// only, as the pair kernel does.  Measured: 8885 -> 396 us for 65536 cube pairs
+// only, as the pair kernel does.  Measured: 8885 -> 333 us for 65536 cube pairs
 // at contact 0.85; bound by instruction issue (about 3500 a sample).
 constexpr int kCoarse = 5;
 constexpr int kCand = 64;
