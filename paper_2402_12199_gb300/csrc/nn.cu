@@ -16,8 +16,8 @@
 //   tau_i = s x G_s - tau_j
 // and finally a rotation by R(q_i) into the space frame.
 //
-// Kernel layout: one CTA of 256 threads per SM, persistent over tiles of P
-// pairs.  Layer activations live in shared memory as [unit][pair]; each thread
+// Kernel layout: one CTA of 256 threads per SM (or three of 128, see
+// small_tiles), persistent over tiles of P pairs.  Layer activations live in shared memory as [unit][pair]; each thread
 // owns a 4-pair x 8-unit register block of every layer GEMM, accumulated with
 // packed FP32x2 FMAs over pairs of units (the pair value is the broadcast
 // operand).  The GEMM weights (transposed copies for the forward
@@ -83,8 +83,8 @@ __device__ inline float sigmoidf_(float z) { return __fdividef(1.f, 1.f + __expf
 // acc_at(acc, i, j) += sum_k A[k][p0 + i] * B[k][o0 + j] for i = 0..3 and
 // j = 0..7: A in shared memory as [K][P], B the next K/KC weight chunks.
 // Units (j, j+1) of pair i share one FP32x2 accumulator.
-template <int W, int P, int KC>
-__device__ inline void gemm_tile(const float* __restrict__ As, int K, ChunkFeed<W, KC>& feed,
+template <int W, int P, int KC, int T>
+__device__ inline void gemm_tile(const float* __restrict__ As, int K, ChunkFeed<W, KC, T>& feed,
                                  int p0, int o0, float2 (&acc)[2][8]) {
     for (int kc = 0; kc < K; kc += KC) {
         const float* Bs = feed.acquire();
@@ -114,21 +114,23 @@ __device__ inline float acc_at(const float2 (&acc)[2][8], int i, int j) {
     return (j & 1) ? v.y : v.x;
 }
 
-template <int W, int P, int KC, bool SYSTEM>
-__global__ void __launch_bounds__(kF32Threads, 1)
+template <int W, int P, int KC, int T, int CTAS, bool SYSTEM>
+__global__ void __launch_bounds__(T, CTAS)
     k_nn_f32(NetArgs net, PairSrc src, PairDst dst) {
     extern __shared__ float4 smem4[];
     float* smem = reinterpret_cast<float*>(smem4);
     constexpr int NTP = P / 4;              // threads along pairs
-    constexpr int NG = kF32Threads / NTP;   // thread groups along units
-    constexpr int NS = kF32Threads / P;     // unit slices of the dE/dx reduction
+    constexpr int NG = T / NTP;   // thread groups along units
+    constexpr int NS = T / P;     // unit slices of the dE/dx reduction
     static_assert(NG * 8 == W, "register blocks must tile the layer width");
     static_assert(NS * kIn * P <= W * P, "dE/dx partial sums must fit in the activation buffer");
     pdl_wait();
     const int D = net.D;
-    using Feed = ChunkFeed<W, KC>;
-    float* Zs = smem;                          // D x [W][P]: silu'(z_l), then G_l
-    float* Hs = Zs + (size_t)D * W * P;        // [W][P]: h_l; dE/dx partial sums at the end
+    using Feed = ChunkFeed<W, KC, T>;
+    // max(D, 2) x [W][P]: silu'(z_l), then G_l; the last block holds h_l until
+    // G_D takes its place, and the dE/dx partial sums once G_D has been read
+    float* Zs = smem;
+    float* Hs = Zs + (size_t)(max(D, 2) - 1) * W * P;
     float* Bs = Hs + (size_t)W * P;            // 2 x [KC][W] weight chunks
     float* Xs = Bs + (size_t)2 * KC * W;       // [16][P] normalised features
     float* Red = Xs + (size_t)kInPad * P;      // [NG][P] energy partial sums
@@ -141,15 +143,15 @@ __global__ void __launch_bounds__(kF32Threads, 1)
     const int tp = threadIdx.x % NTP, to = threadIdx.x / NTP;
     const int p0 = tp * 4, o0 = to * 8;
     const float* flat = net.flat;
-    for (int t = threadIdx.x; t < kIn; t += kF32Threads) {
+    for (int t = threadIdx.x; t < kIn; t += T) {
         misc[t] = flat[net.fl.mu + t];
         misc[16 + t] = flat[net.fl.inv_sd + t];
     }
-    for (int t = threadIdx.x; t < D * W; t += kF32Threads) {
+    for (int t = threadIdx.x; t < D * W; t += T) {
         const int l = 1 + t / W, o = t % W;
         bias[t] = flat[net.fl.b_(l, W) + o];
     }
-    for (int t = threadIdx.x; t < W; t += kF32Threads) wo[t] = flat[net.fl.wo + t];
+    for (int t = threadIdx.x; t < W; t += T) wo[t] = flat[net.fl.wo + t];
     const float b_o = flat[net.fl.bo], e_scale = flat[net.fl.escale], e_shift = flat[net.fl.eshift];
 
     const int64_t n_total = SYSTEM ? (int64_t)(*src.n_pairs_ptr) : src.n_explicit;
@@ -195,10 +197,10 @@ __global__ void __launch_bounds__(kF32Threads, 1)
             for (int i = 0; i < 2; ++i)
 #pragma unroll
                 for (int j = 0; j < 8; ++j) acc[i][j] = make_float2(0.f, 0.f);
-            gemm_tile<W, P, KC>(l == 1 ? Xs : Hs, l == 1 ? kInPad : W, feed, p0, o0, acc);
+            gemm_tile<W, P, KC, T>(l == 1 ? Xs : Hs, l == 1 ? kInPad : W, feed, p0, o0, acc);
             float* Z = Zs + (size_t)(l - 1) * W * P;
+            if (l > 1) __syncthreads();  // every read of Hs by this GEMM is done
             if (l < D) {
-                if (l > 1) __syncthreads();  // every read of Hs by this GEMM is done
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const float b = bias[(l - 1) * W + o0 + j];
@@ -242,7 +244,7 @@ __global__ void __launch_bounds__(kF32Threads, 1)
             for (int i = 0; i < 2; ++i)
 #pragma unroll
                 for (int j = 0; j < 8; ++j) acc[i][j] = make_float2(0.f, 0.f);
-            gemm_tile<W, P, KC>(Zs + (size_t)(l - 1) * W * P, W, feed, p0, o0, acc);
+            gemm_tile<W, P, KC, T>(Zs + (size_t)(l - 1) * W * P, W, feed, p0, o0, acc);
             float* Z = Zs + (size_t)(l - 2) * W * P;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -304,21 +306,21 @@ __global__ void __launch_bounds__(kF32Threads, 1)
 
 constexpr size_t kSmemMax = 227 * 1024;
 
-template <int W, int P, int KC>
+template <int W, int P, int KC, int T>
 static size_t f32_smem_bytes(int D) {
-    constexpr int NG = kF32Threads / (P / 4);
-    return sizeof(float) * ((size_t)D * W * P + (size_t)W * P + (size_t)2 * KC * W +
+    constexpr int NG = T / (P / 4);
+    return sizeof(float) * ((size_t)std::max(D, 2) * W * P + (size_t)2 * KC * W +
                             (size_t)kInPad * P + (size_t)NG * P + 32 + (size_t)D * W + W);
 }
 
-template <int W, int P, int KC, bool SYSTEM>
-static rb_status launch_f32(const rb_mlp* m, cudaStream_t stream, int num_sms, const PairSrc& src,
+template <int W, int P, int KC, int T, int CTAS, bool SYSTEM>
+static rb_status launch_f32(const rb_mlp* m, cudaStream_t stream, int grid, const PairSrc& src,
                             const PairDst& dst) {
-    const size_t smem = f32_smem_bytes<W, P, KC>(m->depth);
+    const size_t smem = f32_smem_bytes<W, P, KC, T>(m->depth);
+    auto kern = k_nn_f32<W, P, KC, T, CTAS, SYSTEM>;
     static bool attr_set = false;
     if (!attr_set) {
-        RB_CUDA(cudaFuncSetAttribute(k_nn_f32<W, P, KC, SYSTEM>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        RB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
         attr_set = true;
     }
     if (smem > kSmemMax) return fail(RB_ENOTSUP, "network too deep for the FP32 kernel");
@@ -330,31 +332,46 @@ static rb_status launch_f32(const rb_mlp* m, cudaStream_t stream, int num_sms, c
     net.W = m->width;
     net.D = m->depth;
     if (SYSTEM)  // inside an MD step: may start while the list kernels drain
-        RB_CUDA(launch_pdl(k_nn_f32<W, P, KC, SYSTEM>, num_sms, kF32Threads, smem, stream, net,
-                           src, dst));
+        RB_CUDA(launch_pdl(kern, grid, T, smem, stream, net, src, dst));
     else
-        k_nn_f32<W, P, KC, SYSTEM><<<num_sms, kF32Threads, smem, stream>>>(net, src, dst);
+        kern<<<grid, T, smem, stream>>>(net, src, dst);
     RB_CUDA(cudaGetLastError());
     return RB_OK;
 }
 
-// Widest weight chunk (32 KB) whose shared-memory footprint fits the depth,
-// else 16 KB chunks.
-template <int W, int P, int KC_BIG, int KC_SMALL, bool SYSTEM>
-static rb_status launch_f32_fit(const rb_mlp* m, cudaStream_t stream, int num_sms,
-                                const PairSrc& src, const PairDst& dst) {
-    if (f32_smem_bytes<W, P, KC_BIG>(m->depth) <= kSmemMax)
-        return launch_f32<W, P, KC_BIG, SYSTEM>(m, stream, num_sms, src, dst);
-    return launch_f32<W, P, KC_SMALL, SYSTEM>(m, stream, num_sms, src, dst);
+// Width 128: tiles of 64 pairs, one CTA per SM, or of 32 pairs, three CTAs of
+// 128 threads per SM (the same sums in the same order).  In steady state the
+// larger tiles are a little faster (200000 pairs: 594 against 638 us), but they
+// end in a round that may be almost empty.  In units of a round of 64-pair
+// tiles (28 us at depth 3) a full round of three 32-pair tiles per SM measures
+// 1.62 and a last one of at most half as many 1.02, so the smaller tiles are
+// taken where that sum is below the rounds of the larger: 10000 pairs 58.6 ->
+// 47.9 us, 20000 86.8 -> 76.8, 50003 171.7 -> 161.5; and up to a tile per SM,
+// for the latency of one (30.9 -> 26.7).  Just past each of these lines the
+// larger are faster: 5000 pairs 31.0 against 35.6, 15000 59.2 against 64.4,
+// 24320 87.4 against 93.0.
+static bool small_tiles(int64_t n, int num_sms) {
+    const int64_t t32 = (n + 31) / 32, t64 = (n + 63) / 64;
+    if (t32 <= num_sms) return true;
+    const int64_t full = t32 / (3 * num_sms), rem = t32 % (3 * num_sms);
+    const double last = rem == 0 ? 0.0 : 2 * rem <= 3 * num_sms ? 1.02 : 1.62;
+    return 1.62 * (double)full + last < (double)((t64 + num_sms - 1) / num_sms);
 }
 
 template <bool SYSTEM>
 static rb_status dispatch_f32(const rb_mlp* m, cudaStream_t stream, int num_sms,
                               const PairSrc& src, const PairDst& dst) {
     switch (m->width) {
-        case 64: return launch_f32<64, 128, 64, SYSTEM>(m, stream, num_sms, src, dst);
-        case 128: return launch_f32_fit<128, 64, 64, 32, SYSTEM>(m, stream, num_sms, src, dst);
-        case 256: return launch_f32_fit<256, 32, 32, 16, SYSTEM>(m, stream, num_sms, src, dst);
+        case 64: return launch_f32<64, 128, 64, kF32Threads, 1, SYSTEM>(m, stream, num_sms, src, dst);
+        case 128:
+            if constexpr (!SYSTEM) {  // a system's pair count is not known here
+                if ((m->depth == 2 || m->depth == 3) && small_tiles(src.n_explicit, num_sms))
+                    return launch_f32<128, 32, 16, 128, 3, false>(
+                        m, stream, (int)std::min<int64_t>((src.n_explicit + 31) / 32, (int64_t)3 * num_sms),
+                        src, dst);
+            }
+            return launch_f32<128, 64, 64, kF32Threads, 1, SYSTEM>(m, stream, num_sms, src, dst);
+        case 256: return launch_f32<256, 32, 32, kF32Threads, 1, SYSTEM>(m, stream, num_sms, src, dst);
         default: return fail(RB_ENOTSUP, "FP32 network kernel supports widths 64, 128, 256");
     }
 }

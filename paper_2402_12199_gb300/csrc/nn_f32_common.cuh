@@ -37,7 +37,7 @@ __device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_group 0
 // The weight chunks one tile consumes, in order: layer-1 (16 rows), the
 // forward chunks of W_2..W_D, the reverse chunks of W_D..W_2.  A CTA consumes
 // this sequence once per tile; chunk c lives in buffer c % 2.
-template <int W, int KC>
+template <int W, int KC, int T = kF32Threads>
 struct ChunkFeed {
     static_assert(KC >= kInPad && W % KC == 0, "chunk rows must divide the width");
     static constexpr int NK = W / KC;  // chunks per hidden matrix
@@ -73,7 +73,7 @@ struct ChunkFeed {
         source((int)(cc % n_chunks), p, rows);
         const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(buf + (cc & 1) * KC * W));
         const int pieces = rows * W / 4;
-        for (int t = threadIdx.x; t < pieces; t += kF32Threads) cp_async16(dst + 16u * t, p + 4 * t);
+        for (int t = threadIdx.x; t < pieces; t += T) cp_async16(dst + 16u * t, p + 4 * t);
         cp_async_commit();
     }
     // Wait for chunk c (this thread's copies, then everyone's via the
