@@ -487,37 +487,4 @@ __device__ inline bool bead_pair_cols(const float (&bx)[NS], const float (&by)[N
     return any;
 }
 
-// Smallest squared bead-bead distance between the two bodies (warp min).
-template <int NP>
-__device__ inline float min_dist2_warp(const float3 s, const Mat3& Rr, const float4* sT,
-                                       int n_beads, int lane) {
-    constexpr int MB = 2 * NP;
-    float bx[MB], by[MB], bz[MB];
-#pragma unroll
-    for (int m = 0; m < MB; ++m) {
-        const int l = lane + 32 * m;
-        if (l < n_beads) {
-            const float4 d = sT[l];
-            const float3 b = mul(Rr, make_float3(d.x, d.y, d.z));
-            bx[m] = s.x + b.x;
-            by[m] = s.y + b.y;
-            bz[m] = s.z + b.z;
-        } else {
-            bx[m] = by[m] = bz[m] = 1e18f;
-        }
-    }
-    float mn = 3.0e38f;
-    for (int k = 0; k < n_beads; ++k) {
-        const float4 d = sT[k];
-#pragma unroll
-        for (int m = 0; m < MB; ++m) {
-            const float rx = bx[m] - d.x, ry = by[m] - d.y, rz = bz[m] - d.z;
-            mn = fminf(mn, rx * rx + ry * ry + rz * rz);
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-    return mn;
-}
-
 }  // namespace rb

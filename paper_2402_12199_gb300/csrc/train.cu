@@ -70,24 +70,59 @@ namespace rb {
 //   * those test the listed pairs alone, two per lane, and stop when the middle
 //     no longer differs from an end of the bracket in FP32.
 // A list longer than kCand (parallel faces) is tried again after another
-// halving.  Every halving is decided as the scan of all pairs would decide it
-// (up to FP32 rounding of the distances): the labels' error against FP64 is
-// 5.4e-6 (5.6e-6 with full scans).  The label takes the columns near body j
-// only, as the pair kernel does.  Measured: 8885 -> 333 us for 65536 cube pairs
-// at contact 0.85; bound by instruction issue (about 3500 a sample).
+// halving.  A grazing contact amplifies the last bit of a distance and the
+// label's repulsion that of the separation (by up to 3e-3 of the labels' rms in
+// one element), so every quantity that a halving or a label depends on is
+// rounded as the scan of all pairs rounds it, operation by operation (rotation,
+// place, bead_dist2, bead_terms): separations and labels are those of the full scan,
+// bit for bit.  The label takes the columns near body j only, and of those the
+// beads inside the cutoff; the others would add exact zeros.  Measured: 8885 ->
+// 366 us for 65536 cube pairs at contact 0.85; bound by instruction issue.
 constexpr int kCoarse = 5;
 constexpr int kCand = 64;
 
-// Smallest squared distance between one column of body i (at x, y) and the
-// lane's beads of j, continued from mn.  The x-y part of a bead's squared
-// distance is shared along the column.
+// Squared distance from its components, in the full scan's rounding: the x-y
+// part first, so that it is shared along a column.
+__device__ __forceinline__ float bead_dist2_xy(float rx, float ry) {
+    return __fmaf_rn(rx, rx, __fmul_rn(ry, ry));
+}
+__device__ __forceinline__ float bead_dist2(float rx, float ry, float rz) {
+    return __fmaf_rn(rz, rz, bead_dist2_xy(rx, ry));
+}
+// R(q) (as qmat) with the roundings spelled out: the compiler's choice of which
+// product of a sum is fused differs between instantiations.
+__device__ __forceinline__ Mat3 rotation(const float4& q) {
+    const float w = q.x, x = q.y, y = q.z, z = q.w;
+    const float xx = __fmul_rn(x, x), zz = __fmul_rn(z, z), xz = __fmul_rn(x, z), wz = __fmul_rn(w, z),
+                wx = __fmul_rn(w, x);
+    Mat3 R;
+    R.m[0] = __fmaf_rn(-2.f, __fmaf_rn(y, y, zz), 1.f);
+    R.m[1] = 2.f * __fmaf_rn(x, y, -wz);
+    R.m[2] = 2.f * __fmaf_rn(w, y, xz);
+    R.m[3] = 2.f * __fmaf_rn(x, y, wz);
+    R.m[4] = __fmaf_rn(-2.f, __fmaf_rn(z, z, xx), 1.f);
+    R.m[5] = 2.f * __fmaf_rn(y, z, -wx);
+    R.m[6] = 2.f * __fmaf_rn(-w, y, xz);
+    R.m[7] = 2.f * __fmaf_rn(y, z, wx);
+    R.m[8] = __fmaf_rn(-2.f, __fmaf_rn(y, y, xx), 1.f);
+    return R;
+}
+// R d, the products of each component fused except the second.
+__device__ __forceinline__ float3 rotate_bead(const Mat3& R, const float4& d) {
+    return make_float3(__fmaf_rn(R.m[2], d.z, __fmaf_rn(R.m[0], d.x, __fmul_rn(R.m[1], d.y))),
+                       __fmaf_rn(R.m[5], d.z, __fmaf_rn(R.m[3], d.x, __fmul_rn(R.m[4], d.y))),
+                       __fmaf_rn(R.m[8], d.z, __fmaf_rn(R.m[6], d.x, __fmul_rn(R.m[7], d.y))));
+}
+
+// Smallest squared distance between the beads of one column of body i (at x, y)
+// and the lane's beads of j.
 template <int NP, int C>
 __device__ inline float column_min(float x, float y, const BeadCols& cols, const float (&bx)[2 * NP],
-                                   const float (&by)[2 * NP], const float (&bz)[2 * NP], float mn) {
+                                   const float (&by)[2 * NP], const float (&bz)[2 * NP]) {
+    float mn = 3.0e38f;
 #pragma unroll
     for (int m = 0; m < 2 * NP; ++m) {
-        const float rx = bx[m] - x, ry = by[m] - y;
-        const float p = __fmaf_rn(ry, ry, __fmul_rn(rx, rx));
+        const float p = bead_dist2_xy(bx[m] - x, by[m] - y);
 #pragma unroll
         for (int z = 0; z < C; ++z) {
             const float rz = bz[m] - cols.z[z];
@@ -96,17 +131,36 @@ __device__ inline float column_min(float x, float y, const BeadCols& cols, const
     }
     return mn;
 }
+// The column's beads (bit z) with one of the lane's beads within sqrt(r2).
+template <int NP, int C>
+__device__ inline unsigned column_hits(float x, float y, const BeadCols& cols, const float (&bx)[2 * NP],
+                                       const float (&by)[2 * NP], const float (&bz)[2 * NP], float r2) {
+    float mn[C];
+#pragma unroll
+    for (int z = 0; z < C; ++z) mn[z] = 3.0e38f;
+#pragma unroll
+    for (int m = 0; m < 2 * NP; ++m) {
+        const float p = bead_dist2_xy(bx[m] - x, by[m] - y);
+#pragma unroll
+        for (int z = 0; z < C; ++z) {
+            const float rz = bz[m] - cols.z[z];
+            mn[z] = fminf(mn[z], __fmaf_rn(rz, rz, p));
+        }
+    }
+    unsigned hits = 0u;
+#pragma unroll
+    for (int z = 0; z < C; ++z) hits |= mn[z] < r2 ? 1u << z : 0u;
+    return hits;
+}
 
 template <int NP, int C, int POT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, NP <= 3 || C == 0 ? 2 : 1)
     k_sample_pairs(int64_t n, const float* __restrict__ u, const float4* __restrict__ tmpl,
                    int n_beads, BeadCols cols, float r_circ, float Rc, float contact, BeadPot pot,
                    float4* __restrict__ cfg, float4* __restrict__ lab, float* __restrict__ rho_c) {
     constexpr int MB = 2 * NP;
     __shared__ float4 sT[kMaxBeads + 1];
-    // any template: its distance-test form; columns: per warp the packed beads of j
-    constexpr int kSN = C == 0 ? 2 * (kMaxBeads + kPadBeads) : 8 * 32 * MB;
-    __shared__ float4 sN[kSN];
+    __shared__ float4 sN[C == 0 ? 2 * (kMaxBeads + kPadBeads) : 1];  // any template: its distance-test form
     __shared__ ColShared sc;
     __shared__ unsigned short s_cand[8][kCand];  // bead of i << 8 | bead of j
     if (C == 0) {
@@ -120,6 +174,8 @@ __global__ void __launch_bounds__(256)
     const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     const float sig2 = contact * contact;
+    // what rounding can take from a listed pair's distance
+    const float slack = 1e-3f + 4e-6f * (Rc + contact);
     unsigned short* cand = s_cand[warp];
     for (int64_t b = gw; b < n; b += nw) {
         const float* ub = u + 6 * b;
@@ -133,25 +189,27 @@ __global__ void __launch_bounds__(256)
         sincospif(2.f * ub[4], &s4, &c4);
         const float a = sqrtf(1.f - ub[2]), bq = sqrtf(ub[2]);
         const float4 q = make_float4(a * s3, a * c3, bq * s4, bq * c4);
-        const Mat3 Rr = qmat(q);
+        const Mat3 Rr = rotation(q);
         float px[MB], py[MB], pz[MB];  // R d_l of the lane's beads l = lane + 32 m
 #pragma unroll
         for (int m = 0; m < MB; ++m) {
             const int l = lane + 32 * m;
-            const float4 d = sT[min(l, n_beads - 1)];
-            const float3 r = mul(Rr, make_float3(d.x, d.y, d.z));
+            const float3 r = rotate_bead(Rr, sT[min(l, n_beads - 1)]);
             px[m] = l < n_beads ? r.x : 1e18f;
             py[m] = l < n_beads ? r.y : 1e18f;
             pz[m] = l < n_beads ? r.z : 1e18f;
         }
         float bx[MB], by[MB], bz[MB];
+        auto centre = [&](float rho) {
+            return make_float3(__fmul_rn(rho, dir.x), __fmul_rn(rho, dir.y), __fmul_rn(rho, dir.z));
+        };
         auto place = [&](float rho) {  // the lane's beads with j's centre at rho dir
-            const float3 s = make_float3(rho * dir.x, rho * dir.y, rho * dir.z);
+            const float3 s = centre(rho);
 #pragma unroll
             for (int m = 0; m < MB; ++m) {
-                bx[m] = s.x + px[m];
-                by[m] = s.y + py[m];
-                bz[m] = s.z + pz[m];
+                bx[m] = __fadd_rn(s.x, px[m]);
+                by[m] = __fadd_rn(s.y, py[m]);
+                bz[m] = __fadd_rn(s.z, pz[m]);
             }
             return s;
         };
@@ -176,12 +234,18 @@ __global__ void __launch_bounds__(256)
                     while (near[wd]) {
                         const int c = 32 * wd + __ffs(near[wd]) - 1;
                         near[wd] &= near[wd] - 1u;
-                        const float mn = column_min<NP, C>(sc.xy[c].x, sc.xy[c].y, cols, bx, by, bz, 3.0e38f);
+                        const float mn = column_min<NP, C>(sc.xy[c].x, sc.xy[c].y, cols, bx, by, bz);
                         if (__any_sync(0xffffffffu, mn < sig2)) return true;
                     }
                 return false;
             } else {
-                return min_dist2_warp<NP>(s, Rr, sT, n_beads, lane) < sig2;
+                float mn = 3.0e38f;
+                for (int k = 0; k < n_beads; ++k) {
+                    const float4 d = sT[k];
+#pragma unroll
+                    for (int m = 0; m < MB; ++m) mn = fminf(mn, bead_dist2(bx[m] - d.x, by[m] - d.y, bz[m] - d.z));
+                }
+                return __any_sync(0xffffffffu, mn < sig2) != 0;
             }
         };
         // bead pairs closer than `reach` with j's centre at rho: their number,
@@ -193,8 +257,7 @@ __global__ void __launch_bounds__(256)
             auto test = [&](int k, float x, float y, float zz) {
 #pragma unroll
                 for (int m = 0; m < MB; ++m) {
-                    const float rx = bx[m] - x, ry = by[m] - y, rz = bz[m] - zz;
-                    const bool hit = __fmaf_rn(rz, rz, __fmaf_rn(ry, ry, __fmul_rn(rx, rx))) < r2;
+                    const bool hit = bead_dist2(bx[m] - x, by[m] - y, bz[m] - zz) < r2;
                     const unsigned w = __ballot_sync(0xffffffffu, hit);
                     if (w) {
                         const int at = nc + __popc(w & ((1u << lane) - 1u));
@@ -211,7 +274,7 @@ __global__ void __launch_bounds__(256)
                         const int c = 32 * wd + __ffs(near[wd]) - 1;
                         near[wd] &= near[wd] - 1u;
                         const float x = sc.xy[c].x, y = sc.xy[c].y;
-                        const float mn = column_min<NP, C>(x, y, cols, bx, by, bz, 3.0e38f);
+                        const float mn = column_min<NP, C>(x, y, cols, bx, by, bz);
                         if (!__any_sync(0xffffffffu, mn < r2)) continue;
                         for (int k = 0; k < C; ++k) test(C * c + k, x, y, cols.z[k]);
                     }
@@ -233,14 +296,13 @@ __global__ void __launch_bounds__(256)
             const float mid = 0.5f * (lo + hi);
             if (lo > 0.f && hi < Rc && (mid <= lo || mid >= hi)) break;  // both ends tested: settled
             if (nc > kCand && it >= kCoarse) {
-                nc = list_pairs(mid, contact + 0.5f * (hi - lo) + 1e-3f);
+                nc = list_pairs(mid, contact + 0.5f * (hi - lo) + slack);
                 if (nc <= kCand) {
                     auto entry = [&](int e, float3& o, float3& d) {
                         if (e >= nc) return;
                         const int k = cand[e] >> 8, l = cand[e] & 0xFF;
-                        const float4 tl = sT[l], tk = sT[k];
-                        o = mul(Rr, make_float3(tl.x, tl.y, tl.z));
-                        d = make_float3(tk.x, tk.y, tk.z);
+                        o = rotate_bead(Rr, sT[l]);
+                        d = xyz(sT[k]);
                     };
                     entry(lane, o0, d0);
                     entry(lane + 32, o1, d1);
@@ -249,10 +311,9 @@ __global__ void __launch_bounds__(256)
             }
             bool hit;
             if (nc <= kCand) {
-                const float3 s = make_float3(mid * dir.x, mid * dir.y, mid * dir.z);
+                const float3 s = centre(mid);
                 auto dist2 = [&](const float3& o, const float3& d) {
-                    const float rx = (s.x + o.x) - d.x, ry = (s.y + o.y) - d.y, rz = (s.z + o.z) - d.z;
-                    return __fmaf_rn(rz, rz, __fmaf_rn(ry, ry, __fmul_rn(rx, rx)));
+                    return bead_dist2(__fadd_rn(s.x, o.x) - d.x, __fadd_rn(s.y, o.y) - d.y, __fadd_rn(s.z, o.z) - d.z);
                 };
                 hit = __any_sync(0xffffffffu, fminf(dist2(o0, d0), dist2(o1, d1)) < sig2);
             } else {
@@ -265,16 +326,38 @@ __global__ void __launch_bounds__(256)
         }
         const float rc = 0.5f * (lo + hi);
         const float rho = rc + ub[5] * (Rc - rc);
-        const float3 s = make_float3(rho * dir.x, rho * dir.y, rho * dir.z);
+        const float3 s = centre(rho);
         float v[7];
         if constexpr (C > 0) {
             place(rho);
-            float w[7];
-            float t = 0.f;
-            if (bead_pair_cols<MB, C, POT>(bx, by, bz, sc, cols, pot, sN + 32 * MB * warp, lane, w))
-                t = warp_scatter7(w);
+            float2 Bx[NP], By[NP], Bz[NP];
 #pragma unroll
-            for (int k = 0; k < 7; ++k) v[k] = __shfl_sync(0xffffffffu, t, 4 * k);
+            for (int p = 0; p < NP; ++p) {
+                Bx[p] = make_float2(bx[2 * p], bx[2 * p + 1]);
+                By[p] = make_float2(by[2 * p], by[2 * p + 1]);
+                Bz[p] = make_float2(bz[2 * p], bz[2 * p + 1]);
+            }
+            LJAcc<NP> acc;
+            acc.zero();
+#pragma unroll
+            for (int wd = 0; wd < kColWords; ++wd) {
+                if (32 * wd >= cols.n_cols) break;
+                unsigned near = __ballot_sync(0xffffffffu, column_near<C>(s, sc, cols, 32 * wd + lane, pot.cull2));
+                while (near) {
+                    const int c = 32 * wd + __ffs(near) - 1;
+                    near &= near - 1u;
+                    const float x = sc.xy[c].x, y = sc.xy[c].y;
+                    unsigned hits = __reduce_or_sync(0xffffffffu,
+                                                     column_hits<NP, C>(x, y, cols, bx, by, bz, pot.rc2_test));
+                    while (hits) {
+                        const float mz = -2.f * sc.z[__ffs(hits) - 1];
+                        hits &= hits - 1u;
+                        bead_terms<NP, POT>(make_float2(-2.f * x, -2.f * x), make_float2(-2.f * y, -2.f * y),
+                                            make_float2(mz, mz), Bx, By, Bz, pot, acc);
+                    }
+                }
+            }
+            warp_finish<NP>(bx, by, bz, acc, pot, v);
         } else {
             bead_pair_warp<NP, POT>(s, Rr, sT, sN, n_beads, pot, lane, v);
         }

@@ -1,0 +1,54 @@
+"""Sampled pairs against recorded ones, bit for bit: draws (some at grazing contacts, where the last
+bit of a distance moves the separation and a close label by up to 3e-3 of the labels' rms) with the
+separations, configurations and labels that the scan of every bead pair in every halving gives
+(golden/sampled_pairs.json, hexadecimal FP32).  The half-power half-cosine's labels go through
+hardware approximations whose argument the compiler may round differently: within 1e-5 of their rms."""
+import json
+import os
+
+import numpy as np
+import pytest
+
+from tests.test_gpu_templates import _grid
+
+pytestmark = pytest.mark.gpu
+
+with open(os.path.join(os.path.dirname(__file__), "golden", "sampled_pairs.json")) as f:
+    GOLDEN = json.load(f)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+
+    __graft_entry__.build()
+
+
+def _floats(rows):
+    return np.array([[int(w, 16) for w in r.split()] for r in rows], np.uint32).view(np.float32)
+
+
+@pytest.mark.parametrize("g", GOLDEN, ids=lambda g: f"{g['shape']}-{g['grid']}-{g['potential']}")
+def test_sampled_pairs_are_the_recorded_ones(g):
+    import torch
+
+    from paper_2402_12199_gb300 import api
+
+    kw = {}
+    if g["grid"]:
+        kw["template"] = _grid(g["grid"])
+    if g["potential"] == "hphc":
+        kw.update(potential="hphc", hphc=g["hphc"])
+    s = api.System(8, [80.0] * 3, g["shape"], **kw)
+    u = torch.from_numpy(_floats(g["uniforms"])).cuda()
+    cfg, lab, rc = (x.cpu().numpy() for x in api.sample_pairs(s, u, g["contact"]))
+    assert rc.view(np.uint32).tolist() == _floats(g["rho_contact"]).view(np.uint32).ravel().tolist()
+    assert cfg.view(np.uint32).tolist() == _floats(g["cfg"]).view(np.uint32).tolist()
+    want = _floats(g["labels"])
+    if g["potential"] == "lj":
+        assert lab.view(np.uint32).tolist() == want.view(np.uint32).tolist()
+    else:
+        assert np.abs(lab - want).max() <= 1e-5 * np.sqrt((want.astype(np.float64) ** 2).mean())
