@@ -340,11 +340,6 @@ __device__ __forceinline__ void pair_build_body(
             s_nslow = 0;
         }
         __syncthreads();
-        // a block whose surroundings do not cross a face of the box (and a box
-        // of at least four cells a side, so that two cells span less than half
-        // of it) needs no minimum image: the image shift would be an exact zero
-        const bool wrap = b0.x == 0 || b0.y == 0 || b0.z == 0 || b0.x + w.x == nc.x || b0.y + w.y == nc.y ||
-                          b0.z + w.z == nc.z || min(min(nc.x, nc.y), nc.z) < 4;
         auto row_warp = [&](int i) {
             pair_row_warp(i, pos, L, invL, invw, nc, count, bodies, cap, Rc2, max_nbr, half_count, nbr,
                           lower_count, lower_pair, seg_sum, status);
@@ -358,6 +353,7 @@ __device__ __forceinline__ void pair_build_body(
             __syncthreads();
             continue;
         }
+        bool out = false;  // a centre stored outside [0, L): any image of a position is valid
         for (int c = tid; c < kHalo; c += 256) {
             const int st = s_start[c], n = s_start[c + 1] - st;
             if (n == 0) continue;
@@ -374,13 +370,20 @@ __device__ __forceinline__ void pair_build_body(
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     if (s + u >= n) break;
+                    out |= !(q[u].x >= 0.f && q[u].x < L.x && q[u].y >= 0.f && q[u].y < L.y && q[u].z >= 0.f &&
+                             q[u].z < L.z);
                     q[u].w = __int_as_float(j[u]);
                     s_body[st + s + u] = q[u];
                     if (own) s_list[at + s + u] = c << 16 | (st + s + u);
                 }
             }
         }
-        __syncthreads();
+        // A block whose surroundings do not cross a face of the box (nor span half
+        // of it: at least four cells a side), with every centre stored in [0, L),
+        // needs no minimum image: the image shift would be an exact zero.
+        const bool face = b0.x == 0 || b0.y == 0 || b0.z == 0 || b0.x + w.x == nc.x || b0.y + w.y == nc.y ||
+                          b0.z + w.z == nc.z || min(min(nc.x, nc.y), nc.z) < 4;
+        const bool wrap = __syncthreads_or(out) != 0 || face;
         // stencil offsets as in pair_row_warp: a side of two cells has them
         // once each, a side of one only the cell itself
         const int xl = nc.x >= 3 ? -1 : 0, xh = nc.x >= 2 ? 1 : 0;
