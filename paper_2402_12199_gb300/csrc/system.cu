@@ -142,7 +142,8 @@ __device__ __forceinline__ void cell_assign_body(const float4* __restrict__ pos,
                                                  int* __restrict__ count, int* __restrict__ bodies,
                                                  int cap, unsigned* status, int* rebuild,
                                                  int* zero_count, int* __restrict__ seg_sum,
-                                                 int force, int bid) {
+                                                 int* __restrict__ half_count,
+                                                 int* __restrict__ lower_count, int force, int bid) {
     pdl_chain();
     if (zero_count && bid == 0 && threadIdx.x == 0) *zero_count = 0;
     if (force) {
@@ -160,18 +161,21 @@ __device__ __forceinline__ void cell_assign_body(const float4* __restrict__ pos,
     int cz = min(max(int(z * invw.z), 0), nc.z - 1);
     int c = (cz * nc.y + cy) * nc.x + cx;
     int slot = atomicAdd(&count[c], 1);
-    if (slot < cap)
+    if (slot < cap) {
         bodies[c * cap + slot] = i;
-    else
+    } else {  // in no cell's list: k_pair_build visits it for nobody, so its row is emptied here
+        half_count[i] = lower_count[i] = 0;
         atomicOr(status, ST_CELL_OVERFLOW);
+    }
 }
 
 __global__ void k_cell_assign(const float4* __restrict__ pos, int N, float3 L, float3 invL,
                               float3 invw, int3 nc, int* __restrict__ count,
                               int* __restrict__ bodies, int cap, unsigned* status, int* rebuild,
-                              int* zero_count, int* __restrict__ seg_sum, int force) {
+                              int* zero_count, int* __restrict__ seg_sum, int* __restrict__ half_count,
+                              int* __restrict__ lower_count, int force) {
     cell_assign_body(pos, N, L, invL, invw, nc, count, bodies, cap, status, rebuild, zero_count,
-                     seg_sum, force, blockIdx.x);
+                     seg_sum, half_count, lower_count, force, blockIdx.x);
 }
 
 __device__ inline void sort_row(int* row, int n) {
@@ -1007,7 +1011,8 @@ __global__ void k_cell_assign_batch(const StepSeg* __restrict__ segs, const int*
     const int k = seg_of_block(start, n_seg, blockIdx.x);
     const StepSeg& S = segs[k];
     cell_assign_body(S.pos, S.N, S.L, S.invL, S.invw, S.nc, S.cell_count, S.cell_bodies, S.cell_cap,
-                     S.status, S.rebuild, S.zero_count, S.seg, 0, blockIdx.x - start[k]);
+                     S.status, S.rebuild, S.zero_count, S.seg, S.half_count, S.lower_count, 0,
+                     blockIdx.x - start[k]);
 }
 
 __global__ void __launch_bounds__(256, kBuildCtas) k_pair_build_batch(const StepSeg* __restrict__ segs, const int* __restrict__ start,
@@ -1062,7 +1067,8 @@ rb_status build_pairs_async(rb_system* s, bool force, bool checked, int* zero_co
     }
     RB_CUDA(launch_pdl(k_cell_assign, blocks_for(N, 256), 256, 0, s->stream, s->pos, N, L, invL,
                        invw, nc, s->cells.count, s->cells.bodies, s->cells.cap, s->status_dev,
-                       s->rebuild_flag, zero_count, s->pl.seg, force ? 1 : 0));
+                       s->rebuild_flag, zero_count, s->pl.seg, s->pl.half_count, s->pl.lower_count,
+                       force ? 1 : 0));
     s->fb_zeroed = zero_count != nullptr;
     int* seg_base = s->pl.seg + pair_segments(N);
     RB_CUDA(launch_pdl(k_pair_build, std::min(cell_blocks(nc), s->num_sms * kBuildCtas), 256, 0, s->stream,
