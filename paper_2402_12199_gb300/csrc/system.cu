@@ -14,6 +14,8 @@
 #include <functional>
 #include <new>
 
+#include <cuda.h>
+
 #include "rb_internal.cuh"
 
 namespace rb {
@@ -2009,19 +2011,34 @@ static rb_status read_energy(rb_system* s, double* energy, double* virial9) {
     return RB_OK;
 }
 
-// The caller's force or torque rows if the reduction can write them itself
-// (float4 stores), else null; finish_forces copies what it could not.
-static float* direct_rows(float* p) {
-    return (reinterpret_cast<uintptr_t>(p) & 15) == 0 ? p : nullptr;
+// The caller's force or torque rows if the reduction can write them itself: on a
+// 16-byte boundary (float4 stores) and inside one allocation of this device.
+// Else null: a copy writes them, which also reaches memory that the kernel could
+// not (another device's, managed, host) and refuses what is no such memory.
+static float* direct_rows(const rb_system* s, float* p) {
+    if (!p || (reinterpret_cast<uintptr_t>(p) & 15) != 0) return nullptr;
+    unsigned type = 0;
+    int managed = 0, device = -1;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    CUpointer_attribute which[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                   CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                   CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* out[] = {&type, &managed, &device, &start, &size};
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    if (cuPointerGetAttributes(5, which, out, at) != CUDA_SUCCESS) return nullptr;
+    return type == CU_MEMORYTYPE_DEVICE && !managed && device == s->device && at >= start &&
+                   at - start + sizeof(float4) * (size_t)s->N <= size
+               ? p
+               : nullptr;
 }
 
+// Rows that the reduction has not written (null: written, or not asked for).
 static rb_status finish_forces(rb_system* s, float* force, float* torque, double* energy,
                                double* virial9) {
     const size_t b = sizeof(float4) * s->N;
-    if (force && !direct_rows(force))
-        RB_CUDA(cudaMemcpyAsync(force, s->force, b, cudaMemcpyDeviceToDevice, s->stream));
-    if (torque && !direct_rows(torque))
-        RB_CUDA(cudaMemcpyAsync(torque, s->torque, b, cudaMemcpyDeviceToDevice, s->stream));
+    if (force) RB_CUDA(cudaMemcpyAsync(force, s->force, b, cudaMemcpyDeviceToDevice, s->stream));
+    if (torque) RB_CUDA(cudaMemcpyAsync(torque, s->torque, b, cudaMemcpyDeviceToDevice, s->stream));
     if (energy || virial9) RB_TRY(read_energy(s, energy, virial9));
     return RB_OK;
 }
@@ -2031,12 +2048,13 @@ rb_status rb_forces_beads(rb_system* s, float* force, float* torque, double* ene
     if (!s) return fail(RB_EINVAL, "null system");
     RB_TRY(build_pairs_async(s, false, false));
     RB_TRY(bead_pairs_async(s));
-    RB_TRY(reduce_forces_async(s, 0.f, nullptr, direct_rows(force), direct_rows(torque)));
+    float *df = direct_rows(s, force), *dt = direct_rows(s, torque);
+    RB_TRY(reduce_forces_async(s, 0.f, nullptr, df, dt));
     s->forces_valid = true;
     s->forces_path = RB_PATH_BEADS;
     s->forces_precision = RB_FP32;
     s->forces_mlp = nullptr;
-    return finish_forces(s, force, torque, energy, virial9);
+    return finish_forces(s, df ? nullptr : force, dt ? nullptr : torque, energy, virial9);
 }
 
 rb_status rb_forces_nn(rb_system* s, const rb_mlp* m, int32_t precision, float* force,
@@ -2047,13 +2065,14 @@ rb_status rb_forces_nn(rb_system* s, const rb_mlp* m, int32_t precision, float* 
     RB_TRY(build_pairs_async(s, false, false, fallback_counter(s)));
     RB_TRY(nn_pairs_system_async(s, m, precision));
     RB_TRY(bead_fallback_async(s));
-    RB_TRY(reduce_forces_async(s, 0.f, nullptr, direct_rows(force), direct_rows(torque)));
+    float *df = direct_rows(s, force), *dt = direct_rows(s, torque);
+    RB_TRY(reduce_forces_async(s, 0.f, nullptr, df, dt));
     s->forces_valid = true;
     s->forces_path = RB_PATH_NN;
     s->forces_precision = precision;
     s->forces_mlp = m;
     s->forces_mlp_version = m->version;
-    return finish_forces(s, force, torque, energy, virial9);
+    return finish_forces(s, df ? nullptr : force, dt ? nullptr : torque, energy, virial9);
 }
 
 // model: the rb_mlp of RB_PATH_NN or the rb_fnet of RB_PATH_FNET (unused for beads)
@@ -2190,13 +2209,14 @@ rb_status rb_forces_fnet(rb_system* s, const rb_fnet* f, float* force, float* to
     RB_TRY(fnet_ready(f));
     RB_TRY(build_pairs_async(s, false, false));
     RB_TRY(fnet_pairs_system_async(s, f));
-    RB_TRY(reduce_forces_async(s, 0.f, nullptr, direct_rows(force), direct_rows(torque)));
+    float *df = direct_rows(s, force), *dt = direct_rows(s, torque);
+    RB_TRY(reduce_forces_async(s, 0.f, nullptr, df, dt));
     s->forces_valid = true;
     s->forces_path = RB_PATH_FNET;
     s->forces_precision = RB_FP32;
     s->forces_mlp = f;
     s->forces_mlp_version = fnet_version(f);
-    return finish_forces(s, force, torque, nullptr, virial9);
+    return finish_forces(s, df ? nullptr : force, dt ? nullptr : torque, nullptr, virial9);
 }
 
 rb_status rb_set_skin(rb_system* s, float skin) {
