@@ -157,10 +157,14 @@ __device__ inline FnFrame fn_frame(const float3 s, const float4 q) {
     return f;
 }
 
-// SiLU of two pre-activations: z / (1 + 2^(-z log2 e)) with the hardware base-2
-// exponential and reciprocal (the exponential of expf's fast form; the IEEE
-// division after it, a third of the kernel's instructions, gained no accuracy:
-// the exponential's rounding is the larger).
+// SiLU of two pre-activations, z sigma(z) with sigma(z) = 1 / (1 + 2^(-z log2 e))
+// (e^-z written with base 2), by the hardware base-2 exponential and reciprocal,
+// which flush what is below 2^-126: for z < -88 the exponential or the
+// reciprocal saturates and the result is -0 instead of some -1e-36, for z > 88
+// it is z.  An IEEE division in the place of the reciprocal was a third of the
+// kernel's instructions and gained no accuracy (error against FP64 of the forces
+// of 30000 cylinders 1.5e-6 both ways); __expf and __fdividef, which treat
+// subnormals, give the same accuracy at 68 us a step instead of 61.
 __device__ __forceinline__ float2 fn_silu2(float2 z) {
     constexpr float kLog2e = 1.4426950408889634f;
     const float2 t = __fmul2_rn(z, make_float2(-kLog2e, -kLog2e));
