@@ -117,9 +117,10 @@ __device__ inline int block_scan256(int v, int& total) {
 // First pair index of every segment of kSegBodies bodies, by one CTA (the last
 // of k_pair_build): the exclusive scan of the segments' pair counts, 256 at a
 // time.  Only for very large systems (kScanSegments): below, every CTA of
-// k_pair_emit adds up the segments before its own, which is off the critical
-// path of the build (at 524288 bodies the scan of 4096 sums by one CTA took
-// about 20 us; reading them costs each emitting CTA 16 loads a thread at most).
+// k_pair_emit adds up the segments before its own in each of its passes, which
+// is off the critical path of the build (at 524288 bodies the scan of 4096 sums
+// by one CTA took about 20 us; reading them is at most 16 loads a thread and
+// pass, and 64 at the limit of 16384 segments, where a CTA takes 13 passes).
 constexpr int kScanSegments = 16384;
 __device__ inline void scan_segments(const int* __restrict__ seg_sum, int* __restrict__ seg_base, int N) {
     const int S = pair_segments(N);
@@ -280,8 +281,8 @@ __device__ __noinline__ void pair_row_warp(int i, const float4* __restrict__ pos
 // chain of three L2 latencies per block; a warp per body had that chain (two
 // loads deep) once per occupied stencil slot, and sorted its rows in global
 // memory.  The whole build
-// (cell assignment, rows, offsets and emission, back to back): 1407 -> 244 us for
-// 524288 cubes, 111 -> 40 us for 32768 cylinders, 66 -> 35 us for 20011 cubes.
+// (cell assignment, rows, offsets and emission, back to back): 1407 -> 246 us for
+// 524288 cubes, 111 -> 41 us for 32768 cylinders, 66 -> 36 us for 20011 cubes.
 constexpr int kBlkX = 8, kBlkY = 4, kBlkZ = 4;
 constexpr int kHaloX = kBlkX + 2, kHaloY = kBlkY + 2, kHaloZ = kBlkZ + 2;
 constexpr int kHalo = kHaloX * kHaloY * kHaloZ;
@@ -376,8 +377,10 @@ __device__ __forceinline__ void pair_build_body(
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     if (s + u >= n) break;
-                    out |= !(q[u].x >= 0.f && q[u].x < L.x && q[u].y >= 0.f && q[u].y < L.y && q[u].z >= 0.f &&
-                             q[u].z < L.z);
+                    // (a negative or NaN coordinate is a larger unsigned number than any L)
+                    out |= __float_as_uint(q[u].x) >= __float_as_uint(L.x) ||
+                           __float_as_uint(q[u].y) >= __float_as_uint(L.y) ||
+                           __float_as_uint(q[u].z) >= __float_as_uint(L.z);
                     q[u].w = __int_as_float(j[u]);
                     s_body[st + s + u] = q[u];
                     if (own) s_list[at + s + u] = c << 16 | (st + s + u);
@@ -462,9 +465,9 @@ __global__ void __launch_bounds__(256, kBuildCtas) k_pair_build(
 // that stands for i (found in j's ascending lower neighbours).  A thread per
 // pair instead of per body keeps the dependent loads of the ~3 pairs of a
 // body in flight together.  Then remember
-// the positions the list was built for and clear the cell counts and the
-// segment sum for the next rebuild.  The CTA that finishes last lowers the
-// rebuild flag (every CTA has read it by then).
+// the positions the list was built for and clear the cell counts for the next
+// rebuild (which clears the segment sums itself, k_cell_assign).  The CTA that
+// finishes last lowers the rebuild flag (every CTA has read it by then).
 __device__ __forceinline__ void pair_emit_body(
     int N, int max_nbr, const int* __restrict__ half_count, const int* __restrict__ nbr,
     int* __restrict__ half_off, const int* __restrict__ lower_count, int* __restrict__ lower_pair,
