@@ -2020,6 +2020,19 @@ static rb_status read_energy(rb_system* s, double* energy, double* virial9) {
 // not (another device's, managed, host) and refuses what is no such memory.
 static float* direct_rows(const rb_system* s, float* p) {
     if (!p || (reinterpret_cast<uintptr_t>(p) & 15) != 0) return nullptr;
+    // looked up, not linked: the library loads where there is no driver
+    using Query = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    static const Query query = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &r) !=
+                cudaSuccess ||
+            r != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Query>(f);
+    }();
     unsigned type = 0;
     int managed = 0, device = -1;
     CUdeviceptr start = 0;
@@ -2029,7 +2042,7 @@ static float* direct_rows(const rb_system* s, float* p) {
                                    CU_POINTER_ATTRIBUTE_RANGE_SIZE};
     void* out[] = {&type, &managed, &device, &start, &size};
     const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
-    if (cuPointerGetAttributes(5, which, out, at) != CUDA_SUCCESS) return nullptr;
+    if (!query || query(5, which, out, at) != CUDA_SUCCESS) return nullptr;
     return type == CU_MEMORYTYPE_DEVICE && !managed && device == s->device && at >= start &&
                    at - start + sizeof(float4) * (size_t)s->N <= size
                ? p
