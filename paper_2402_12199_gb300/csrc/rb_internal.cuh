@@ -152,7 +152,7 @@ struct PairList {
     int* lower_pair = nullptr;  // N x max_nbr: pair index of each lower neighbour
     int* half_off = nullptr;    // N + 1
     int* seg = nullptr;         // pair count, then first pair, of each segment of bodies
-    int* done = nullptr;        // 2 counters of the last-CTA hand-offs of a rebuild (0 between)
+    int* done = nullptr;        // 2 counters of the last-CTA hand-offs of a rebuild, bodies in crowded cells (0 between)
     int2* pairs = nullptr;      // cap_pairs
     int* n_pairs = nullptr;     // device scalar
 };
@@ -381,7 +381,7 @@ struct StepSeg {
     int force_rebuild;  // no skin: every step rebuilds the list
     int* cell_count;
     int* cell_bodies;
-    int cell_cap, n_cells;
+    int cell_cap, n_cells, rows;  // rows: the list's rows by a warp per body
     float Rl2;
     int max_nbr;
     int *half_count, *nbr, *lower_count, *lower_pair, *half_off, *seg, *n_pairs, *done;

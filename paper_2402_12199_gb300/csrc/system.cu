@@ -8,6 +8,7 @@
 // integrator; this one is velocity Verlet with the NO_SQUISH free-rotor split
 // (Miller et al., J. Chem. Phys. 116, 8649 (2002)).
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -140,13 +141,16 @@ __device__ inline void scan_segments(const int* __restrict__ seg_sum, int* __res
 // index among the system's blocks (bid) and their number (nblk): the kernel
 // of one system passes its own grid, the batched kernels a system's share.
 // force: rebuild whatever the flag says (and raise it for the kernels that follow).
+// crowd: counts the bodies that found kCellFew others in their cell (see crowded).
+constexpr int kCellFew = 4;
 __device__ __forceinline__ void cell_assign_body(const float4* __restrict__ pos, int N, float3 L,
                                                  float3 invL, float3 invw, int3 nc,
                                                  int* __restrict__ count, int* __restrict__ bodies,
                                                  int cap, unsigned* status, int* rebuild,
                                                  int* zero_count, int* __restrict__ seg_sum,
                                                  int* __restrict__ half_count,
-                                                 int* __restrict__ lower_count, int force, int bid) {
+                                                 int* __restrict__ lower_count, int* crowd, int force,
+                                                 int bid) {
     pdl_chain();
     if (zero_count && bid == 0 && threadIdx.x == 0) *zero_count = 0;
     if (force) {
@@ -170,27 +174,17 @@ __device__ __forceinline__ void cell_assign_body(const float4* __restrict__ pos,
         half_count[i] = lower_count[i] = 0;
         atomicOr(status, ST_CELL_OVERFLOW);
     }
+    const unsigned live = __activemask(), many = __ballot_sync(live, slot >= kCellFew);
+    if (many && (threadIdx.x & 31) == __ffs(many) - 1) atomicAdd(crowd, __popc(many));
 }
 
 __global__ void k_cell_assign(const float4* __restrict__ pos, int N, float3 L, float3 invL,
                               float3 invw, int3 nc, int* __restrict__ count,
                               int* __restrict__ bodies, int cap, unsigned* status, int* rebuild,
                               int* zero_count, int* __restrict__ seg_sum, int* __restrict__ half_count,
-                              int* __restrict__ lower_count, int force) {
+                              int* __restrict__ lower_count, int* crowd, int force) {
     cell_assign_body(pos, N, L, invL, invw, nc, count, bodies, cap, status, rebuild, zero_count,
-                     seg_sum, half_count, lower_count, force, blockIdx.x);
-}
-
-__device__ inline void sort_row(int* row, int n) {
-    for (int a = 1; a < n; ++a) {
-        int v = row[a];
-        int b = a - 1;
-        while (b >= 0 && row[b] > v) {
-            row[b + 1] = row[b];
-            --b;
-        }
-        row[b + 1] = v;
-    }
+                     seg_sum, half_count, lower_count, crowd, force, blockIdx.x);
 }
 
 // Neighbour rows.  Row i of `nbr` holds every neighbour of body i (minimum-
@@ -203,10 +197,11 @@ __device__ inline void sort_row(int* row, int n) {
 // The row of body i by one warp, for any number of neighbours: lane c < 27
 // scans one cell of the 3x3x3 stencil (lanes whose cell repeats another's,
 // when a box side holds fewer than 3 cells, stay idle), hits are appended with
-// warp ballots and lane 0 sorts the row.  The block form below sends here the
-// bodies with more neighbours than its shared rows hold and the blocks whose
-// bodies do not fit its shared memory.
-__device__ __noinline__ void pair_row_warp(int i, const float4* __restrict__ pos, float3 L, float3 invL,
+// warp ballots and written to their ranks (compared 32 at a time by shuffles; a
+// sort by one lane was most of a long row's time).  k_pair_rows builds all rows
+// so; the block form below sends here the bodies with more neighbours than its
+// shared rows hold and the blocks whose bodies do not fit its shared memory.
+__device__ __forceinline__ void row_by_warp(int i, const float4* __restrict__ pos, float3 L, float3 invL,
                                            float3 invw, int3 nc, const int* __restrict__ count,
                                            const int* __restrict__ bodies, int cap, float Rc2,
                                            int max_nbr, int* __restrict__ half_count,
@@ -232,6 +227,7 @@ __device__ __noinline__ void pair_row_warp(int i, const float4* __restrict__ pos
     int nmax = n;
     for (int o = 16; o > 0; o >>= 1) nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
     int* row = nbr + (size_t)i * max_nbr;
+    int* found = lower_pair + (size_t)i * max_nbr;  // in the order found, before its own use
     int m = 0;
     const unsigned lt = (1u << lane) - 1u;
     const int* cb = bodies + (size_t)cell * cap;
@@ -249,24 +245,45 @@ __device__ __noinline__ void pair_row_warp(int i, const float4* __restrict__ pos
         const unsigned b = __ballot_sync(0xffffffffu, hit);
         if (hit) {
             const int k = m + __popc(b & lt);
-            if (k < max_nbr) row[k] = j;
+            if (k < max_nbr) found[k] = j;
         }
         m += __popc(b);
     }
+    if (m > max_nbr) {
+        if (lane == 0) atomicOr(status, ST_NBR_OVERFLOW);
+        m = max_nbr;
+    }
     __syncwarp();
-    if (lane == 0) {
-        if (m > max_nbr) {
-            atomicOr(status, ST_NBR_OVERFLOW);
-            m = max_nbr;
+    int nl = 0;
+    for (int a = 0; a < m; a += 32) {  // each entry to its rank
+        const int v = a + lane < m ? found[a + lane] : INT_MAX;
+        int rank = 0;
+        for (int c = 0; c < m; c += 32) {
+            const int w = c + lane < m ? found[c + lane] : INT_MAX;
+#pragma unroll
+            for (int t = 0; t < 32; ++t) rank += __shfl_sync(0xffffffffu, w, t) < v ? 1 : 0;
         }
-        sort_row(row, m);
-        int nl = 0;
-        for (int k = 0; k < m; ++k)
-            if (row[k] < i) lower_pair[(size_t)i * max_nbr + nl++] = -1;
+        if (a + lane < m) row[rank] = v;
+        nl += __popc(__ballot_sync(0xffffffffu, v < i));
+    }
+    __syncwarp();
+    for (int a = lane; a < nl; a += 32) found[a] = -1;
+    if (lane == 0) {
         lower_count[i] = nl;
         half_count[i] = m - nl;
         atomicAdd(seg_sum + i / kSegBodies, m - nl);
     }
+}
+
+__device__ __noinline__ void pair_row_warp(int i, const float4* __restrict__ pos, float3 L, float3 invL,
+                                           float3 invw, int3 nc, const int* __restrict__ count,
+                                           const int* __restrict__ bodies, int cap, float Rc2,
+                                           int max_nbr, int* __restrict__ half_count,
+                                           int* __restrict__ nbr, int* __restrict__ lower_count,
+                                           int* __restrict__ lower_pair, int* __restrict__ seg_sum,
+                                           unsigned* status) {
+    row_by_warp(i, pos, L, invL, invw, nc, count, bodies, cap, Rc2, max_nbr, half_count, nbr, lower_count,
+                lower_pair, seg_sum, status);
 }
 
 // Pair rows, a block of kBlkX x kBlkY x kBlkZ cells per CTA: the bodies of the
@@ -289,17 +306,40 @@ constexpr int kHalo = kHaloX * kHaloY * kHaloZ;
 constexpr int kBlkCap = 1024;  // bodies of a block and its surroundings in shared memory
 constexpr int kRowCap = 16;    // neighbours per shared row
 constexpr int kBuildCtas = 4;  // CTAs per SM: one wave of the grid-stride loop over blocks
+constexpr int kRowCtas = 8;    // and of the loop over bodies
 
 __host__ __device__ inline int cell_blocks(int3 nc) {
     return ((nc.x + kBlkX - 1) / kBlkX) * ((nc.y + kBlkY - 1) / kBlkY) * ((nc.z + kBlkZ - 1) / kBlkZ);
 }
+// The two forms of the row build, by size and mean bodies per cell (N / cells),
+// whole list build in us, rows by warps / by blocks of cells, of bodies on a
+// jittered lattice | at random:
+//   4000 bodies     0.3: 14/19|14/22   1: 19/31|20/34    2.2: 27/58|29/76    6: 50/53|57/64
+//   20011           0.3: 22/23|23/26   1: 30/36|32/45    2.2: 47/77|48/89    6: 97/165|88/195
+//   32768           0.3: 27/30|30/36   1: 38/29|46/40    2.2: 61/77|65/101   6: 121/209|118/230
+//   262144          0.3: 119/155|155/211  1: 164/98|208/139  2.2: 251/158|270/198  6: 430/889|450/1041
+// A small system has too few blocks to hide their latency; cells with less than
+// half a body make a block's halo mostly empty; and where rows outgrow a block's
+// shared rows (a body with more than kRowCap neighbours) or its cells its shared
+// memory, the block falls back to warps with eight of them per CTA (9.9 ms for 32768
+// bodies with 100 neighbours each; 0.6 ms a warp per body): at 524288 bodies the
+// forms are even at 2.6 bodies a cell, at 32768 already at 1.8.
+constexpr float kDense = 2.4f;
+static bool dense_cells(int N, int3 nc) { return (float)N > kDense * (float)nc.x * (float)nc.y * (float)nc.z; }
+static bool rows_by_warps(int N, int3 nc) {
+    return N < 24000 || dense_cells(N, nc) || (float)N < 0.4f * (float)nc.x * (float)nc.y * (float)nc.z;
+}
+// Bodies beyond the kCellFew-th of their cell, counted by the cell assignment: a
+// tenth of all (random positions: at 2.9 a cell) are a system crowded in a part of
+// its box, whatever its mean; k_pair_build then takes the rows by warps itself.
+__device__ inline bool crowded(int N, int crowd) { return crowd > N / 10; }
 
 __device__ __forceinline__ void pair_build_body(
     const float4* __restrict__ pos, int N, float3 L, float3 invL, float3 invw, int3 nc,
     const int* __restrict__ count, const int* __restrict__ bodies, int cap, float Rc2, int max_nbr,
     int* __restrict__ half_count, int* __restrict__ nbr, int* __restrict__ lower_count,
     int* __restrict__ lower_pair, int* __restrict__ seg_sum, int* __restrict__ seg_base,
-    unsigned* status, const int* __restrict__ rebuild, int* done, int bid, int nblk) {
+    unsigned* status, const int* __restrict__ rebuild, int* done, bool rows, int bid, int nblk) {
     pdl_chain();
     if (!*rebuild) return;
     __shared__ float4 s_body[kBlkCap];            // position, body index in w
@@ -314,7 +354,13 @@ __device__ __forceinline__ void pair_build_body(
     const int3 nb = make_int3((nc.x + kBlkX - 1) / kBlkX, (nc.y + kBlkY - 1) / kBlkY,
                               (nc.z + kBlkZ - 1) / kBlkZ);
     const int n_blocks = nb.x * nb.y * nb.z;
-    for (int blk = bid; blk < n_blocks; blk += nblk) {
+    const bool by_warps = rows || crowded(N, done[2]);
+    if (by_warps) {
+        for (int i = bid * 8 + warp; i < N; i += nblk * 8)
+            pair_row_warp(i, pos, L, invL, invw, nc, count, bodies, cap, Rc2, max_nbr, half_count, nbr,
+                          lower_count, lower_pair, seg_sum, status);
+    }
+    for (int blk = by_warps ? n_blocks : bid; blk < n_blocks; blk += nblk) {
         const int3 b0 = make_int3(blk % nb.x * kBlkX, blk / nb.x % nb.y * kBlkY, blk / (nb.x * nb.y) * kBlkZ);
         const int3 w = make_int3(min(kBlkX, nc.x - b0.x), min(kBlkY, nc.y - b0.y), min(kBlkZ, nc.z - b0.z));
         // global cell of shared cell c, -1 outside this block's surroundings
@@ -455,8 +501,22 @@ __global__ void __launch_bounds__(256, kBuildCtas) k_pair_build(
     int* __restrict__ lower_pair, int* __restrict__ seg_sum, int* __restrict__ seg_base,
     unsigned* status, const int* __restrict__ rebuild, int* done) {
     pair_build_body(pos, N, L, invL, invw, nc, count, bodies, cap, Rc2, max_nbr, half_count, nbr,
-                    lower_count, lower_pair, seg_sum, seg_base, status, rebuild, done, blockIdx.x,
+                    lower_count, lower_pair, seg_sum, seg_base, status, rebuild, done, false, blockIdx.x,
                     gridDim.x);
+}
+
+__global__ void __launch_bounds__(256, kRowCtas) k_pair_rows(
+    const float4* __restrict__ pos, int N, float3 L, float3 invL, float3 invw, int3 nc,
+    const int* __restrict__ count, const int* __restrict__ bodies, int cap, float Rc2, int max_nbr,
+    int* __restrict__ half_count, int* __restrict__ nbr, int* __restrict__ lower_count,
+    int* __restrict__ lower_pair, int* __restrict__ seg_sum, int* __restrict__ seg_base,
+    unsigned* status, const int* __restrict__ rebuild, int* done) {
+    pdl_chain();
+    if (!*rebuild) return;
+    for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < N; i += gridDim.x * 8)
+        row_by_warp(i, pos, L, invL, invw, nc, count, bodies, cap, Rc2, max_nbr, half_count, nbr, lower_count,
+                    lower_pair, seg_sum, status);
+    if (pair_segments(N) > kScanSegments && last_cta_done(done, gridDim.x)) scan_segments(seg_sum, seg_base, N);
 }
 
 // Emit the compact pair list, a segment of kSegBodies bodies per CTA and pass:
@@ -544,7 +604,7 @@ __device__ __forceinline__ void pair_emit_body(
         __syncthreads();
     }
     for (int c = bid * 256 + tid; c < n_cells; c += nblk * 256) cell_count[c] = 0;
-    if (last_cta_done(done, nblk) && threadIdx.x == 0) *rebuild = 0;
+    if (last_cta_done(done, nblk) && threadIdx.x == 0) *rebuild = done[1] = 0;
 }
 
 __global__ void __launch_bounds__(256) k_pair_emit(
@@ -1016,8 +1076,8 @@ __global__ void k_cell_assign_batch(const StepSeg* __restrict__ segs, const int*
     const int k = seg_of_block(start, n_seg, blockIdx.x);
     const StepSeg& S = segs[k];
     cell_assign_body(S.pos, S.N, S.L, S.invL, S.invw, S.nc, S.cell_count, S.cell_bodies, S.cell_cap,
-                     S.status, S.rebuild, S.zero_count, S.seg, S.half_count, S.lower_count, 0,
-                     blockIdx.x - start[k]);
+                     S.status, S.rebuild, S.zero_count, S.seg, S.half_count, S.lower_count, S.done + 2,
+                     0, blockIdx.x - start[k]);
 }
 
 __global__ void __launch_bounds__(256, kBuildCtas) k_pair_build_batch(const StepSeg* __restrict__ segs, const int* __restrict__ start,
@@ -1026,7 +1086,8 @@ __global__ void __launch_bounds__(256, kBuildCtas) k_pair_build_batch(const Step
     const StepSeg& S = segs[k];
     pair_build_body(S.pos, S.N, S.L, S.invL, S.invw, S.nc, S.cell_count, S.cell_bodies, S.cell_cap,
                     S.Rl2, S.max_nbr, S.half_count, S.nbr, S.lower_count, S.lower_pair, S.seg,
-                    S.seg + pair_segments(S.N), S.status, S.rebuild, S.done, blockIdx.x - start[k], start[k + 1] - start[k]);
+                    S.seg + pair_segments(S.N), S.status, S.rebuild, S.done, S.rows != 0, blockIdx.x - start[k],
+                    start[k + 1] - start[k]);
 }
 
 __global__ void __launch_bounds__(256) k_pair_emit_batch(const StepSeg* __restrict__ segs, const int* __restrict__ start,
@@ -1049,6 +1110,12 @@ __global__ void k_reduce_batch(const StepSeg* __restrict__ segs, const int* __re
 }
 
 static inline int blocks_for(int64_t n, int t) { return (int)std::max<int64_t>(1, (n + t - 1) / t); }
+// CTAs of the row build: a warp per body, or a CTA per block of cells (and
+// enough warps where a crowded system takes the other form)
+static int build_ctas(int N, int3 nc, int num_sms, bool rows) {
+    return rows ? std::min(blocks_for(N, 8), num_sms * kRowCtas)
+                : std::min(std::max(cell_blocks(nc), blocks_for(N, 128)), num_sms * kBuildCtas);
+}
 
 static inline float3 f3(const float* a) { return make_float3(a[0], a[1], a[2]); }
 static inline float3 inv3(const float* a) { return make_float3(1.f / a[0], 1.f / a[1], 1.f / a[2]); }
@@ -1073,10 +1140,11 @@ rb_status build_pairs_async(rb_system* s, bool force, bool checked, int* zero_co
     RB_CUDA(launch_pdl(k_cell_assign, blocks_for(N, 256), 256, 0, s->stream, s->pos, N, L, invL,
                        invw, nc, s->cells.count, s->cells.bodies, s->cells.cap, s->status_dev,
                        s->rebuild_flag, zero_count, s->pl.seg, s->pl.half_count, s->pl.lower_count,
-                       force ? 1 : 0));
+                       s->pl.done + 2, force ? 1 : 0));
     s->fb_zeroed = zero_count != nullptr;
     int* seg_base = s->pl.seg + pair_segments(N);
-    RB_CUDA(launch_pdl(k_pair_build, std::min(cell_blocks(nc), s->num_sms * kBuildCtas), 256, 0, s->stream,
+    const bool rows = rows_by_warps(N, nc);
+    RB_CUDA(launch_pdl(rows ? k_pair_rows : k_pair_build, build_ctas(N, nc, s->num_sms, rows), 256, 0, s->stream,
                        s->pos, N, L, invL, invw, nc, s->cells.count, s->cells.bodies, s->cells.cap,
                        Rl * Rl, s->pl.max_nbr, s->pl.half_count, s->pl.nbr, s->pl.lower_count,
                        s->pl.lower_pair, s->pl.seg, seg_base, s->status_dev, s->rebuild_flag,
@@ -1245,6 +1313,7 @@ static StepSeg step_seg(const rb_system* s, float dt) {
     q.lower_pair = s->pl.lower_pair;
     q.half_off = s->pl.half_off;
     q.n_pairs = s->pl.n_pairs;
+    q.rows = dense_cells(s->N, q.nc);  // small replicas fill the GPU together: blocks of cells
     q.done = s->pl.done;
     q.cap_pairs = s->pl.cap_pairs;
     q.pairs = s->pl.pairs;
@@ -1330,7 +1399,8 @@ rb_status batch_create(const std::vector<BatchMember>& members, const BatchTable
             const int N = (int)s->N;
             need[0].push_back(blocks_for(N, 256));
             need[1].push_back(blocks_for(N, 256));
-            need[2].push_back(std::min(cell_blocks(seg[k].nc), num_sms * kBuildCtas));
+            need[2].push_back(seg[k].rows ? std::min(blocks_for(N, 16), num_sms * kBuildCtas)
+                                          : build_ctas(N, seg[k].nc, num_sms, false));
             need[3].push_back(std::min(blocks_for(std::max(N, s->cells.n_cells), 256), num_sms * 8));
             need[4].push_back(blocks_for((int64_t)N * 4, 256));
         }
@@ -1686,7 +1756,7 @@ rb_status rb_create_system(const rb_system_desc* d, void* stream, rb_system** ou
     ALLOC(s->pl.lower_pair, sizeof(int) * N * mn);
     ALLOC(s->pl.seg, sizeof(int) * 2 * pair_segments(s->N));
     ALLOC(s->pl.half_off, sizeof(int) * (N + 1));
-    ALLOC(s->pl.done, sizeof(int) * 2);
+    ALLOC(s->pl.done, sizeof(int) * 3);
     ALLOC(s->pl.pairs, sizeof(int2) * cp);
     ALLOC(s->pl.n_pairs, sizeof(int));
     ALLOC(s->pair_F, sizeof(float4) * cp);
@@ -1721,7 +1791,7 @@ rb_status rb_create_system(const rb_system_desc* d, void* stream, rb_system** ou
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->status_dev, 0, sizeof(unsigned), s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->pl.n_pairs, 0, sizeof(int), s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->pl.done, 0, sizeof(int) * 2, s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->pl.done, 0, sizeof(int) * 3, s->stream);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(s->pl.seg, 0, sizeof(int) * 2 * pair_segments(s->N), s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->rebuild_flag, 1, sizeof(int), s->stream);  // no list yet
