@@ -69,15 +69,17 @@ namespace rb {
 //     by at most d, so only these can decide the halvings that are left;
 //   * those test the listed pairs alone, two per lane, and stop when the middle
 //     no longer differs from an end of the bracket in FP32.
-// A list longer than kCand (parallel faces) is tried again after another
-// halving.  A grazing contact amplifies the last bit of a distance and the
-// label's repulsion that of the separation (by up to 3e-3 of the labels' rms in
-// one element), so every quantity that a halving or a label depends on is
-// rounded as the scan of all pairs rounds it, operation by operation (rotation,
-// place, bead_dist2, bead_terms): separations and labels are those of the full scan,
-// bit for bit.  The label takes the columns near body j only, and of those the
-// beads inside the cutoff; the others would add exact zeros.  Measured: 8885 ->
-// 366 us for 65536 cube pairs at contact 0.85; bound by instruction issue.
+// A list longer than kCand (parallel faces; contacts far beyond the bead spacing,
+// where many pairs are nearly equally far) is given up and tried again after two
+// more halvings.
+// A grazing contact amplifies the last bit of a distance and the label's
+// repulsion that of the separation (by up to 3e-3 of the labels' rms in one
+// element), so every quantity that a halving or a label depends on is rounded as
+// the scan of all pairs rounds it, operation by operation (rotation, place,
+// bead_dist2, bead_terms): separations and labels are those of the full scan, bit
+// for bit.  The label takes the columns near body j only, and of those the beads
+// inside the cutoff; the others would add exact zeros.  Measured: 8885 -> 366 us
+// for 65536 cube pairs at contact 0.85; bound by instruction issue.
 constexpr int kCoarse = 5;
 constexpr int kCand = 64;
 
@@ -239,17 +241,21 @@ __global__ void __launch_bounds__(256, NP <= 3 || C == 0 ? 2 : 1)
                     }
                 return false;
             } else {
-                float mn = 3.0e38f;
-                for (int k = 0; k < n_beads; ++k) {
-                    const float4 d = sT[k];
+                for (int k0 = 0; k0 < n_beads; k0 += 32) {
+                    float mn = 3.0e38f;
+                    for (int k = k0; k < min(k0 + 32, n_beads); ++k) {
+                        const float4 d = sT[k];
 #pragma unroll
-                    for (int m = 0; m < MB; ++m) mn = fminf(mn, bead_dist2(bx[m] - d.x, by[m] - d.y, bz[m] - d.z));
+                        for (int m = 0; m < MB; ++m)
+                            mn = fminf(mn, bead_dist2(bx[m] - d.x, by[m] - d.y, bz[m] - d.z));
+                    }
+                    if (__any_sync(0xffffffffu, mn < sig2)) return true;
                 }
-                return __any_sync(0xffffffffu, mn < sig2) != 0;
+                return false;
             }
         };
-        // bead pairs closer than `reach` with j's centre at rho: their number,
-        // the first kCand of them in cand
+        // bead pairs closer than `reach` with j's centre at rho: their number
+        // (some number above kCand if there are more), the first kCand of them in cand
         auto list_pairs = [&](float rho, float reach) {
             const float3 s = place(rho);
             const float r2 = reach * reach;
@@ -277,11 +283,17 @@ __global__ void __launch_bounds__(256, NP <= 3 || C == 0 ? 2 : 1)
                         const float mn = column_min<NP, C>(x, y, cols, bx, by, bz);
                         if (!__any_sync(0xffffffffu, mn < r2)) continue;
                         for (int k = 0; k < C; ++k) test(C * c + k, x, y, cols.z[k]);
+                        if (nc > kCand) return nc;
                     }
             } else {
                 for (int k = 0; k < n_beads; ++k) {
                     const float4 d = sT[k];
+                    float mn = 3.0e38f;
+#pragma unroll
+                    for (int m = 0; m < MB; ++m) mn = fminf(mn, bead_dist2(bx[m] - d.x, by[m] - d.y, bz[m] - d.z));
+                    if (!__any_sync(0xffffffffu, mn < r2)) continue;
                     test(k, d.x, d.y, d.z);
+                    if (nc > kCand) return nc;
                 }
             }
             __syncwarp();
@@ -294,8 +306,8 @@ __global__ void __launch_bounds__(256, NP <= 3 || C == 0 ? 2 : 1)
         d0 = d1 = make_float3(0.f, 0.f, 0.f);
         for (int it = 0; it < 40; ++it) {
             const float mid = 0.5f * (lo + hi);
-            if (lo > 0.f && hi < Rc && (mid <= lo || mid >= hi)) break;  // both ends tested: settled
-            if (nc > kCand && it >= kCoarse) {
+            if ((lo > 0.f && mid <= lo) || (hi < Rc && mid >= hi)) break;  // an end tested before: settled
+            if (nc > kCand && it >= kCoarse && ((it - kCoarse) & 1) == 0) {
                 nc = list_pairs(mid, contact + 0.5f * (hi - lo) + slack);
                 if (nc <= kCand) {
                     auto entry = [&](int e, float3& o, float3& d) {
