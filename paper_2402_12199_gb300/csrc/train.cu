@@ -412,15 +412,21 @@ __global__ void __launch_bounds__(256, NP <= 3 || C == 0 ? 2 : 1)
 constexpr int kTrSlotFloats = 4 * 256;  // x CPT: one quantity of one layer, all threads
 __host__ __device__ inline int tr_slots(int D) { return 2 * D + 1; }  // phi', phi'' term per layer, h_D
 
-template <int W, int CPT, int KC>
+// DG: h_dot_1 .. h_dot_{D-1} in the CTA's global scratch instead of shared memory
+// (width 256 at depth 4, whose arrays for four samples a thread would not fit).
+template <int W, int CPT, int KC, bool DG = false>
 struct TrShape {
     static constexpr int S = 1024 * CPT / W;  // samples per tile
     static constexpr int LD = S + 4;
     static constexpr int NTP = S / CPT;       // thread groups along samples
     static constexpr int NG = 256 / NTP;      // along units
     static_assert(NG * 4 == W && NTP <= 32, "4 units per thread; a unit's samples within a warp");
+    // floats of a CTA's scratch
+    __host__ __device__ static size_t scratch(int D) {
+        return (size_t)tr_slots(D) * kTrSlotFloats * CPT + (DG ? (size_t)(D - 1) * W * LD : 0);
+    }
     static size_t smem(int D) {
-        return sizeof(float) * ((size_t)(3 * D - 1) * W * LD + 2 * (size_t)KC * W + 2 * (size_t)kInPad * LD +
+        return sizeof(float) * ((size_t)(DG ? 2 * D : 3 * D - 1) * W * LD + 2 * (size_t)KC * W + 2 * (size_t)kInPad * LD +
                                 (size_t)NG * S + 32 + (size_t)D * W + W + S);
     }
 };
@@ -596,20 +602,22 @@ __device__ __forceinline__ void tr_weight_grad(const float* __restrict__ A1, con
         }
 }
 
-template <int W, int CPT, int KC>
+template <int W, int CPT, int KC, bool DG>
 __global__ void __launch_bounds__(256, 1)
     k_train_tile(const float* __restrict__ flat, const float* __restrict__ prep, FlatLayout fl, F32Layout pl,
                  int D, PairSrc src, TrArgs A, float* __restrict__ part, int64_t np,
                  float* __restrict__ scratch, double* __restrict__ loss_part) {
-    using Sh = TrShape<W, CPT, KC>;
+    using Sh = TrShape<W, CPT, KC, DG>;
     constexpr int S = Sh::S, LD = Sh::LD, NTP = Sh::NTP, NG = Sh::NG;
     constexpr int NS = 256 / S < W / 16 ? 256 / S : W / 16;  // unit slices of the dE/dx reduction
     static_assert(NS * kIn * S <= W * LD, "dE/dx partial sums fit in one array");
     pdl_wait();
     extern __shared__ float4 smem4[];
     float* Hs = reinterpret_cast<float*>(smem4);   // h_1 .. h_{D-1}
-    float* Ds = Hs + (size_t)(D - 1) * W * LD;     // h_dot_1 .. h_dot_{D-1}
-    float* Gs = Ds + (size_t)(D - 1) * W * LD;     // g_1 .. g_D, then a_z_{l-1} in the place of g_l
+    float* own = scratch + (size_t)blockIdx.x * Sh::scratch(D);
+    float* Ds = DG ? own + (size_t)tr_slots(D) * kTrSlotFloats * CPT  // h_dot_1 .. h_dot_{D-1}
+                   : Hs + (size_t)(D - 1) * W * LD;
+    float* Gs = Hs + (size_t)(DG ? 1 : 2) * (D - 1) * W * LD;  // g_1 .. g_D, then a_z_{l-1} in the place of g_l
     float* Zs = Gs + (size_t)D * W * LD;           // dE/dx partial sums, then a_z_D
     float* Bs = Zs + (size_t)W * LD;               // 2 x [KC][W] weight chunks
     float* Xs = Bs + (size_t)2 * KC * W;           // [16][LD] normalised features
@@ -622,7 +630,7 @@ __global__ void __launch_bounds__(256, 1)
     float* cs = wo + W;                            // S
     const int tid = threadIdx.x, tp = tid % NTP, to = tid / NTP;
     const int p0 = tp * CPT, o0 = to * 4;
-    float* mine = scratch + (size_t)blockIdx.x * tr_slots(D) * kTrSlotFloats * CPT + (size_t)tid * CPT;
+    float* mine = own + (size_t)tid * CPT;
     auto slot = [&](int k, int j) { return mine + ((size_t)k * 4 + j) * 256 * CPT; };  // unit j of the thread
     float* gp = part + (size_t)blockIdx.x * np;
 
@@ -939,27 +947,30 @@ static inline unsigned nblk(int64_t n, int t) { return (unsigned)std::max<int64_
 // Tiles of 4 samples per thread; 2 where a batch would leave half of the SMs
 // without a tile (a step of width 128: 59.6 against 73.9 us for 1000 samples,
 // 63.7 against 75.9 us for 2048; from 3000 on both forms fill the GPU), and at
-// depth 4, whose arrays would not fit.
+// depth 4 below width 256, whose arrays would not fit.  At width 256 the gradient
+// shares of a tile (0.8 MB at depth 4) are most of its traffic, so there h_dot
+// leaves shared memory instead: a gradient of 4096 samples 1020 -> 668 us, of 65536
+// 14.1 -> 8.9 ms (as separate GEMMs 858 us and 8.3 ms).
 static int tr_cols(const rb_trainer* t, int64_t B) {
     const int W = t->mlp->width;
-    return t->mlp->depth > 3 || B * W <= (int64_t)4096 * (t->sms / 2) ? 2 : 4;
+    return (t->mlp->depth > 3 && W < 256) || B * W <= (int64_t)4096 * (t->sms / 2) ? 2 : 4;
 }
 static int tr_grid(const rb_trainer* t, int64_t B, int cols) {
     const int64_t S = 1024 * cols / t->mlp->width;
     return (int)std::min<int64_t>((B + S - 1) / S, t->sms);
 }
 
-template <int W, int CPT, int KC>
+template <int W, int CPT, int KC, bool DG = false>
 static rb_status launch_tile(rb_trainer* t, int grid, const PairSrc& src, const TrArgs& A) {
     rb_mlp* m = t->mlp;
-    const size_t smem = TrShape<W, CPT, KC>::smem(m->depth);
+    const size_t smem = TrShape<W, CPT, KC, DG>::smem(m->depth);
     static std::atomic<size_t> allowed{0};
     if (smem > allowed.load()) {
-        RB_CUDA(cudaFuncSetAttribute(k_train_tile<W, CPT, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        RB_CUDA(cudaFuncSetAttribute(k_train_tile<W, CPT, KC, DG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      227 * 1024));
         allowed.store(227 * 1024);
     }
-    RB_CUDA(launch_pdl(k_train_tile<W, CPT, KC>, grid, 256, smem, m->stream, m->params, m->f32_prep,
+    RB_CUDA(launch_pdl(k_train_tile<W, CPT, KC, DG>, grid, 256, smem, m->stream, m->params, m->f32_prep,
                        flat_layout(W, m->depth), f32_layout(W, m->depth), m->depth, src, A, t->part,
                        m->n_params, t->scratch, t->loss_part));
     return RB_OK;
@@ -982,7 +993,12 @@ static rb_status train_pass(rb_trainer* t, TrArgs A, float* grad, bool step) {
         case 64 * 8 + 2: RB_TRY((launch_tile<64, 2, 64>(t, grid, src, A))); break;
         case 128 * 8 + 4: RB_TRY((launch_tile<128, 4, 64>(t, grid, src, A))); break;
         case 128 * 8 + 2: RB_TRY((launch_tile<128, 2, 32>(t, grid, src, A))); break;
-        case 256 * 8 + 4: RB_TRY((launch_tile<256, 4, 16>(t, grid, src, A))); break;
+        case 256 * 8 + 4:
+            if (m->depth > 3)
+                RB_TRY((launch_tile<256, 4, 16, true>(t, grid, src, A)));
+            else
+                RB_TRY((launch_tile<256, 4, 16>(t, grid, src, A)));
+            break;
         case 256 * 8 + 2: RB_TRY((launch_tile<256, 2, 16>(t, grid, src, A))); break;
         default: return fail(RB_ENOTSUP, "training supports widths 64, 128, 256");
     }
@@ -1123,7 +1139,10 @@ rb_status rb_trainer_create(rb_mlp* mlp, int64_t max_batch, float lr, float beta
     if (e == cudaSuccess) e = cudaMalloc(&t->pred, sizeof(float4) * 3 * max_batch);
     if (e == cudaSuccess) e = cudaMalloc(&t->part, sizeof(float) * np * ctas);
     if (e == cudaSuccess)
-        e = cudaMalloc(&t->scratch, sizeof(float) * tr_slots(mlp->depth) * kTrSlotFloats * 4 * ctas);
+        e = cudaMalloc(&t->scratch, sizeof(float) * ctas *
+                                        (mlp->width == 256 && mlp->depth > 3
+                                             ? TrShape<256, 4, 16, true>::scratch(mlp->depth)
+                                             : (size_t)tr_slots(mlp->depth) * kTrSlotFloats * 4));
     if (e == cudaSuccess) e = cudaMalloc(&t->loss_part, sizeof(double) * ctas);
     if (e == cudaSuccess) e = cudaMalloc(&t->loss_out, sizeof(double));
     if (e == cudaSuccess) e = cudaMemsetAsync(t->m, 0, sizeof(float) * np, mlp->stream);

@@ -54,21 +54,24 @@ def test_sampled_pairs_are_the_recorded_ones(g):
         assert np.abs(lab - want).max() <= 1e-5 * np.sqrt((want.astype(np.float64) ** 2).mean())
 
 
-def test_long_contacts_cost_no_more_than_full_scans():
-    """20000 pairs of a template without columns at contact 5: 1.4 ms; with the lists of near pairs made
-    in full at every halving 6.5 ms, all pairs in every halving 2.2 ms."""
+def test_long_contacts_are_not_listed_over_and_over():
+    """20000 pairs of a template without columns at contact 5 against contact 1: 3.4 times the time (1.4
+    and 0.43 ms); with the list of near pairs made in full at every halving 15 times."""
     import torch
 
     from paper_2402_12199_gb300 import api
 
     s = api.System(8, [80.0] * 3, "custom", template=_grid((5, 5, 4)))
     u = torch.from_numpy(np.random.default_rng(1).random((20000, 6)).astype(np.float32)).cuda()
-    api.sample_pairs(s, u, 5.0)
-    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    torch.cuda.synchronize()
-    a.record()
-    for _ in range(5):
-        api.sample_pairs(s, u, 5.0)
-    b.record()
-    torch.cuda.synchronize()
-    assert a.elapsed_time(b) / 5 < 3.5
+    best = {}
+    for contact in (1.0, 5.0):
+        t = []
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            api.sample_pairs(s, u, contact)
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b))
+        best[contact] = min(t)
+    assert best[5.0] < 8.0 * best[1.0]
