@@ -517,7 +517,8 @@ static rb_status launch_f16x3_impl(const rb_mlp* m, cudaStream_t stream, int gri
     static bool attr = false;
     if (!attr) {
         RB_CUDA(cudaFuncSetAttribute(f16x3::k_nn_f16x3<SYSTEM, P6>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)f16x3::smem_layout(3).total + 1024));  // any depth
         attr = true;
     }
     const unsigned char* img = static_cast<const unsigned char*>(m->f16x3_img);

@@ -407,7 +407,7 @@ static rb_status launch_tc(const rb_mlp* m, cudaStream_t stream, int grid, const
     static bool attr[2] = {false, false};
     if (!attr[SYSTEM ? 1 : 0]) {
         RB_CUDA(cudaFuncSetAttribute(tc::k_nn_tc<SYSTEM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
+                                     (int)tc::layout(3).total + 1024));  // any depth
         attr[SYSTEM ? 1 : 0] = true;
     }
     if (SYSTEM)  // inside an MD step: may start while the list kernels drain

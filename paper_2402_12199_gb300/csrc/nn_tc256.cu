@@ -418,7 +418,8 @@ static rb_status launch_tc256_impl(const rb_mlp* m, cudaStream_t stream, int gri
     static bool attr = false;
     if (!attr) {
         RB_CUDA(cudaFuncSetAttribute(tc256::k_nn_tc256<SYSTEM, BATCH>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)tc256::layout(3).s_total + 1024));  // any depth
         attr = true;
     }
     if (SYSTEM)  // inside an MD step: may start while the list kernels drain

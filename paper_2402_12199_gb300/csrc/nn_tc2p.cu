@@ -409,7 +409,8 @@ static rb_status launch_tc2p_impl(const rb_mlp* m, cudaStream_t stream, int grid
     static bool attr = false;
     if (!attr) {
         RB_CUDA(cudaFuncSetAttribute(tc2p::k_nn_tc2p<SYSTEM, P6, BATCH>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)tc2p::layout(3).total + 1024));  // any depth
         attr = true;
     }
     if (SYSTEM)  // inside an MD step: may start while the list kernels drain
