@@ -298,8 +298,9 @@ __device__ __noinline__ void pair_row_warp(int i, const float4* __restrict__ pos
 // chain of three L2 latencies per block; a warp per body had that chain (two
 // loads deep) once per occupied stencil slot, and sorted its rows in global
 // memory.  The whole build
-// (cell assignment, rows, offsets and emission, back to back): 1407 -> 246 us for
-// 524288 cubes, 111 -> 41 us for 32768 cylinders, 66 -> 36 us for 20011 cubes.
+// (cell assignment, rows, offsets and emission, back to back): 1407 -> 250 us for
+// 524288 cubes, 111 -> 42 us for 32768 cylinders (20011 cubes, rows by warps: 66 ->
+// 32 us).
 constexpr int kBlkX = 8, kBlkY = 4, kBlkZ = 4;
 constexpr int kHaloX = kBlkX + 2, kHaloY = kBlkY + 2, kHaloZ = kBlkZ + 2;
 constexpr int kHalo = kHaloX * kHaloY * kHaloZ;
