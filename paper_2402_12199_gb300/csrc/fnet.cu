@@ -1000,7 +1000,8 @@ rb_status rb_fnet_trainer_create(rb_fnet* f, int64_t max_batch, float lr, float 
 
 rb_status rb_fnet_trainer_destroy(rb_fnet_trainer* t) {
     if (!t) return RB_OK;
-    if (t->f && t->f->stream) cudaStreamSynchronize(t->f->stream);
+    // the network may be gone already (destroyed in any order at a process's end):
+    // cudaFree waits for the work in flight
     cudaFree(t->m);
     cudaFree(t->v);
     cudaFree(t->grad);

@@ -1163,7 +1163,8 @@ rb_status rb_trainer_set_lr(rb_trainer* t, float lr) {
 
 rb_status rb_trainer_destroy(rb_trainer* t) {
     if (!t) return RB_OK;
-    if (t->mlp && t->mlp->stream) cudaStreamSynchronize(t->mlp->stream);
+    // the network may be gone already (destroyed in any order at a process's end):
+    // cudaFree waits for the work in flight
     void* ptrs[] = {t->m, t->v, t->grad, t->pred, t->part, t->scratch, t->loss_part, t->loss_out};
     for (void* p : ptrs)
         if (p) cudaFree(p);
