@@ -349,10 +349,11 @@ static rb_status launch_f32(const rb_mlp* m, cudaStream_t stream, int grid, cons
 // 47.9 us, 20000 86.8 -> 76.8, 50003 171.7 -> 161.5; and up to a tile per SM,
 // for the latency of one (30.9 -> 26.7).  Just past each of these lines the
 // larger are faster: 5000 pairs 31.0 against 35.6, 15000 59.2 against 64.4,
-// 24320 87.4 against 93.0.  At depth 2 the ratios are 1.58 and 1.14; over 32
-// sizes from 32 to 200000 the rule takes the smaller tiles at neither depth
+// 24320 87.4 against 93.0.  Over 32 sizes from 32 to
+// 200000, at depth 2 as well as 3, the rule takes the smaller tiles at no size
 // where they are slower (depth 2: 20000 pairs 50.9 -> 43.9 us, 50003 99.6 ->
-// 90.0).
+// 90.0), and leaves out some where they are faster (31000 pairs, 67.3 against
+// 59.0 at depth 2 and 114.9 against 104.4 at depth 3).
 static bool small_tiles(int64_t n, int num_sms) {
     const int64_t t32 = (n + 31) / 32, t64 = (n + 63) / 64;
     if (t32 <= num_sms) return true;
